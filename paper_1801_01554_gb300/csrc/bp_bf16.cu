@@ -1,26 +1,31 @@
 // bfloat16 back-propagation step on the sm_103a tensor cores.
 //
-// Every contraction of the step is a GEMM C[M,N] = A[M,K] * B[N,K]^T with both
-// operands K-major in global memory, fed by TMA (128-byte swizzle) into a
-// multi-stage shared-memory ring, multiplied by tcgen05.mma (kind::f16, bf16
-// in, fp32 accumulate) into a double-buffered TMEM accumulator, and finished
-// by an epilogue that reads TMEM with tcgen05.ld:
+// Every contraction of the step is a GEMM C[M,N] = A[M,K] * B[N,K]^T fed by TMA
+// (128-byte swizzle) into a multi-stage shared-memory ring, multiplied by
+// tcgen05.mma (kind::f16, bf16 in, fp32 accumulate) into a double-buffered TMEM
+// accumulator, and finished by an epilogue that reads TMEM with tcgen05.ld:
 //
 //   forward  (Section 3)      A_l  = sigma(A_{l-1} W_l^T + b_l)
 //                               epilogue: bias, logistic, bf16 stores of A_l
-//                               row-major and transposed
 //   output   (Sections 3, 8)  o = sigma(...); delta_L = (t - o) o (1 - o);
 //                               error sum; bias-gradient column sums
 //   hidden delta (Section 3)  delta_{l-1} = (delta_l W_l) * a (1 - a), for
 //                               l = L..2 only: no delta for the input units
 //                               (Section 6.1)
 //   pooled change (Sec. 4.1)  G_l = delta_l^T A_{l-1}, K = the batch, split
-//                               over K into fp32 partial sums
+//                               over K into fp32 partial sums; the layers
+//                               share one launch
 //
-// The transposed copies (A_l^T, delta_l^T, X^T, W_l^T) keep every operand
-// K-major.  The update kernel sums the partial changes, applies the momentum
-// rule of Section 6.2.1 to the fp32 master weights and rewrites both bf16
-// weight copies.  All device-side waits are bounded and latch kFlagTimeout.
+// Activations, deltas and weights are stored once, row-major.  An operand whose
+// rows run along K is staged as it lies; one whose rows run along M or N (W_l in
+// the hidden delta, delta_l and A_{l-1} in the pooled change) is staged as 64 x
+// 64 blocks and handed to the tensor cores as an MN-major operand, so that no
+// transposed copy is ever written.  The update kernel sums the partial changes,
+// applies the momentum rule of Section 6.2.1 to the fp32 master weights and
+// rewrites the bf16 weight copy.  The kernels of a step are launched with
+// programmatic stream serialisation: each sets up its barriers and TMEM while
+// its predecessor drains, and waits (griddepcontrol.wait) before it touches
+// global memory.  All device-side waits are bounded and latch kFlagTimeout.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -31,6 +36,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "bp_bf16.h"
@@ -56,22 +62,34 @@ enum Mode : int { MODE_FWD = 0, MODE_FWD_OUT = 1, MODE_DX = 2, MODE_DW = 3 };
 struct GemmArgs {
     int M, N, K;
     int num_m, num_n;       // tiles along M and N
-    int splits;             // K splits (pooled change only)
-    int kb_per_split;       // K blocks per split
-    int kb_total;
+    int kb_total;           // K blocks
     const float* bias;      // [N]                          FWD, FWD_OUT
     bf16* out;              // [M, ldo] row-major            FWD: A_l; FWD_OUT: A_L; DX: delta
     int ldo;
-    bf16* out2;             // [M, ld2] row-major            FWD_OUT: delta_L
+    bf16* out2;             // [M, ld2] row-major            FWD_OUT: delta_L (with T), else a second copy of A_L
     int ld2;
-    bf16* out_t;            // [N, ldt] transposed           FWD: A_l^T; FWD_OUT/DX: delta^T
-    int ldt;
     const bf16* aux;        // FWD_OUT: T [M, ld_aux]; DX: A_{l-1} [M, ld_aux]
     int ld_aux;
-    float* gpart;           // DW: [splits, M, N]
     float* bias_part;       // [num_m, N]                    FWD_OUT (with T), DX
     float* sse_part;        // [num_m * num_n]               FWD_OUT (with T)
     int* flags;
+};
+
+// The pooled-change GEMMs of all layers, one launch: layer l's tiles are the
+// items [item0[l], item0[l + 1]), times `splits` runs of kb_per_split K blocks.
+struct DwLayer {
+    int M, N;               // n_l, n_{l-1}
+    int num_m, num_n;
+    int tile0;              // first tile of the layer
+    float* gpart;           // [splits, M, N]
+};
+struct DwArgs {
+    int L, tiles, splits, kb_per_split, kb_total;
+    DwLayer ly[kMaxL];
+    int* flags;
+};
+struct DwMaps {
+    CUtensorMap a[kMaxL], b[kMaxL];   // delta_l, A_{l-1}
 };
 
 // ------------------------------------------------------------ PTX helpers
@@ -132,23 +150,37 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
         : "memory");
 }
 
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
-// 128 bytes, 8-row groups 1024 bytes apart (tcgen05 descriptor version 1).
+// Programmatic dependent launch: wait for the kernels this one depends on (their
+// writes are then visible), and let the next kernel of the stream start its setup.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Shared-memory matrix descriptor, 128-byte swizzle (tcgen05 descriptor version 1).
+//   K-major:  the operand's rows are 128 bytes (64 of K); 8-row groups 1024 bytes
+//             apart (stride offset); the leading offset is unused.
+//   MN-major: blocks of 64 K rows x 64 of M or N (128 bytes); 8 K rows are 1024
+//             bytes apart (stride offset), the next 64 of M or N one block, 8 KB
+//             (leading offset).
+constexpr uint32_t kMnBlockBytes = BK * 64 * 2;
+template <bool MN>
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
     uint64_t d = 0;
     d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;      // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024u >> 4) << 32;    // stride byte offset: next 8-row group
+    d |= (uint64_t)((MN ? kMnBlockBytes : 16u) >> 4) << 16;   // leading byte offset
+    d |= (uint64_t)(1024u >> 4) << 32;    // stride byte offset
     d |= (uint64_t)1 << 46;               // descriptor version
     d |= (uint64_t)2 << 61;               // 128-byte swizzle
     return d;
 }
+// Bytes from one K step of UMMA_K to the next inside a stage.
+template <bool MN>
+__device__ __forceinline__ constexpr uint32_t k_step_bytes() { return MN ? UMMA_K * 128 : UMMA_K * 2; }
 
-// Instruction descriptor of tcgen05.mma kind::f16: bf16 A and B, fp32 D,
-// both operands K-major, M x N tile.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-           ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor of tcgen05.mma kind::f16: bf16 A and B, fp32 D, M x N
+// tile, each operand K-major or MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool b_mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
@@ -200,20 +232,6 @@ __device__ __forceinline__ float bf16_round(float x) {
     return __bfloat162float(__float2bfloat16_rn(x));
 }
 
-// Afterwards lane k holds in v[0] the warp sum of value k (31 shuffles).
-__device__ __forceinline__ void reduce_scatter32(float (&v)[32], int lane) {
-#pragma unroll
-    for (int half = 16; half >= 1; half >>= 1) {
-        const bool up = (lane & half) != 0;
-#pragma unroll
-        for (int k = 0; k < half; ++k) {
-            const float send = up ? v[k] : v[k + half];
-            const float keep = up ? v[k + half] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-        }
-    }
-}
-
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // ------------------------------------------------------------ epilogue
@@ -222,7 +240,7 @@ __device__ __forceinline__ void load_row32(float (&a)[32], const bf16* p, bool w
     if (whole) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(p) + k);
+            const uint4 u = reinterpret_cast<const uint4*>(p)[k];
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -237,33 +255,28 @@ __device__ __forceinline__ void load_row32(float (&a)[32], const bf16* p, bool w
     }
 }
 
+// One 32-column chunk of a pooled-change tile: this lane's row m of the partial sums.
+__device__ __forceinline__ void store_partial(float* gpart, int M, int N, int m, int n0, int split, const float (&v)[32]) {
+    if (m >= M) return;
+    float* dst = gpart + ((size_t)split * M + m) * N + n0;   // N is a multiple of 8
+#pragma unroll
+    for (int c = 0; c < 32; c += 4)
+        if (n0 + c < N) *reinterpret_cast<float4*>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+}
+
 // One 32-column chunk of the tile for the 32 rows of one epilogue warp (this
-// lane's row m).  Values are rounded to bf16 and staged in the warp's 2 KB
-// shared-memory block, first by rows (16-byte pieces permuted by row so that
-// the lanes' writes hit distinct banks), then transposed.  After each staging
-// the warp writes every 64-byte row (or column) segment with four lanes'
-// 16-byte stores, eight segments per instruction.  The column sums of a delta
-// block (bias change) are read back from the transposed block.
+// lane's row m).  Values are rounded to bf16 and staged by rows in the warp's
+// 2 KB shared-memory block (16-byte pieces permuted by row so that the lanes'
+// writes hit distinct banks); the warp then writes every 64-byte row segment
+// with four lanes' 16-byte stores, eight segments per instruction.  The column
+// sums of a delta block (bias change) are taken from the pieces on their way
+// out: each lane adds its four rows of 8 columns, then the eight lanes of a
+// piece reduce-scatter them (7 shuffles).
 template <int MODE>
-__device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0, int n0, int split,
-                                               float (&v)[32], float& sse, bool row_ok, bf16* sS,
-                                               const float* sbias, float* colsum_slot) {
+__device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0, int n0, float (&v)[32], float& sse,
+                                               bool row_ok, bf16* sS, const float* sbias, float* colsum_slot) {
     const int N = g.N;
     const int lane = threadIdx.x & 31;
-    if (MODE == MODE_DW) {
-        if (row_ok) {
-            float* dst = g.gpart + ((size_t)split * g.M + m) * N + n0;
-            if (n0 + 32 <= N && (N & 3) == 0) {
-#pragma unroll
-                for (int c = 0; c < 32; c += 4)
-                    *reinterpret_cast<float4*>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
-            } else {
-                for (int c = 0; c < 32; ++c)
-                    if (n0 + c < N) dst[c] = v[c];
-            }
-        }
-        return;
-    }
     const bool whole = (n0 + 32 <= N);
     const int valid = min(32, N - n0);
     const bool with_t = (MODE == MODE_FWD_OUT) && (g.aux != nullptr);
@@ -301,72 +314,56 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0,
             vals[c] = ok ? bf16_round(v[c] * a[c] * (1.f - a[c])) : 0.f;
         }
     }
-    // rows: A_l, A_L or delta_L (training output layer), or delta_{l-1}
+    // rows: A_l, A_L (and the caller's copy) or delta_L (training output layer), or delta_{l-1}
     bf16* const rows = with_t ? g.out2 : g.out;
     const int ldr = with_t ? g.ld2 : g.ldo;
-    const bool has_r = rows != nullptr;
-    const bool has_t = (MODE == MODE_FWD && g.out_t != nullptr) || with_t || (MODE == MODE_DX);
+    bf16* const copy = (MODE == MODE_FWD_OUT && !with_t) ? g.out2 : nullptr;
     uint4* sS4 = reinterpret_cast<uint4*>(sS);
     const int piece = lane & 3;   // 16-byte piece of a 64-byte segment
-    if (has_r) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            __align__(16) __nv_bfloat162 h[4];
+    for (int k = 0; k < 4; ++k) {
+        __align__(16) __nv_bfloat162 h[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(vals[8 * k + 2 * q], vals[8 * k + 2 * q + 1]);
-            sS4[lane * 4 + (k ^ ((lane >> 1) & 3))] = *reinterpret_cast<const uint4*>(h);
-        }
-        __syncwarp();
-        const int pieces = valid >> 3;   // N is a multiple of 8
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = j * 8 + (lane >> 2);
-            if (m0 + r < g.M && piece < pieces)
-                *reinterpret_cast<uint4*>(rows + (size_t)(m0 + r) * ldr + n0 + piece * 8) =
-                    sS4[r * 4 + (piece ^ ((r >> 1) & 3))];
-        }
-        __syncwarp();   // the block is rewritten below
+        for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(vals[8 * k + 2 * q], vals[8 * k + 2 * q + 1]);
+        sS4[lane * 4 + (k ^ ((lane >> 1) & 3))] = *reinterpret_cast<const uint4*>(h);
     }
-    if (has_t) {
+    __syncwarp();
+    const int pieces = valid >> 3;   // N is a multiple of 8
+    float cs[8];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) sS[c * 32 + lane] = __float2bfloat16_rn(vals[c]);
-        __syncwarp();
+    for (int q = 0; q < 8; ++q) cs[q] = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = j * 8 + (lane >> 2);
-            const int left = g.M - (m0 + piece * 8);   // rows of this piece inside the batch
-            if (c < valid && left > 0) {
-                const uint4 u = sS4[c * 4 + piece];
-                bf16* dst = g.out_t + (size_t)(n0 + c) * g.ldt + m0 + piece * 8;
-                if (left >= 8) {
-                    *reinterpret_cast<uint4*>(dst) = u;
-                } else {
-                    const bf16* e = reinterpret_cast<const bf16*>(&u);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < left) dst[i] = e[i];
-                }
-            }
+    for (int j = 0; j < 4; ++j) {
+        const int r = j * 8 + (lane >> 2);
+        const uint4 u = sS4[r * 4 + (piece ^ ((r >> 1) & 3))];
+        if (m0 + r < g.M && piece < pieces) {
+            *reinterpret_cast<uint4*>(rows + (size_t)(m0 + r) * ldr + n0 + piece * 8) = u;
+            if (copy != nullptr) *reinterpret_cast<uint4*>(copy + (size_t)(m0 + r) * g.ld2 + n0 + piece * 8) = u;
         }
-    }
-    if (colsum_slot != nullptr) {
-        // lane c sums column c of the block over the warp's 32 rows
-        const uint4* col = reinterpret_cast<const uint4*>(sS + lane * 32);
-        float sum = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint4 u = col[k];
+        if (colsum_slot != nullptr) {   // rows past the batch and columns past N hold zeros
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float2 f = __bfloat1622float2(h[q]);
-                sum += f.x;
-                sum += f.y;
+                cs[2 * q] += f.x;
+                cs[2 * q + 1] += f.y;
             }
         }
-        colsum_slot[lane] = sum;
     }
-    __syncwarp();   // the staging blocks may be rewritten
+    if (colsum_slot != nullptr) {
+#pragma unroll
+        for (int half = 4; half >= 1; half >>= 1) {
+            const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+            for (int k = 0; k < half; ++k) {
+                const float send = up ? cs[k] : cs[k + half];
+                const float keep = up ? cs[k + half] : cs[k];
+                cs[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * half);
+            }
+        }
+        colsum_slot[piece * 8 + (lane >> 2)] = cs[0];
+    }
+    __syncwarp();   // the staging block may be rewritten
 }
 
 // ------------------------------------------------------------ GEMM kernel
@@ -386,9 +383,9 @@ __device__ __forceinline__ void tile_coords(int tile, int num_m, int num_n, int&
     nb = local / gm;
 }
 
-template <int BN, int MODE>
+template <int BN>
 struct GemmCfg {
-    static constexpr int kStages = BN == 256 ? 4 : 6;
+    static constexpr int kStages = BN == 256 ? 4 : BN == 128 ? 6 : 8;
     static constexpr int kABytes = BM * BK * 2;
     static constexpr int kBBytes = BN * BK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
@@ -402,12 +399,67 @@ struct GemmCfg {
         1024 + kRingBytes + kColsumBytes + kStageOutBytes + kBiasBytes + 256;
 };
 
-template <int BN, int MODE>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-    k_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-           GemmArgs g) {
-    using Cfg = GemmCfg<BN, MODE>;
+// A work item of a GEMM launch: a tile and its run of K blocks.
+struct Item {
+    int mb, nb, kb0, kb1;
+    int l, split;            // pooled change only
+};
+// Work of the forward and hidden-delta launches: one problem, whole K.
+template <int MODE>
+struct OneGemm {
+    static constexpr int kMode = MODE;
+    static constexpr bool kAMn = false, kBMn = MODE == MODE_DX;
+    const GemmArgs& g;
+    const CUtensorMap *ma, *mb_;
+    __device__ int items() const { return g.num_m * g.num_n; }
+    __device__ Item item(int it) const {
+        Item w{0, 0, 0, g.kb_total, 0, 0};
+        tile_coords(it, g.num_m, g.num_n, w.mb, w.nb);
+        return w;
+    }
+    __device__ const CUtensorMap* map_a(const Item&) const { return ma; }
+    __device__ const CUtensorMap* map_b(const Item&) const { return mb_; }
+};
+// Work of the pooled-change launch: every layer's tiles, `splits` times over.
+struct DwGemm {
+    static constexpr int kMode = MODE_DW;
+    static constexpr bool kAMn = true, kBMn = true;
+    const DwArgs& g;
+    const DwMaps& maps;
+    __device__ int items() const { return g.tiles * g.splits; }
+    __device__ Item item(int it) const {
+        Item w;
+        w.split = it / g.tiles;
+        const int tile = it - w.split * g.tiles;
+        w.l = 0;
+        while (w.l + 1 < g.L && tile >= g.ly[w.l + 1].tile0) ++w.l;
+        const DwLayer& y = g.ly[w.l];
+        tile_coords(tile - y.tile0, y.num_m, y.num_n, w.mb, w.nb);
+        w.kb0 = w.split * g.kb_per_split;
+        w.kb1 = min(g.kb_total, w.kb0 + g.kb_per_split);
+        return w;
+    }
+    __device__ const CUtensorMap* map_a(const Item& w) const { return &maps.a[w.l]; }
+    __device__ const CUtensorMap* map_b(const Item& w) const { return &maps.b[w.l]; }
+};
+
+// Copies one operand's stage: ROWS of M or N by BK of K from K block kb.
+template <int ROWS, bool MN>
+__device__ __forceinline__ void load_operand(uint8_t* dst, const CUtensorMap* map, int row0, int kb, uint64_t* bar) {
+    if (MN) {
+#pragma unroll
+        for (int i = 0; i < ROWS / 64; ++i) tma_load_2d(dst + i * kMnBlockBytes, map, row0 + 64 * i, kb * BK, bar);
+    } else {
+        tma_load_2d(dst, map, kb * BK, row0, bar);
+    }
+}
+
+template <int BN, class Work>
+__device__ __forceinline__ void gemm_body(const Work work) {
+    using Cfg = GemmCfg<BN>;
+    constexpr int MODE = Work::kMode;
     constexpr int S = Cfg::kStages;
+    const auto& g = work.g;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* ring = smem;
@@ -426,9 +478,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = g.num_m * g.num_n;
-    const int items = tiles * g.splits;
+    const int items = work.items();
 
+    pdl_launch();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -453,6 +505,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();   // every thread, before its first access to what earlier kernels wrote or still read
 
     if (warp == 0) {
         // ---------------- TMA producer
@@ -463,18 +516,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int s = 0; s < S; ++s) issued_parity[s] = -1;
             bool ok = true;
             for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-                const int tile = it % tiles, split = it / tiles;
-                int mb, nb;
-                tile_coords(tile, g.num_m, g.num_n, mb, nb);
-                const int kb0 = split * g.kb_per_split;
-                const int kb1 = min(g.kb_total, kb0 + g.kb_per_split);
-                for (int kb = kb0; kb < kb1; ++kb) {
+                const Item w = work.item(it);
+                const CUtensorMap *ma = work.map_a(w), *mb = work.map_b(w);
+                for (int kb = w.kb0; kb < w.kb1; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
                     uint8_t* sa = ring + stage * Cfg::kStageBytes;
-                    uint8_t* sb = sa + Cfg::kABytes;
                     mbar_expect_tx(&full[stage], Cfg::kStageBytes);
-                    tma_load_2d(sa, &map_a, kb * BK, mb * BM, &full[stage]);
-                    tma_load_2d(sb, &map_b, kb * BK, nb * BN, &full[stage]);
+                    load_operand<BM, Work::kAMn>(sa, ma, w.mb * BM, kb, &full[stage]);
+                    load_operand<BN, Work::kBMn>(sa + Cfg::kABytes, mb, w.nb * BN, kb, &full[stage]);
                     issued_parity[stage] = (int)phase;
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
@@ -493,7 +542,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(BM, BN);
+            constexpr uint32_t idesc = idesc_bf16(BM, BN, Work::kAMn, Work::kBMn);
             int stage = 0;
             unsigned phase = 0;
             int acc = 0;
@@ -501,22 +550,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             bool ok = true;
             bool issued_any = false;
             for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-                const int split = it / tiles;
-                const int kb0 = split * g.kb_per_split;
-                const int kb1 = min(g.kb_total, kb0 + g.kb_per_split);
+                const Item w = work.item(it);
                 if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
-                for (int kb = kb0; kb < kb1; ++kb) {
+                for (int kb = w.kb0; kb < w.kb1; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.flags)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a0 = smem_u32(ring + stage * Cfg::kStageBytes);
                     const uint32_t b0 = a0 + Cfg::kABytes;
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                        const uint64_t ad = smem_desc_sw128(a0 + kk * UMMA_K * 2);
-                        const uint64_t bd = smem_desc_sw128(b0 + kk * UMMA_K * 2);
-                        umma_bf16(tmem_d, ad, bd, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
+                        const uint64_t ad = smem_desc_sw128<Work::kAMn>(a0 + kk * k_step_bytes<Work::kAMn>());
+                        const uint64_t bd = smem_desc_sw128<Work::kBMn>(b0 + kk * k_step_bytes<Work::kBMn>());
+                        umma_bf16(tmem_d, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
                     }
                     issued_any = true;
                     umma_commit(&empty[stage]);
@@ -543,65 +590,75 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         int acc = 0;
         unsigned acc_phase = 0;
         for (int it = blockIdx.x; it < items; it += gridDim.x) {
-            const int tile = it % tiles, split = it / tiles;
-            int mb, nb;
-            tile_coords(tile, g.num_m, g.num_n, mb, nb);
+            const Item w = work.item(it);
             float* sbias = bias_s + acc * BN;
-            if (MODE == MODE_FWD || MODE == MODE_FWD_OUT) {
+            if constexpr (MODE == MODE_FWD || MODE == MODE_FWD_OUT) {
                 // block acc was last read two tiles ago, before the barrier of the previous tile
                 for (int c = threadIdx.x - 64; c < BN; c += kEpiThreads) {
-                    const int n = nb * BN + c;
-                    sbias[c] = n < g.N ? __ldg(g.bias + n) : 0.f;
+                    const int n = w.nb * BN + c;
+                    sbias[c] = n < g.N ? g.bias[n] : 0.f;
                 }
             }
             mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
             epi_bar();                     // the epilogue warps leave together on an abort
             if (*abort_flag) break;
             tc_fence_after();
-            const int m = mb * BM + q * 32 + lane;
-            const bool row_ok = m < g.M;
-            float sse = 0.f;
+            const int m = w.mb * BM + q * 32 + lane;
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
-            const int m0 = mb * BM + q * 32;
-            bf16* sS = stage_out + ew * 1024;
-            const bool want_colsum = (MODE == MODE_DX) || (MODE == MODE_FWD_OUT && g.aux != nullptr);
-            for (int c0 = cbeg; c0 < cbeg + BN / 2; c0 += 32) {
-                const int n0 = nb * BN + c0;
-                float v[32];
-                tmem_ld32(tbase + (uint32_t)c0, v);
-                if (n0 >= g.N) {
-                    if (want_colsum) colsum[slot * BN + c0 + lane] = 0.f;
-                    continue;
+            if constexpr (MODE == MODE_DW) {
+                const DwLayer& y = g.ly[w.l];
+                for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(tbase + (uint32_t)c0, v);
+                    store_partial(y.gpart, y.M, y.N, m, w.nb * BN + c0, w.split, v);
                 }
-                epilogue_chunk<MODE>(g, m, m0, n0, split, v, sse, row_ok, sS, sbias + c0,
-                                     want_colsum ? colsum + slot * BN + c0 : nullptr);
-            }
-            // TMEM is free for the next accumulation into this buffer
-            tc_fence_before();
-            mbar_arrive(&tempty[acc]);
-            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-            if (MODE == MODE_DX || (MODE == MODE_FWD_OUT && g.aux != nullptr)) {
-                epi_bar();
-                const int t = threadIdx.x - 64;   // 0 .. kEpiThreads - 1
-                for (int c = t; c < BN; c += kEpiThreads) {
-                    const int n = nb * BN + c;
-                    if (n < g.N) {
-                        const float s = (colsum[c] + colsum[BN + c]) + (colsum[2 * BN + c] + colsum[3 * BN + c]);
-                        g.bias_part[(size_t)mb * g.N + n] = s;
+                tc_fence_before();
+                mbar_arrive(&tempty[acc]);
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            } else {
+                const bool row_ok = m < g.M;
+                float sse = 0.f;
+                const int m0 = w.mb * BM + q * 32;
+                bf16* sS = stage_out + ew * 1024;
+                const bool want_colsum = (MODE == MODE_DX) || (MODE == MODE_FWD_OUT && g.aux != nullptr);
+                for (int c0 = cbeg; c0 < cbeg + BN / 2; c0 += 32) {
+                    const int n0 = w.nb * BN + c0;
+                    float v[32];
+                    tmem_ld32(tbase + (uint32_t)c0, v);
+                    if (n0 >= g.N) {
+                        if (want_colsum) colsum[slot * BN + c0 + lane] = 0.f;
+                        continue;
                     }
+                    epilogue_chunk<MODE>(g, m, m0, n0, v, sse, row_ok, sS, sbias + c0,
+                                         want_colsum ? colsum + slot * BN + c0 : nullptr);
                 }
-                if (MODE == MODE_FWD_OUT) {
-                    // tile error sum: warp sums, then the eight warps in a fixed order
+                // TMEM is free for the next accumulation into this buffer
+                tc_fence_before();
+                mbar_arrive(&tempty[acc]);
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                if (want_colsum) {
+                    epi_bar();
+                    const int t = threadIdx.x - 64;   // 0 .. kEpiThreads - 1
+                    for (int c = t; c < BN; c += kEpiThreads) {
+                        const int n = w.nb * BN + c;
+                        if (n < g.N) {
+                            const float s = (colsum[c] + colsum[BN + c]) + (colsum[2 * BN + c] + colsum[3 * BN + c]);
+                            g.bias_part[(size_t)w.mb * g.N + n] = s;
+                        }
+                    }
+                    if (MODE == MODE_FWD_OUT) {
+                        // tile error sum: warp sums, then the eight warps in a fixed order
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) sse += __shfl_xor_sync(0xffffffffu, sse, o);
+                        for (int o = 16; o > 0; o >>= 1) sse += __shfl_xor_sync(0xffffffffu, sse, o);
+                        epi_bar();
+                        if (lane == 0) colsum[ew] = sse;
+                        epi_bar();
+                        if (t == 0)
+                            g.sse_part[it] = ((colsum[0] + colsum[1]) + (colsum[2] + colsum[3])) +
+                                             ((colsum[4] + colsum[5]) + (colsum[6] + colsum[7]));
+                    }
                     epi_bar();
-                    if (lane == 0) colsum[ew] = sse;
-                    epi_bar();
-                    if (t == 0)
-                        g.sse_part[tile] = ((colsum[0] + colsum[1]) + (colsum[2] + colsum[3])) +
-                                           ((colsum[4] + colsum[5]) + (colsum[6] + colsum[7]));
                 }
-                epi_bar();
             }
         }
     }
@@ -615,110 +672,113 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
 }
 
-// ------------------------------------------------------------ SIMT kernels
-// dst[c][r] = src[r][c] for a [rows, cols] bf16 matrix whose column count and
-// both pitches are multiples of 8 (64 x 64 tiles, 256 threads).  Rows of src
-// and of dst move in 16-byte pieces; the shared-memory pitch of 33 words keeps
-// the lanes' 4-byte writes conflict-free.
-__global__ void __launch_bounds__(256) k_transpose(const bf16* __restrict__ src, int rows, int cols,
-                                                   int lds, bf16* __restrict__ dst, int ldd) {
-    __shared__ __align__(16) uint32_t tile[64][33];   // [r][pair of columns]
-    const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
-    const int t = threadIdx.x, p = t & 7;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int r = (t >> 3) + 32 * h, c = c0 + p * 8;
-        uint4 u = make_uint4(0u, 0u, 0u, 0u);
-        if (r0 + r < rows && c < cols) u = *reinterpret_cast<const uint4*>(src + (size_t)(r0 + r) * lds + c);
-        tile[r][p * 4] = u.x;
-        tile[r][p * 4 + 1] = u.y;
-        tile[r][p * 4 + 2] = u.z;
-        tile[r][p * 4 + 3] = u.w;
-    }
-    __syncthreads();
-    const bf16* tb = reinterpret_cast<const bf16*>(&tile[0][0]);   // element (r, c) at r * 66 + c
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int c = (t >> 3) + 32 * h, r = p * 8;   // dst row c0 + c, columns r0 + r .. +7
-        if (c0 + c >= cols || r0 + r >= rows) continue;
-        __align__(16) bf16 e[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) e[k] = tb[(r + k) * 66 + c];
-        bf16* d = dst + (size_t)(c0 + c) * ldd + r0 + r;
-        if (r0 + r + 8 <= rows) {
-            *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(e);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (r0 + r + k < rows) d[k] = e[k];
-        }
-    }
+template <int BN, int MODE>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    k_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+           const __grid_constant__ GemmArgs g) {
+    gemm_body<BN>(OneGemm<MODE>{g, &map_a, &map_b});
 }
 
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    k_gemm_dw(const __grid_constant__ DwMaps maps, const __grid_constant__ DwArgs g) {
+    gemm_body<BN>(DwGemm{g, maps});
+}
+
+// ------------------------------------------------------------ SIMT kernels
 // Output deltas from stored outputs (bp_backward): delta = (t - o) o (1 - o),
-// delta rows and transposed copy, per-128-row column sums and error sums.
-// One block of 128 threads per (128-row tile, 32-column chunk).
-__global__ void k_output_delta(const bf16* __restrict__ O, const bf16* __restrict__ T, int M, int N,
-                               int ld, bf16* __restrict__ Drow, bf16* __restrict__ Dt, int ldt,
-                               float* __restrict__ bias_part, float* __restrict__ sse_part,
-                               int num_n_chunks) {
-    __shared__ float cs[4][32];
-    __shared__ float ss[4];
+// delta rows, per-128-row column sums and error sums.  One block of 256 threads
+// per 128 rows x 64 columns; a thread moves 8 columns of 4 rows in 16-byte pieces.
+__global__ void __launch_bounds__(256) k_output_delta(const bf16* O, const bf16* T, int M, int N, bf16* D,
+                                                      float* bias_part, float* sse_part) {
+    __shared__ float cs[8][64];
+    __shared__ float ss[8];
     const int mb = blockIdx.y, nc = blockIdx.x;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m = mb * 128 + threadIdx.x;
-    const bool row_ok = m < M;
-    float d[32];
+    const int piece = threadIdx.x & 7;
+    const int n = nc * 64 + piece * 8;   // N is a multiple of 8: a piece is whole or outside
+    pdl_launch();
+    pdl_wait();
+    float sums[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sums[q] = 0.f;
     float sse = 0.f;
-    for (int c = 0; c < 32; ++c) {
-        const int n = nc * 32 + c;
-        const bool ok = row_ok && n < N;
-        float dv = 0.f;
-        if (ok) {
-            const float o = __bfloat162float(O[(size_t)m * ld + n]);
-            const float err = __bfloat162float(T[(size_t)m * ld + n]) - o;
-            sse = fmaf(err, err, sse);
-            dv = bf16_round(err * o * (1.f - o));
-            Drow[(size_t)m * ld + n] = __float2bfloat16_rn(dv);
-            Dt[(size_t)n * ldt + m] = __float2bfloat16_rn(dv);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int m = mb * 128 + j * 32 + (threadIdx.x >> 3);
+        if (m >= M || n >= N) continue;
+        const size_t e = (size_t)m * N + n;
+        const uint4 uo = *reinterpret_cast<const uint4*>(O + e);
+        const uint4 ut = *reinterpret_cast<const uint4*>(T + e);
+        const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&uo);
+        const __nv_bfloat162* ht = reinterpret_cast<const __nv_bfloat162*>(&ut);
+        __align__(16) __nv_bfloat162 hd[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 o = __bfloat1622float2(ho[q]), t = __bfloat1622float2(ht[q]);
+            const float e0 = t.x - o.x, e1 = t.y - o.y;
+            sse = fmaf(e0, e0, sse);
+            sse = fmaf(e1, e1, sse);
+            hd[q] = __floats2bfloat162_rn(e0 * o.x * (1.f - o.x), e1 * o.y * (1.f - o.y));
+            const float2 d = __bfloat1622float2(hd[q]);
+            sums[2 * q] += d.x;
+            sums[2 * q + 1] += d.y;
         }
-        d[c] = dv;
+        *reinterpret_cast<uint4*>(D + e) = *reinterpret_cast<const uint4*>(hd);
     }
-    reduce_scatter32(d, lane);
-    cs[w][lane] = d[0];
+    // the four rows of a warp's lanes per piece (lane bits 3, 4), then the eight warps
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        sums[q] += __shfl_xor_sync(0xffffffffu, sums[q], 8);
+        sums[q] += __shfl_xor_sync(0xffffffffu, sums[q], 16);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sse += __shfl_xor_sync(0xffffffffu, sse, o);
+    if (lane < 8) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) cs[w][lane * 8 + q] = sums[q];
+    }
     if (lane == 0) ss[w] = sse;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const int n = nc * 32 + threadIdx.x;
-        if (n < N) bias_part[(size_t)mb * N + n] = (cs[0][threadIdx.x] + cs[1][threadIdx.x]) +
-                                                   (cs[2][threadIdx.x] + cs[3][threadIdx.x]);
+    if (threadIdx.x < 64) {
+        const int c = nc * 64 + threadIdx.x;
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += cs[k][threadIdx.x];
+        if (c < N) bias_part[(size_t)mb * N + c] = s;
     }
-    if (threadIdx.x == 0) sse_part[(size_t)mb * num_n_chunks + nc] = (ss[0] + ss[1]) + (ss[2] + ss[3]);
+    if (threadIdx.x == 64) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += ss[k];
+        sse_part[(size_t)mb * gridDim.x + nc] = s;
+    }
 }
 
-constexpr int kUT = 64;   // update kernel: weight tile edge
+constexpr int kUpdThreads = 256;
+constexpr int kUpdPieces = 2;                                    // float4 pieces per thread of a weight block
+constexpr int kUpdFloats = kUpdThreads * kUpdPieces * 4;         // weights per block
+constexpr int kUpdBiases = 32, kUpdSlices = kUpdThreads / kUpdBiases;   // biases per block, threads per bias
 
 struct LayerUpd {
-    int n_out, n_in;
+    long long nw;               // n_out * n_in, a multiple of 64
+    int n_out;
     long long woff, boff;       // offsets in theta / V / G
-    const float* gpart;         // [splits, n_out, n_in] (null: none)
-    int splits;
+    const float* gpart;         // [splits, n_out, n_in]
     const float* bias_part;     // [mtiles, n_out]
-    int mtiles;
     bf16* wb;                   // [n_out, n_in]
-    bf16* wt;                   // [n_in, n_out]
+    int block0, bias0;          // first weight block and first bias block of the layer
 };
 struct UpdArgs {
     int L;
     LayerUpd ly[kMaxL];
-    int tile0[kMaxL + 1];       // kUT x kUT weight tiles (+ one bias row band) per layer
+    int blocks;                 // weight and bias blocks of all layers
+    int splits, mtiles;         // pending partial changes (0: none)
     float* theta;
     float* V;
     float* G;
     float lr_gs, momentum;
-    int mode;                   // 0: apply update; 1: accumulate into G; 2: refresh bf16 copies
+    int mode;                   // 0: apply update; 1: accumulate into G; 2: refresh the bf16 copy
     int fold_g;
     const float* sse_part;
     int n_sse;
@@ -737,159 +797,121 @@ __device__ __forceinline__ float guard_change(const UpdArgs& a, float g) {
     }
     return g;
 }
+__device__ __forceinline__ float4 add4(float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); }
 
-// Momentum update of Section 6.2.1 over 64 x 64 weight tiles plus the biases:
-// g = sum of partial changes (+ pending G); v = lr*gs*g + m*v; w += v; then the
-// bf16 copy and its transpose.  Mode 1 adds the partial changes into G instead.
-// The kernel waits on DRAM latency: three CTAs per SM (80 registers, no spill),
-// and two partial planes' loads issued together, keep more bytes in flight.
-__global__ void __launch_bounds__(256, 3) k_update_bf16(UpdArgs a) {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.sse_out != nullptr) {
-        float s = 0.f;
-        for (int k = 0; k < a.n_sse; ++k) s += a.sse_part[k];
-        *a.sse_out = s;
-        if (!isfinite(s)) atomicOr(a.flags, kFlagNonfinite);
-    }
-    const int total = a.tile0[a.L];
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        int l = 0;
-        while (t >= a.tile0[l + 1]) ++l;
-        const LayerUpd& u = a.ly[l];
-        const int lt = t - a.tile0[l];
-        const int cols = (u.n_in + kUT - 1) / kUT;
-        const int rb = lt / cols, cb = lt - rb * cols;   // rb == row-tile count: the biases
-        const int rows_w = (u.n_out + kUT - 1) / kUT;
-        if (rb < rows_w) {
-            // Warp w covers rows 16*(w/2) .. +16 and columns 32*(w%2) .. +32 of the
-            // tile; a lane holds 4 consecutive rows x 4 consecutive columns, so the
-            // fp32 rows move as float4 (8 lanes: one 128-byte line per row) and
-            // both bf16 copies as 8-byte pieces (the transposed copy's 4 rows are
-            // the lane's own).  Layer sizes are multiples of 8: a lane's 4 x 4
-            // block is either inside the layer or outside it.  All loads of the
-            // lane come before its stores.
-            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-            const int i = cb * kUT + (w & 1) * 32 + (lane & 7) * 4;
-            const int j0 = rb * kUT + (w >> 1) * 16 + (lane >> 3) * 4;
-            if (i < u.n_in && j0 < u.n_out) {
-                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                float4 gs[4], w4[4], v4[4];
-                const size_t e0 = (size_t)j0 * u.n_in + i;
-                const float* th = a.theta + u.woff + e0;
-                float* vv = a.V + u.woff + e0;
-                float* gg = a.G + u.woff + e0;
+// The bias blocks' and the error sum's reduction: slice k of `rows` partials,
+// then the slices in order (the same order on every run).
+__device__ __forceinline__ float slice_sum(const float* p, int rows, size_t pitch, int k, int slices) {
+    const int per = (rows + slices - 1) / slices;
+    const int lo = k * per, hi = min(rows, lo + per);
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = lo; r < hi; ++r) s += p[(size_t)r * pitch];
+    return s;
+}
+
+// Momentum update of Section 6.2.1: g = sum of partial changes (+ pending G);
+// v = lr*gs*g + m*v; w += v; then the bf16 copy.  Mode 1 adds the partial changes
+// into G instead.  Bound by DRAM: a block owns 2,048 consecutive weights, every
+// thread two float4 pieces whose loads (weights, changes, up to two partial
+// planes at a time) are all issued before the first store.
+__global__ void __launch_bounds__(kUpdThreads) k_update_bf16(const __grid_constant__ UpdArgs a) {
+    __shared__ float red[kUpdSlices][kUpdBiases];
+    const int t = threadIdx.x;
+    pdl_launch();
+    pdl_wait();
+    const int b = blockIdx.x;
+    if (b == a.blocks) {   // the last block: the group's error sum
+        float s = slice_sum(a.sse_part, a.n_sse, 1, t, kUpdThreads);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    gs[r] = z;
-                    v4[r] = z;
-                    w4[r] = *reinterpret_cast<const float4*>(th + (size_t)r * u.n_in);
-                    if (a.mode == 0) v4[r] = *reinterpret_cast<const float4*>(vv + (size_t)r * u.n_in);
-                }
-                if (a.mode != 2) {
-                    const size_t plane = (size_t)u.n_out * u.n_in;
-                    int s0 = 0;
-                    for (; s0 + 2 <= u.splits; s0 += 2) {
-                        const float* gp = u.gpart + s0 * plane + e0;
-                        float4 p0[4], p1[4];
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            p0[r] = __ldcs(reinterpret_cast<const float4*>(gp + (size_t)r * u.n_in));
-                            p1[r] = __ldcs(reinterpret_cast<const float4*>(gp + plane + (size_t)r * u.n_in));
-                        }
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            gs[r].x += p0[r].x;
-                            gs[r].y += p0[r].y;
-                            gs[r].z += p0[r].z;
-                            gs[r].w += p0[r].w;
-                            gs[r].x += p1[r].x;
-                            gs[r].y += p1[r].y;
-                            gs[r].z += p1[r].z;
-                            gs[r].w += p1[r].w;
-                        }
-                    }
-                    for (int s = s0; s < u.splits; ++s) {
-                        const float* gp = u.gpart + s * plane + e0;
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const float4 p = __ldcs(reinterpret_cast<const float4*>(gp + (size_t)r * u.n_in));
-                            gs[r].x += p.x;
-                            gs[r].y += p.y;
-                            gs[r].z += p.z;
-                            gs[r].w += p.w;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const size_t o = (size_t)r * u.n_in;
-                    if (a.mode == 1) {
-                        float4 g4 = *reinterpret_cast<const float4*>(gg + o);
-                        g4.x += gs[r].x;
-                        g4.y += gs[r].y;
-                        g4.z += gs[r].z;
-                        g4.w += gs[r].w;
-                        *reinterpret_cast<float4*>(gg + o) = g4;
-                    } else if (a.mode == 0) {
-                        const float4 gp4 = a.fold_g ? *reinterpret_cast<const float4*>(gg + o) : z;
-                        float* wc = &w4[r].x;
-                        float* vc = &v4[r].x;
-                        const float* gc = &gs[r].x;
-                        const float* pc = &gp4.x;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float vel = a.lr_gs * guard_change(a, gc[c] + pc[c]) + a.momentum * vc[c];
-                            vc[c] = vel;
-                            wc[c] += vel;
-                        }
-                        *reinterpret_cast<float4*>(vv + o) = v4[r];
-                        *reinterpret_cast<float4*>(a.theta + u.woff + e0 + o) = w4[r];
-                        if (a.fold_g) *reinterpret_cast<float4*>(gg + o) = z;
-                    }
-                    if (a.mode != 1) {
-                        __align__(8) __nv_bfloat162 h[2];
-                        h[0] = __floats2bfloat162_rn(w4[r].x, w4[r].y);
-                        h[1] = __floats2bfloat162_rn(w4[r].z, w4[r].w);
-                        *reinterpret_cast<uint2*>(u.wb + e0 + o) = *reinterpret_cast<const uint2*>(h);
-                    }
-                }
-                if (a.mode != 1) {
-                    // W_l^T rows i .. i+3, columns j0 .. j0+3
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        __align__(8) __nv_bfloat162 h[2];
-                        h[0] = __floats2bfloat162_rn((&w4[0].x)[c], (&w4[1].x)[c]);
-                        h[1] = __floats2bfloat162_rn((&w4[2].x)[c], (&w4[3].x)[c]);
-                        *reinterpret_cast<uint2*>(u.wt + (size_t)(i + c) * u.n_out + j0) =
-                            *reinterpret_cast<const uint2*>(h);
-                    }
-                }
-            }
-        } else {
-            // biases of this layer, spread over the `cols` tiles of the bias row (one
-            // tile with the rest idle left a long tail of dependent partial-sum loads);
-            // each bias sums its row-block partials in order, loads issued 16 ahead
-            const int per = (u.n_out + cols - 1) / cols;
-            const int j_hi = min(u.n_out, (cb + 1) * per);
-            for (int j = cb * per + threadIdx.x; j < j_hi; j += 256) {
-                const long long idx = u.boff + j;
-                float gsum = 0.f;
-                if (a.mode != 2) {
-#pragma unroll 16
-                    for (int mt = 0; mt < u.mtiles; ++mt) gsum += u.bias_part[(size_t)mt * u.n_out + j];
-                }
-                if (a.mode == 1) {
-                    a.G[idx] += gsum;
-                } else if (a.mode == 0) {
-                    if (a.fold_g) {
-                        gsum += a.G[idx];
-                        a.G[idx] = 0.f;
-                    }
-                    const float vel = a.lr_gs * guard_change(a, gsum) + a.momentum * a.V[idx];
-                    a.V[idx] = vel;
-                    a.theta[idx] += vel;
-                }
-            }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((t & 31) == 0) red[0][t >> 5] = s;
+        __syncthreads();
+        if (t == 0) {
+            s = 0.f;
+            for (int w = 0; w < kUpdThreads / 32; ++w) s += red[0][w];
+            *a.sse_out = s;
+            if (!isfinite(s)) atomicOr(a.flags, kFlagNonfinite);
         }
+        return;
+    }
+    int l = 0;
+    while (l + 1 < a.L && b >= a.ly[l + 1].block0) ++l;
+    const LayerUpd& u = a.ly[l];
+    if (b >= u.bias0) {
+        // biases: kUpdSlices threads share each one's row-block partials
+        const int j = (b - u.bias0) * kUpdBiases + (t & (kUpdBiases - 1)), k = t / kUpdBiases;
+        red[k][t & (kUpdBiases - 1)] =
+            j < u.n_out ? slice_sum(u.bias_part + j, a.mtiles, u.n_out, k, kUpdSlices) : 0.f;
+        __syncthreads();
+        if (t >= kUpdBiases || j >= u.n_out) return;
+        float g = 0.f;
+#pragma unroll
+        for (int q = 0; q < kUpdSlices; ++q) g += red[q][t];
+        const long long idx = u.boff + j;
+        if (a.mode == 1) {
+            a.G[idx] += g;
+        } else if (a.mode == 0) {
+            if (a.fold_g) {
+                g += a.G[idx];
+                a.G[idx] = 0.f;
+            }
+            const float vel = a.lr_gs * guard_change(a, g) + a.momentum * a.V[idx];
+            a.V[idx] = vel;
+            a.theta[idx] += vel;
+        }
+        return;
+    }
+    const long long e0 = (long long)(b - u.block0) * kUpdFloats + t * 4;
+    float4 g4[kUpdPieces], w4[kUpdPieces], v4[kUpdPieces];
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < kUpdPieces; ++k) {
+        const long long e = e0 + k * (kUpdThreads * 4);
+        g4[k] = w4[k] = v4[k] = z;
+        if (e >= u.nw) continue;
+        if (a.mode != 1) w4[k] = *reinterpret_cast<const float4*>(a.theta + u.woff + e);
+        if (a.mode == 0) v4[k] = *reinterpret_cast<const float4*>(a.V + u.woff + e);
+        if (a.mode == 1 || a.fold_g) g4[k] = *reinterpret_cast<const float4*>(a.G + u.woff + e);
+    }
+    float4 p4[kUpdPieces];
+#pragma unroll
+    for (int k = 0; k < kUpdPieces; ++k) p4[k] = z;
+#pragma unroll 2
+    for (int s = 0; s < a.splits; ++s) {
+#pragma unroll
+        for (int k = 0; k < kUpdPieces; ++k) {
+            const long long e = e0 + k * (kUpdThreads * 4);
+            if (e < u.nw) p4[k] = add4(p4[k], __ldcs(reinterpret_cast<const float4*>(u.gpart + s * u.nw + e)));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kUpdPieces; ++k) {
+        const long long e = e0 + k * (kUpdThreads * 4);
+        if (e >= u.nw) continue;
+        const float4 g = add4(p4[k], g4[k]);
+        if (a.mode == 1) {
+            *reinterpret_cast<float4*>(a.G + u.woff + e) = g;
+            continue;
+        }
+        if (a.mode == 0) {
+            const float* gc = &g.x;
+            float* wc = &w4[k].x;
+            float* vc = &v4[k].x;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float vel = a.lr_gs * guard_change(a, gc[c]) + a.momentum * vc[c];
+                vc[c] = vel;
+                wc[c] += vel;
+            }
+            *reinterpret_cast<float4*>(a.V + u.woff + e) = v4[k];
+            *reinterpret_cast<float4*>(a.theta + u.woff + e) = w4[k];
+            if (a.fold_g) *reinterpret_cast<float4*>(a.G + u.woff + e) = z;
+        }
+        __align__(8) __nv_bfloat162 h[2];
+        h[0] = __floats2bfloat162_rn(w4[k].x, w4[k].y);
+        h[1] = __floats2bfloat162_rn(w4[k].z, w4[k].w);
+        *reinterpret_cast<uint2*>(u.wb + e) = *reinterpret_cast<const uint2*>(h);
     }
 }
 
@@ -903,12 +925,13 @@ bool get_encoder() {
     return g_encode != nullptr;
 }
 
-// 2-D bf16 tensor map over a row-major [rows, cols] matrix with row pitch `ld`
-// elements, box = box_rows x 64 columns, 128-byte swizzle, zero fill.
-bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int ld, int box_rows) {
+// 2-D bf16 tensor map over a row-major [rows, cols] matrix (pitch cols), box =
+// box_rows x 64 columns, 128-byte swizzle, zero fill.  box_rows is the tile edge
+// for an operand whose rows run along K, BK for one whose rows run along M or N.
+bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
+    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims,
                           strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -917,11 +940,16 @@ bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int ld, in
     return r == CUDA_SUCCESS;
 }
 
-
-template <int BN, int MODE>
+template <int BN>
 cudaError_t gemm_setup() {
-    return cudaFuncSetAttribute(k_gemm<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                GemmCfg<BN, MODE>::kSmemBytes);
+    const void* fns[] = {(const void*)k_gemm<BN, MODE_FWD>, (const void*)k_gemm<BN, MODE_FWD_OUT>,
+                         (const void*)k_gemm<BN, MODE_DX>, (const void*)k_gemm_dw<BN>};
+    for (const void* f : fns) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   GemmCfg<BN>::kSmemBytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 std::mutex g_mu;
@@ -931,22 +959,35 @@ cudaError_t setup_all(int device) {
     std::lock_guard<std::mutex> lk(g_mu);
     if (device < 64 && g_ready[device]) return cudaSuccess;
     cudaError_t e;
-    if ((e = gemm_setup<256, MODE_FWD>()) != cudaSuccess) return e;
-    if ((e = gemm_setup<256, MODE_FWD_OUT>()) != cudaSuccess) return e;
-    if ((e = gemm_setup<256, MODE_DX>()) != cudaSuccess) return e;
-    if ((e = gemm_setup<256, MODE_DW>()) != cudaSuccess) return e;
+    if ((e = gemm_setup<64>()) != cudaSuccess) return e;
+    if ((e = gemm_setup<128>()) != cudaSuccess) return e;
+    if ((e = gemm_setup<256>()) != cudaSuccess) return e;
     if (device < 64) g_ready[device] = true;
     return cudaSuccess;
 }
 
-constexpr int kBN = 256;
+// Launch whose setup may overlap the previous kernel's tail (the kernel calls pdl_wait).
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*k)(P...), int grid_x, int grid_y, int threads, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid_x, grid_y);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, std::forward<A>(args)...);
+}
 
 }  // namespace
 
 struct Bf16Net {
     int L = 0;
     int n[BP_MAX_SIZES] = {0};
-    int cap = 0, cap_pad = 0;
+    int cap = 0;
     int num_sms = 0;
     float* theta = nullptr;
     float* V = nullptr;
@@ -955,20 +996,12 @@ struct Bf16Net {
     float guard = 0.f;          // fault guard of Section 8 (0: off)
     long long woff[BP_MAX_SIZES] = {0}, boff[BP_MAX_SIZES] = {0};
     bf16* wb[BP_MAX_SIZES] = {nullptr};     // W_l   [n_l, n_{l-1}]
-    bf16* wt[BP_MAX_SIZES] = {nullptr};     // W_l^T [n_{l-1}, n_l]
     bf16* act[BP_MAX_SIZES] = {nullptr};    // A_l   [cap, n_l], l >= 1
-    bf16* actT[BP_MAX_SIZES] = {nullptr};   // A_l^T [n_l, cap_pad], l = 0..L-1
     bf16* dlt[BP_MAX_SIZES] = {nullptr};    // delta_l [cap, n_l], l >= 1
-    bf16* dltT[BP_MAX_SIZES] = {nullptr};   // delta_l^T [n_l, cap_pad]
-    float* gpart[BP_MAX_SIZES] = {nullptr}; // [splits, n_l, n_{l-1}]
-    int splits[BP_MAX_SIZES] = {0};
+    float* gpart[BP_MAX_SIZES] = {nullptr}; // [max_splits, n_l, n_{l-1}]
+    int max_splits = 1;
     float* bpart[BP_MAX_SIZES] = {nullptr}; // [mtiles(cap), n_l]
-    float* sse_part = nullptr;              // [mtiles(cap) * tiles along n_L]
-    int n_sse_cap = 0;
-    // X^T runs on a stream of the net's own, forked from and joined back into
-    // the caller's stream, beside the hidden-delta GEMMs
-    cudaStream_t side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    float* sse_part = nullptr;              // [mtiles(cap) * 64-column tiles along n_L]
     std::vector<void*> allocs;
 };
 
@@ -982,62 +1015,69 @@ bool alloc(Bf16Net* b, void** p, size_t bytes) {
 
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
-// Splits of K (the batch) for a pooled-change GEMM of `tiles` output tiles:
-// the fewest that minimise, in units of one full-K tile's time on one SM,
-//   ceil(tiles * s / num_sms) / s     (waves of 1/s-K work items)
-//   + s * r                           (the s partial planes: written here, read by the update)
-// with r = (tile bytes of fp32 partials, out and back) / (tile MMA time) =
-// 8 BM BN / HBM  /  (2 BM BN K / (bf16 peak / SM)) = 4 F_sm / (K HBM); the
-// measured ratio of per-SM bf16 peak to HBM bandwidth, 12.7 TFLOP/s to
-// 6.8 TB/s, is 1.87 flop per byte.
-int pick_splits(int tiles, int kb_total, int num_sms, int cap_splits) {
-    if (tiles < 1) tiles = 1;
-    const double r = 4.0 * 1.87 / ((double)kb_total * BK);
-    int best = 1;
-    double best_cost = 0.0;
-    for (int s = 1; s <= cap_splits && s <= kb_total; ++s) {
-        const double waves = (double)(((long long)tiles * s + num_sms - 1) / num_sms) / s;
-        const double cost = waves + s * r * tiles;
-        if (s == 1 || cost < best_cost * (1.0 - 1e-9)) {
-            best = s;
-            best_cost = cost;
+int tiles_of(int M, int N, int bn) { return ceil_div(M, BM) * ceil_div(N, bn); }
+
+// Clocks of a K block (64 of K) of a 128 x bn tile with every SM busy, fitted to
+// whole steps at forced widths.  Half the width costs more than half the time:
+// each SM then re-reads A twice as often from L2.
+constexpr double kb_clocks(int bn) { return bn == 256 ? 560 : bn == 128 ? 380 : 250; }
+
+// Tile width of a launch.  A tile's time is its K loop or its epilogue, whichever
+// is longer (they overlap across tiles), once per wave of tiles over the SMs, plus
+// the other one at the end.  Narrow tiles fill the chip when the batch or the
+// layer is small: a 208-1024-32 step of 512 patterns takes 28.4 / 31.8 / 35.2 us
+// with all launches at 64 / 128 / 256 columns, the forward of 1,001 patterns of
+// 1024-2048-2048-512 54.5 / 38.2 / 45.5 (36.4 by this rule); large batches want
+// 256: 1024-2048-2048-512 at 8,192 540 / 365 / 318 us per step, 512-512-256 at
+// 16,384 37.9 / 30.5 / 27.7 us forward.
+int pick_bn(int M, int N, int kb, int num_sms) {
+    const int bns[3] = {256, 128, 64};
+    int best = 256;
+    double best_t = 0;
+    for (int bn : bns) {
+        const double waves = ceil_div(tiles_of(M, N, bn), num_sms);
+        const double k = kb * kb_clocks(bn), e = 1000.0 + 1200.0 * bn / 64;
+        const double t = waves * (k > e ? k : e) + (k > e ? e : k);
+        if (bn == 256 || t < best_t) {
+            best = bn;
+            best_t = t;
         }
     }
     return best;
 }
 
 template <int MODE>
-cudaError_t launch_gemm(const Bf16Net* b, const CUtensorMap& ma, const CUtensorMap& mb,
-                        GemmArgs g, cudaStream_t s) {
-    g.num_m = ceil_div(g.M, BM);
-    g.num_n = ceil_div(g.N, kBN);
+cudaError_t launch_gemm(const Bf16Net* b, const bf16* A, const bf16* Bop, GemmArgs g, cudaStream_t s) {
     g.kb_total = ceil_div(g.K, BK);
-    if (g.splits < 1) g.splits = 1;
-    g.kb_per_split = ceil_div(g.kb_total, g.splits);
-    g.splits = ceil_div(g.kb_total, g.kb_per_split);   // every split non-empty
+    const int bn = pick_bn(g.M, g.N, g.kb_total, b->num_sms);
+    g.num_m = ceil_div(g.M, BM);
+    g.num_n = ceil_div(g.N, bn);
     g.flags = b->flags;
-    const int items = g.num_m * g.num_n * g.splits;
+    CUtensorMap ma, mb;
+    const bool ok = make_map(&ma, A, g.M, g.K, BM) &&
+                    (MODE == MODE_DX ? make_map(&mb, Bop, g.K, g.N, BK) : make_map(&mb, Bop, g.N, g.K, bn));
+    if (!ok) return cudaErrorInvalidValue;
+    const int items = g.num_m * g.num_n;
     const int grid = items < b->num_sms ? items : b->num_sms;
-    k_gemm<kBN, MODE><<<grid, kGemmThreads, GemmCfg<kBN, MODE>::kSmemBytes, s>>>(ma, mb, g);
-    return cudaGetLastError();
+    switch (bn) {
+        case 64: return launch_pdl(k_gemm<64, MODE>, grid, 1, kGemmThreads, GemmCfg<64>::kSmemBytes, s, ma, mb, g);
+        case 128: return launch_pdl(k_gemm<128, MODE>, grid, 1, kGemmThreads, GemmCfg<128>::kSmemBytes, s, ma, mb, g);
+        default: return launch_pdl(k_gemm<256, MODE>, grid, 1, kGemmThreads, GemmCfg<256>::kSmemBytes, s, ma, mb, g);
+    }
 }
 
 GemmArgs blank_args() {
     GemmArgs g;
     memset(&g, 0, sizeof g);
-    g.splits = 1;
     return g;
 }
 
-// Forward pass of all layers; with T, also the output deltas (training).
+// Forward pass of all layers.  With T, also the output deltas (training), which
+// replace the outputs; without, the outputs go to act[L] (for a backward) and Y.
 cudaError_t run_forward(Bf16Net* b, const bf16* X, int B, const bf16* T, bf16* Y, cudaStream_t s) {
     const int L = b->L;
     for (int l = 1; l <= L; ++l) {
         const bf16* A = (l == 1) ? X : b->act[l - 1];
-        CUtensorMap ma, mb;
-        if (!make_map(&ma, A, B, b->n[l - 1], b->n[l - 1], BM) ||
-            !make_map(&mb, b->wb[l], b->n[l], b->n[l - 1], b->n[l - 1], kBN))
-            return cudaErrorInvalidValue;
         GemmArgs g = blank_args();
         g.M = B;
         g.N = b->n[l];
@@ -1047,128 +1087,139 @@ cudaError_t run_forward(Bf16Net* b, const bf16* X, int B, const bf16* T, bf16* Y
         if (l < L) {
             g.out = b->act[l];
             g.ldo = b->n[l];
-            g.out_t = b->actT[l];
-            g.ldt = b->cap_pad;
-            e = launch_gemm<MODE_FWD>(b, ma, mb, g, s);
+            e = launch_gemm<MODE_FWD>(b, A, b->wb[l], g, s);
         } else {
             if (T != nullptr) {
-                // training: the output deltas (rows and transposed) replace the outputs
                 g.aux = T;
                 g.ld_aux = b->n[L];
                 g.out2 = b->dlt[L];
-                g.ld2 = b->n[L];
-                g.out_t = b->dltT[L];
-                g.ldt = b->cap_pad;
                 g.bias_part = b->bpart[L];
                 g.sse_part = b->sse_part;
             } else {
-                g.out = (Y != nullptr) ? Y : b->act[L];
+                g.out = b->act[L];
                 g.ldo = b->n[L];
+                g.out2 = Y;
             }
-            e = launch_gemm<MODE_FWD_OUT>(b, ma, mb, g, s);
+            g.ld2 = b->n[L];
+            e = launch_gemm<MODE_FWD_OUT>(b, A, b->wb[l], g, s);
         }
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// How the pooled-change launch of a group of B patterns is cut: the tile width
+// and the number of K splits that minimise, in clocks,
+//   ceil(tiles * s / num_sms) * K blocks / s * kb_clocks     (waves of 1/s-K work items)
+//   + s * (fp32 partial planes written here and read by the update) / 3,285 B per clock
+//     (the measured 6.8 TB/s copy rate at 2.07 GHz).
+// All layers share the launch, so their tiles fill the last wave together:
+// 1024-2048-2048-512 has 224 tiles of 256 columns, 98% of three waves in two
+// splits (326 us per step; unsplit 334), 4096^5 has 2,048, 96% of 14 waves
+// unsplit; 512-512-256 at 2,048 patterns takes 35.0 / 31.8 / 31.1 us in 1 / 2 /
+// 3 splits of 64 columns, 40.7 / 36.5 / 34.7 of 256.
+constexpr int kMaxSplits = 16;
+struct DwPlan {
+    int bn, tiles, splits, kb_total, kb_per_split;
+};
+DwPlan dw_plan(const int* n, int L, int B, int num_sms, int max_splits) {
+    DwPlan p{};
+    p.kb_total = ceil_div(B, BK);
+    double best_cost = 0;
+    const int bns[3] = {256, 128, 64};
+    for (int bn : bns) {
+        int tiles = 0;
+        for (int l = 1; l <= L; ++l) tiles += tiles_of(n[l], n[l - 1], bn);
+        for (int s = 1; s <= max_splits && s <= p.kb_total; ++s) {
+            const double waves = (double)(((long long)tiles * s + num_sms - 1) / num_sms) / s;
+            const double cost = waves * p.kb_total * kb_clocks(bn) + s * (8.0 * BM * bn * tiles) / 3285;
+            if (best_cost == 0 || cost < best_cost * (1.0 - 1e-9)) {
+                best_cost = cost;
+                p.bn = bn;
+                p.tiles = tiles;
+                p.splits = s;
+            }
+        }
+    }
+    p.kb_per_split = ceil_div(p.kb_total, p.splits);
+    p.splits = ceil_div(p.kb_total, p.kb_per_split);   // every split non-empty
+    return p;
 }
 
 // Hidden deltas and pooled partial changes for every layer (deltas of layer L
 // and the activations must already be in scratch).
-cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, cudaStream_t s) {
+cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, const DwPlan& p, cudaStream_t s) {
     const int L = b->L;
-    // X^T for the first layer's pooled change, on the side stream: it reads only
-    // X, so it overlaps the hidden-delta GEMMs (one 8.4 KB transpose block fits
-    // beside a GEMM CTA on an SM).  The fork orders it after everything already
-    // on s, the previous group's read of the same buffer included; the join
-    // orders the pooled-change GEMMs after it.
-    {
-        cudaError_t e = cudaEventRecord(b->fork, s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
-        if (e != cudaSuccess) return e;
-        dim3 grid(ceil_div(b->n[0], 64), ceil_div(B, 64));
-        k_transpose<<<grid, 256, 0, b->side>>>(X, B, b->n[0], b->n[0], b->actT[0], b->cap_pad);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaEventRecord(b->join, b->side);
-        if (e != cudaSuccess) return e;
-    }
-    cudaError_t e_dx = cudaSuccess;
-    for (int l = L; l >= 2 && e_dx == cudaSuccess; --l) {
-        // delta_{l-1} = (delta_l W_l) * a (1 - a):  A = delta_l [B, n_l], B-operand = W_l^T
-        CUtensorMap ma, mb;
-        if (!make_map(&ma, b->dlt[l], B, b->n[l], b->n[l], BM) ||
-            !make_map(&mb, b->wt[l], b->n[l - 1], b->n[l], b->n[l], kBN)) {
-            e_dx = cudaErrorInvalidValue;
-            break;
-        }
+    for (int l = L; l >= 2; --l) {
+        // delta_{l-1} = (delta_l W_l) * a (1 - a):  A = delta_l [B, n_l], B-operand = W_l along K
         GemmArgs g = blank_args();
         g.M = B;
         g.N = b->n[l - 1];
         g.K = b->n[l];
-        g.out = (l - 1 >= 2) ? b->dlt[l - 1] : nullptr;
+        g.out = b->dlt[l - 1];
         g.ldo = b->n[l - 1];
-        g.out_t = b->dltT[l - 1];
-        g.ldt = b->cap_pad;
         g.aux = b->act[l - 1];
         g.ld_aux = b->n[l - 1];
         g.bias_part = b->bpart[l - 1];
-        e_dx = launch_gemm<MODE_DX>(b, ma, mb, g, s);
-    }
-    // joined on every path, so that a stream capture on s stays whole
-    const cudaError_t e_join = cudaStreamWaitEvent(s, b->join, 0);
-    if (e_dx != cudaSuccess) return e_dx;
-    if (e_join != cudaSuccess) return e_join;
-    for (int l = 1; l <= L; ++l) {
-        // G_l = delta_l^T A_{l-1}: A = delta_l^T [n_l, B], B-operand = A_{l-1}^T [n_{l-1}, B]
-        CUtensorMap ma, mb;
-        if (!make_map(&ma, b->dltT[l], b->n[l], B, b->cap_pad, BM) ||
-            !make_map(&mb, b->actT[l - 1], b->n[l - 1], B, b->cap_pad, kBN))
-            return cudaErrorInvalidValue;
-        GemmArgs g = blank_args();
-        g.M = b->n[l];
-        g.N = b->n[l - 1];
-        g.K = B;
-        g.gpart = b->gpart[l];
-        g.splits = b->splits[l];
-        const int tiles = ceil_div(g.M, BM) * ceil_div(g.N, kBN);
-        g.splits = pick_splits(tiles, ceil_div(B, BK), b->num_sms, b->splits[l]);
-        cudaError_t e = launch_gemm<MODE_DW>(b, ma, mb, g, s);
+        const cudaError_t e = launch_gemm<MODE_DX>(b, b->dlt[l], b->wb[l], g, s);
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    // G_l = delta_l^T A_{l-1}
+    DwArgs g{};
+    DwMaps maps;
+    memset(&maps, 0, sizeof maps);
+    g.L = L;
+    g.tiles = p.tiles;
+    g.splits = p.splits;
+    g.kb_per_split = p.kb_per_split;
+    g.kb_total = p.kb_total;
+    g.flags = b->flags;
+    int tile = 0;
+    for (int l = 1; l <= L; ++l) {
+        DwLayer& y = g.ly[l - 1];
+        y.M = b->n[l];
+        y.N = b->n[l - 1];
+        y.num_m = ceil_div(y.M, BM);
+        y.num_n = ceil_div(y.N, p.bn);
+        y.tile0 = tile;
+        tile += y.num_m * y.num_n;
+        y.gpart = b->gpart[l];
+        if (!make_map(&maps.a[l - 1], b->dlt[l], B, y.M, BK) ||
+            !make_map(&maps.b[l - 1], l == 1 ? X : b->act[l - 1], B, y.N, BK))
+            return cudaErrorInvalidValue;
+    }
+    const int items = p.tiles * p.splits;
+    const int grid = items < b->num_sms ? items : b->num_sms;
+    switch (p.bn) {
+        case 64: return launch_pdl(k_gemm_dw<64>, grid, 1, kGemmThreads, GemmCfg<64>::kSmemBytes, s, maps, g);
+        case 128: return launch_pdl(k_gemm_dw<128>, grid, 1, kGemmThreads, GemmCfg<128>::kSmemBytes, s, maps, g);
+        default: return launch_pdl(k_gemm_dw<256>, grid, 1, kGemmThreads, GemmCfg<256>::kSmemBytes, s, maps, g);
+    }
 }
 
-// B: patterns whose partial changes are pending (0: none).
-UpdArgs upd_args(Bf16Net* b, int B, int mode, bool fold, float lr_gs, float momentum, float* sse_out,
+// splits, mtiles: partial changes pending (0: none).
+UpdArgs upd_args(Bf16Net* b, int splits, int mtiles, int mode, bool fold, float lr_gs, float momentum, float* sse_out,
                  int n_sse) {
     UpdArgs a;
     memset(&a, 0, sizeof a);
     a.L = b->L;
-    int tiles = 0;
+    int blocks = 0;
     for (int l = 1; l <= b->L; ++l) {
         LayerUpd& u = a.ly[l - 1];
         u.n_out = b->n[l];
-        u.n_in = b->n[l - 1];
+        u.nw = (long long)b->n[l] * b->n[l - 1];
         u.woff = b->woff[l];
         u.boff = b->boff[l];
         u.gpart = b->gpart[l];
-        const int t = ceil_div(u.n_out, BM) * ceil_div(u.n_in, kBN);
-        u.splits = 0;
-        u.mtiles = 0;
-        if (mode != 2 && B > 0) {
-            // the same split of K = B as the pooled-change GEMM used
-            const int kbt = ceil_div(B, BK);
-            const int s0 = pick_splits(t, kbt, b->num_sms, b->splits[l]);
-            const int kps = ceil_div(kbt, s0);
-            u.splits = ceil_div(kbt, kps);
-            u.mtiles = ceil_div(B, BM);
-        }
         u.bias_part = b->bpart[l];
         u.wb = b->wb[l];
-        u.wt = b->wt[l];
-        a.tile0[l - 1] = tiles;
-        tiles += (ceil_div(u.n_out, kUT) + 1) * ceil_div(u.n_in, kUT);
+        u.block0 = blocks;
+        u.bias0 = blocks + ceil_div(u.nw, kUpdFloats);
+        blocks = u.bias0 + ceil_div(u.n_out, kUpdBiases);
     }
-    a.tile0[b->L] = tiles;
+    a.blocks = blocks;
+    a.splits = splits;
+    a.mtiles = mtiles;
     a.theta = b->theta;
     a.V = b->V;
     a.G = b->G;
@@ -1185,12 +1236,8 @@ UpdArgs upd_args(Bf16Net* b, int B, int mode, bool fold, float lr_gs, float mome
     return a;
 }
 
-cudaError_t launch_update(const UpdArgs& a, int num_sms, cudaStream_t s) {
-    int grid = a.tile0[a.L];
-    if (grid > num_sms * 8) grid = num_sms * 8;
-    if (grid < 1) grid = 1;
-    k_update_bf16<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_update(const UpdArgs& a, cudaStream_t s) {
+    return launch_pdl(k_update_bf16, a.blocks + (a.sse_out != nullptr ? 1 : 0), 1, kUpdThreads, 0, s, a);
 }
 
 }  // namespace
@@ -1207,7 +1254,7 @@ bp_status bf16_check_shape(const int* n, int L, int max_batch) {
             return BP_ESHAPE;
         }
     }
-    (void)max_batch;   // transposed copies use a pitch padded to 8; any batch works
+    (void)max_batch;   // any batch works
     return BP_OK;
 }
 
@@ -1229,7 +1276,6 @@ bp_status bf16_create(const int* n, int L, int max_batch, int num_sms, float* th
     b->L = L;
     for (int l = 0; l <= L; ++l) b->n[l] = n[l];
     b->cap = max_batch;
-    b->cap_pad = (max_batch + 7) & ~7;
     b->num_sms = num_sms;
     b->theta = theta;
     b->V = V;
@@ -1243,33 +1289,19 @@ bp_status bf16_create(const int* n, int L, int max_batch, int num_sms, float* th
     }
     bool ok = true;
     const int mt = ceil_div(max_batch, BM);
-    for (int l = 0; l <= L && ok; ++l) {
-        if (l >= 1) {
-            ok = ok && alloc(b, (void**)&b->wb[l], (size_t)n[l] * n[l - 1] * 2);
-            ok = ok && alloc(b, (void**)&b->wt[l], (size_t)n[l] * n[l - 1] * 2);
-            ok = ok && alloc(b, (void**)&b->act[l], (size_t)max_batch * n[l] * 2);
-            ok = ok && alloc(b, (void**)&b->dlt[l], (size_t)max_batch * n[l] * 2);
-            ok = ok && alloc(b, (void**)&b->dltT[l], (size_t)n[l] * b->cap_pad * 2);
-            const int tiles = ceil_div(n[l], BM) * ceil_div(n[l - 1], kBN);
-            b->splits[l] = pick_splits(tiles, ceil_div(max_batch, BK), num_sms, 16);
-            ok = ok && alloc(b, (void**)&b->gpart[l], (size_t)b->splits[l] * n[l] * n[l - 1] * 4);
-            ok = ok && alloc(b, (void**)&b->bpart[l], (size_t)mt * n[l] * 4);
-        }
-        if (l < L) ok = ok && alloc(b, (void**)&b->actT[l], (size_t)n[l] * b->cap_pad * 2);
+    b->max_splits = dw_plan(n, L, max_batch, num_sms, kMaxSplits).splits;
+    for (int l = 1; l <= L && ok; ++l) {
+        ok = ok && alloc(b, (void**)&b->wb[l], (size_t)n[l] * n[l - 1] * 2);
+        ok = ok && alloc(b, (void**)&b->act[l], (size_t)max_batch * n[l] * 2);
+        ok = ok && alloc(b, (void**)&b->dlt[l], (size_t)max_batch * n[l] * 2);
+        ok = ok && alloc(b, (void**)&b->gpart[l], (size_t)b->max_splits * n[l] * n[l - 1] * 4);
+        ok = ok && alloc(b, (void**)&b->bpart[l], (size_t)mt * n[l] * 4);
     }
-    b->n_sse_cap = mt * ceil_div(n[L], kBN) + mt * ceil_div(n[L], 32);
-    ok = ok && alloc(b, (void**)&b->sse_part, (size_t)b->n_sse_cap * 4);
+    ok = ok && alloc(b, (void**)&b->sse_part, (size_t)mt * ceil_div(n[L], 64) * 4);
     if (!ok) {
         g_msg = "cudaMalloc failed for the bfloat16 scratch buffers";
         bf16_destroy(b);
         return BP_ENOMEM;
-    }
-    if (cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess) {
-        g_msg = "could not create the bfloat16 path's side stream and events";
-        bf16_destroy(b);
-        return BP_ECUDA;
     }
     *out = b;
     return BP_OK;
@@ -1277,10 +1309,6 @@ bp_status bf16_create(const int* n, int L, int max_batch, int num_sms, float* th
 
 void bf16_destroy(Bf16Net* b) {
     if (b == nullptr) return;
-    if (b->side) cudaStreamSynchronize(b->side);
-    if (b->fork) cudaEventDestroy(b->fork);
-    if (b->join) cudaEventDestroy(b->join);
-    if (b->side) cudaStreamDestroy(b->side);
     for (void* p : b->allocs) cudaFree(p);
     delete b;
 }
@@ -1289,37 +1317,30 @@ void bf16_set_flags(Bf16Net* b, int* flags) { b->flags = flags; }
 void bf16_set_guard(Bf16Net* b, float guard) { b->guard = guard; }
 
 cudaError_t bf16_refresh_weights(Bf16Net* b, cudaStream_t s) {
-    UpdArgs a = upd_args(b, 0, 2, false, 0.f, 0.f, nullptr, 0);
-    return launch_update(a, b->num_sms, s);
+    return launch_update(upd_args(b, 0, 0, 2, false, 0.f, 0.f, nullptr, 0), s);
 }
 
 cudaError_t bf16_forward(Bf16Net* b, const void* X, int batch, void* Y, cudaStream_t s) {
-    cudaError_t e = run_forward(b, (const bf16*)X, batch, nullptr, b->act[b->L], s);
-    if (e != cudaSuccess || Y == nullptr) return e;
-    return cudaMemcpy2DAsync(Y, (size_t)b->n[b->L] * 2, b->act[b->L], (size_t)b->n[b->L] * 2,
-                             (size_t)b->n[b->L] * 2, batch, cudaMemcpyDeviceToDevice, s);
+    return run_forward(b, (const bf16*)X, batch, nullptr, (bf16*)Y, s);
 }
 
 cudaError_t bf16_backward(Bf16Net* b, const void* X, const void* T, int batch, float* sse,
                           bool /*g_dirty*/, cudaStream_t s) {
     const int L = b->L;
     const int nL = b->n[L];
-    dim3 grid(ceil_div(nL, 32), ceil_div(batch, 128));
-    k_output_delta<<<grid, 128, 0, s>>>(b->act[L], (const bf16*)T, batch, nL, nL, b->dlt[L],
-                                        b->dltT[L], b->cap_pad, b->bpart[L], b->sse_part,
-                                        ceil_div(nL, 32));
-    cudaError_t e = cudaGetLastError();
+    const int nc = ceil_div(nL, 64), mt = ceil_div(batch, BM);
+    cudaError_t e = launch_pdl(k_output_delta, nc, mt, 256, 0, s, b->act[L], (const bf16*)T, batch, nL, b->dlt[L],
+                               b->bpart[L], b->sse_part);
     if (e != cudaSuccess) return e;
-    e = run_backward(b, (const bf16*)X, batch, s);
+    const DwPlan p = dw_plan(b->n, L, batch, b->num_sms, b->max_splits);
+    e = run_backward(b, (const bf16*)X, batch, p, s);
     if (e != cudaSuccess) return e;
-    UpdArgs a = upd_args(b, batch, 1, false, 0.f, 0.f, sse, ceil_div(batch, 128) * ceil_div(nL, 32));
-    return launch_update(a, b->num_sms, s);
+    return launch_update(upd_args(b, p.splits, mt, 1, false, 0.f, 0.f, sse, mt * nc), s);
 }
 
 cudaError_t bf16_update(Bf16Net* b, float lr, float momentum, float grad_scale, cudaStream_t s) {
     // apply G only: no partial changes pending
-    UpdArgs a = upd_args(b, 0, 0, true, lr * grad_scale, momentum, nullptr, 0);
-    return launch_update(a, b->num_sms, s);
+    return launch_update(upd_args(b, 0, 0, 0, true, lr * grad_scale, momentum, nullptr, 0), s);
 }
 
 cudaError_t bf16_train(Bf16Net* b, const void* X, const void* T, int n_patterns, int minibatch,
@@ -1334,12 +1355,13 @@ cudaError_t bf16_train(Bf16Net* b, const void* X, const void* T, int n_patterns,
         const bf16* Ts = (const bf16*)T + p0 * trow;
         cudaError_t e = run_forward(b, Xs, B, Ts, nullptr, s);
         if (e != cudaSuccess) return e;
-        e = run_backward(b, Xs, B, s);
+        const DwPlan p = dw_plan(b->n, L, B, b->num_sms, b->max_splits);
+        e = run_backward(b, Xs, B, p, s);
         if (e != cudaSuccess) return e;
-        const int n_sse = ceil_div(B, BM) * ceil_div(b->n[L], kBN);
-        UpdArgs a = upd_args(b, B, 0, fold, lr * grad_scale, momentum,
-                             sse != nullptr ? sse + step : nullptr, n_sse);
-        e = launch_update(a, b->num_sms, s);
+        const int n_sse = tiles_of(B, b->n[L], pick_bn(B, b->n[L], ceil_div(b->n[L - 1], BK), b->num_sms));
+        e = launch_update(upd_args(b, p.splits, ceil_div(B, BM), 0, fold, lr * grad_scale, momentum,
+                                   sse != nullptr ? sse + step : nullptr, n_sse),
+                          s);
         if (e != cudaSuccess) return e;
         fold = false;
     }

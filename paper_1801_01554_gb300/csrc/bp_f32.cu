@@ -27,14 +27,16 @@
 // A training launch is a persistent cooperative kernel that loops over any
 // number of groups with a grid barrier between the phases; every wait in the
 // barrier is bounded and latches kFlagTimeout instead of hanging.  Groups of at
-// most 4 patterns run on one CTA instead (k_train_small), with the weights
-// resident in its shared memory for the whole launch.
+// most 16 patterns of a one-hidden-layer net run on one cluster instead
+// (bp_f32_cluster.cu), other nets' groups of at most 4 on one CTA
+// (k_train_small), with the weights resident on chip for the whole launch.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 
+#include "bp_f32_device.cuh"
 #include "bp_internal.h"
 
 namespace bp {
@@ -65,10 +67,6 @@ constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s per wait
 constexpr unsigned kWaitIters = 1u << 26;
 
 // ------------------------------------------------------------ small helpers
-// Logistic: CUDA's expf and the fast reciprocal divide (2 ulp, far inside the
-// float32 bar; for 1 + e^-x beyond 2^126 the quotient is 0, the logistic's value).
-__device__ __forceinline__ float sigmoid_f(float x) { return __fdividef(1.0f, 1.0f + expf(-x)); }
-
 // Checked build (-DBP_CHECK): phases test that their shared-memory regions fit
 // the launch's dynamic shared memory and that their rows and tile origins lie
 // inside their buffers; a failed test latches kFlagBounds (bp_check reports it)
@@ -93,30 +91,6 @@ __device__ __forceinline__ bool bounds_ok(bool ok, int* flags) {
     return true;
 }
 
-// Table-lookup logistic (Section 4.3, Figure 3): the logistic at 256 equally
-// spaced points over [-15, 15], built in shared memory by each CTA that runs a
-// forward pass with the table mode on.  Inputs outside the range take the end
-// values; inside, x is remapped to [0, 255], the integer part picks the entry
-// and the fractional part interpolates linearly to the next one.  NaN stays NaN.
-constexpr int kSigPoints = 256;
-__shared__ float s_sigtab[kSigPoints];
-
-__device__ void sigmoid_table_init(const F32View& v) {
-    if (v.sig_table)
-        for (int k = threadIdx.x; k < kSigPoints; k += blockDim.x)
-            s_sigtab[k] = sigmoid_f(-15.f + (30.f * (float)k) / (float)(kSigPoints - 1));
-}
-
-__device__ __forceinline__ float sigmoid_tab(float x) {
-    if (x != x) return x;
-    const float xc = fminf(fmaxf(x, -15.f), 15.f);
-    const float x1 = (xc + 15.f) * ((float)(kSigPoints - 1) / 30.f);
-    const int i = min((int)x1, kSigPoints - 2);   // x1 >= 0: truncation is the floor
-    const float f = x1 - (float)i;
-    const float t0 = s_sigtab[i];
-    return fmaf(f, s_sigtab[i + 1] - t0, t0);
-}
-
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -127,10 +101,6 @@ __device__ __forceinline__ unsigned long long global_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
 // Grid barrier for a cooperative launch.  bar[1] counts arrivals over every
 // launch on the net; bar[0] holds its value at the end of the previous launch.
 // Barrier k of a launch completes when the count reaches bar[0] + k * grid:
@@ -240,13 +210,6 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, unsigned parity, unsig
     const unsigned long long t0 = global_ns();
     while (!mbar_try(bar, parity) && global_ns() - t0 < limit_ns) {
     }
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
 // Starts the copy of theta[0, P) into shared memory Ws: one bulk copy on the
@@ -375,25 +338,6 @@ __device__ void load_rows(const F32View& v, const PatLayout& q, const float* X, 
         }
     }
 }
-
-// Butterfly reduce-scatter of V per-lane values over aligned groups of V lanes:
-// afterwards lane k of a group holds in v[0] the group's sum of value k mod V.
-// A binary-tree sum (Section 10.3), V - 1 shuffles for V sums.
-template <int V>
-__device__ __forceinline__ void reduce_scatter(float (&v)[V], int lane) {
-#pragma unroll
-    for (int half = V / 2; half >= 1; half >>= 1) {
-        const bool up = (lane & half) != 0;
-#pragma unroll
-        for (int k = 0; k < half; ++k) {
-            const float send = up ? v[k] : v[k + half];
-            const float keep = up ? v[k + half] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-        }
-    }
-}
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 // Units per lane group of the forward pass for a group size: every unit's
 // weights are read once per CTA, every activation row once per lane group.
@@ -813,14 +757,6 @@ __device__ __forceinline__ float guard_change(const F32View& v, float g) {
     }
     return g;
 }
-
-// The same test without an atomic per change: zeroes and counts into n_bad.
-__device__ __forceinline__ float guard_count(float guard, float g, unsigned& n_bad) {
-    const bool bad = guard > 0.f && !(fabsf(g) <= guard);
-    n_bad += bad ? 1u : 0u;
-    return bad ? 0.f : g;
-}
-
 
 __device__ __forceinline__ void bulk_load(float* smem_dst, const float* src, unsigned bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
@@ -1538,10 +1474,7 @@ cudaError_t set_smem_attr(size_t bytes) {
 }  // namespace
 
 // ------------------------------------------------------------ host side
-// Dynamic shared memory a CTA may use: the opt-in limit (227 KB on sm_103a)
-// minus room for the kernels' static shared arrays.
-constexpr size_t kStaticSmemReserve = 2048;
-constexpr size_t kSmemLimit = 227 * 1024 - kStaticSmemReserve;
+constexpr size_t kSmemLimit = kF32SmemLimit;
 
 long long f32_layout(F32View& v, const int* n, int L, int cap) {
     v.L = L;
@@ -1676,6 +1609,7 @@ cudaError_t f32_setup(int device) {
     if ((e = set_smem_attr<4>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_smem_attr<8>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_smem_attr<kWidePG>(kSmemLimit)) != cudaSuccess) return e;
+    if ((e = f32_cluster_setup()) != cudaSuccess) return e;
     if ((e = set_small_attr<1>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_small_attr<2>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_small_attr<4>(kSmemLimit)) != cudaSuccess) return e;

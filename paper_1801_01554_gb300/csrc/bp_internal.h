@@ -103,6 +103,11 @@ struct F32Plan {
     int split;       // training launches use the balanced weight phase (large minibatches)
 };
 
+// Dynamic shared memory a float32 CTA may use: the opt-in limit (227 KB on
+// sm_103a) minus room for the kernels' static shared arrays.
+constexpr size_t kStaticSmemReserve = 2048;
+constexpr size_t kF32SmemLimit = 227 * 1024 - kStaticSmemReserve;
+
 // --- float32 path (bp_f32.cu) -------------------------------------------
 // Fills the layout fields of v for the layer sizes and capacity; returns the
 // scratch floats A and D need together.
@@ -136,6 +141,14 @@ cudaError_t f32_train(const F32View& v, const float* X, const float* T, int n_pa
 bool f32_small_ok(const F32View& v, int minibatch);
 cudaError_t f32_train_small(const F32View& v, const float* X, const float* T, int n_patterns,
                             int minibatch, int n_steps, float* sse_out, cudaStream_t s);
+
+// Groups of a few patterns of a one-hidden-layer net on one cluster of up to 8
+// CTAs (bp_f32_cluster.cu); f32_cluster_ok says whether the net and group fit
+// (no pending change G is folded in).
+cudaError_t f32_cluster_setup();
+bool f32_cluster_ok(const F32View& v, int minibatch);
+cudaError_t f32_train_cluster(const F32View& v, const float* X, const float* T, int n_patterns,
+                              int minibatch, int n_steps, float* sse_out, cudaStream_t s);
 
 // Diagnostic mode (Section 8): num_sms CTAs each run the forward pass and error
 // of all `batch` patterns; per-CTA error sums to d_sse, SM ids to d_sm.

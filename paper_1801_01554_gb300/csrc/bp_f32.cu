@@ -63,94 +63,7 @@ constexpr int kWidePG = 32;       // patterns per pass of the whole-row-per-lane
 constexpr size_t kGradFloats = kNBuf * chunk_floats<kTU>() + 256;
 constexpr size_t kGradFloatsW = kNBuf * chunk_floats<kTUW>() + 256;   // balanced weight phase
 
-constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s per wait
-constexpr unsigned kWaitIters = 1u << 26;
-
 // ------------------------------------------------------------ small helpers
-// Checked build (-DBP_CHECK): phases test that their shared-memory regions fit
-// the launch's dynamic shared memory and that their rows and tile origins lie
-// inside their buffers; a failed test latches kFlagBounds (bp_check reports it)
-// and the phase skips its accesses.  Without BP_CHECK the tests compile away.
-extern __shared__ __align__(128) float g_dyn_smem[];   // every kernel's dynamic shared memory
-__device__ __forceinline__ const float* pattern_smem_base() { return g_dyn_smem; }
-__device__ __forceinline__ unsigned dyn_smem_floats() {
-    unsigned b;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(b));
-    return b / 4;
-}
-__device__ __forceinline__ bool bounds_ok(bool ok, int* flags) {
-#ifdef BP_CHECK
-    if (!ok) {
-        atomicOr(flags, kFlagBounds);
-        return false;
-    }
-#else
-    (void)ok;
-    (void)flags;
-#endif
-    return true;
-}
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Grid barrier for a cooperative launch.  bar[1] counts arrivals over every
-// launch on the net; bar[0] holds its value at the end of the previous launch.
-// Barrier k of a launch completes when the count reaches bar[0] + k * grid:
-// thread 0 of each CTA adds its arrival with a fire-and-forget release
-// reduction and then polls the count (no CTA has to relay a release).  The
-// wait is bounded; on a timeout the error word latches kFlagTimeout and the
-// function returns false in every thread of the CTA (the caller must then
-// return).  Counts compare modulo 2^32.
-__device__ __forceinline__ bool count_reached(unsigned v, unsigned target) {
-    return (int)(v - target) >= 0;
-}
-__device__ bool grid_barrier(unsigned* bar, unsigned target, int* flags, unsigned long long limit_ns) {
-    __syncthreads();
-    int ok = 1;
-    if (threadIdx.x == 0) {
-        // the release is cumulative: with the CTA barrier above it also orders
-        // every thread's earlier writes before the arrival (no separate fence)
-        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar + 1), "r"(1u) : "memory");
-        const unsigned long long t0 = global_ns();
-        unsigned it = 0;
-        while (!count_reached(ld_acquire(bar + 1), target)) {
-            ++it;
-            if (it > kWaitIters || ((it & 63u) == 0 && global_ns() - t0 > limit_ns)) {
-                atomicOr(flags, kFlagTimeout);
-                ok = 0;
-                break;
-            }
-        }
-    }
-    return __syncthreads_and(ok) != 0;
-}
-
-// Limit of the grid barrier's wait: 2 s, or in the checked build the limit a
-// test set on the net (bp_debug_wait_test), so that a test can make a wait run
-// out in about a millisecond.
-__device__ __forceinline__ unsigned long long wait_limit_ns(const F32View& v) {
-#ifdef BP_CHECK
-    return v.wait_ns != 0 ? v.wait_ns : kWaitNs;
-#else
-    (void)v;
-    return kWaitNs;
-#endif
-}
-
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
 // Sum held in thread 0 (deterministic order).
 __device__ float block_sum(float x) {
     __shared__ float red[kWarps];
@@ -374,21 +287,41 @@ __device__ void forward_layer(const float* W, int kp, int n_out, const float* s_
             const float* wr[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) wr[u] = W + (size_t)min(j0 + u, n_out - 1) * kp;
-            for (int k = s; k < K4; k += S) {
-                float4 a[PG];
+            if constexpr (V <= 16) {   // sums of even and odd columns, two multiply-adds an instruction
+                f32x2 acc2[V];
 #pragma unroll
-                for (int p = 0; p < PG; ++p) a[p] = ld4(s_in + p * kp + 4 * k);
+                for (int k = 0; k < V; ++k) acc2[k] = 0;
+                for (int k = s; k < K4; k += S) {
+                    ulonglong2 a[PG];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const float4 w = ld4(wr[u] + 4 * k);
+                    for (int p = 0; p < PG; ++p) a[p] = ld4x2(s_in + p * kp + 4 * k);
 #pragma unroll
-                    for (int p = 0; p < PG; ++p) {
-                        float t = acc[u * PG + p];
-                        t = fmaf(w.x, a[p].x, t);
-                        t = fmaf(w.y, a[p].y, t);
-                        t = fmaf(w.z, a[p].z, t);
-                        t = fmaf(w.w, a[p].w, t);
-                        acc[u * PG + p] = t;
+                    for (int u = 0; u < U; ++u) {
+                        const ulonglong2 w = ld4x2(wr[u] + 4 * k);
+#pragma unroll
+                        for (int p = 0; p < PG; ++p)
+                            acc2[u * PG + p] = fma2(w.y, a[p].y, fma2(w.x, a[p].x, acc2[u * PG + p]));
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < V; ++k) acc[k] = sum2(acc2[k]);
+            } else {   // 32 sums: pairs would take 64 registers
+                for (int k = s; k < K4; k += S) {
+                    float4 a[PG];
+#pragma unroll
+                    for (int p = 0; p < PG; ++p) a[p] = ld4(s_in + p * kp + 4 * k);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const float4 w = ld4(wr[u] + 4 * k);
+#pragma unroll
+                        for (int p = 0; p < PG; ++p) {
+                            float t = acc[u * PG + p];
+                            t = fmaf(w.x, a[p].x, t);
+                            t = fmaf(w.y, a[p].y, t);
+                            t = fmaf(w.z, a[p].z, t);
+                            t = fmaf(w.w, a[p].w, t);
+                            acc[u * PG + p] = t;
+                        }
                     }
                 }
             }
@@ -425,25 +358,20 @@ __device__ void forward_layer_lanes(const float* W, int kp, int n_out, const flo
         int wo[U];   // row offsets (rows past the layer repeat its last row)
 #pragma unroll
         for (int u = 0; u < U; ++u) wo[u] = min(j0 + u, n_out - 1) * kp;
-        float acc[U];
+        f32x2 acc[U];   // sums of even and odd columns
 #pragma unroll
-        for (int u = 0; u < U; ++u) acc[u] = 0.f;
+        for (int u = 0; u < U; ++u) acc[u] = 0;
         for (int k = 0; k < K4; ++k) {
-            const float4 x = ld4(a + 4 * k);
+            const ulonglong2 x = ld4x2(a + 4 * k);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const float4 w = ld4(W + wo[u] + 4 * k);
-                float t = acc[u];
-                t = fmaf(w.x, x.x, t);
-                t = fmaf(w.y, x.y, t);
-                t = fmaf(w.z, x.z, t);
-                t = fmaf(w.w, x.w, t);
-                acc[u] = t;
+                const ulonglong2 w = ld4x2(W + wo[u] + 4 * k);
+                acc[u] = fma2(w.y, x.y, fma2(w.x, x.x, acc[u]));
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j0 + u < n_out) s_out[p * kp_out + j0 + u] = table ? sigmoid_tab(acc[u]) : sigmoid_f(acc[u]);
+            if (j0 + u < n_out) s_out[p * kp_out + j0 + u] = table ? sigmoid_tab(sum2(acc[u])) : sigmoid_f(sum2(acc[u]));
     }
 }
 
@@ -473,24 +401,20 @@ __device__ void forward_layer_blocked(const float* W, int kp, int n_out, const f
         const float* w1 = W + min(j0 + 1, n_out - 1) * kp;
         const float* w2 = W + min(j0 + 2, n_out - 1) * kp;
         const float* w3 = W + min(j0 + 3, n_out - 1) * kp;
-        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+        f32x2 c0[4] = {0, 0, 0, 0}, c1[4] = {0, 0, 0, 0};   // sums of even and odd columns
 #pragma unroll 2
         for (int k = 0; k < K4; ++k) {
-            const float4 x0 = ld4(a0 + 4 * k), x1 = ld4(a1 + 4 * k);
-            const float4 w[4] = {ld4(w0 + 4 * k), ld4(w1 + 4 * k), ld4(w2 + 4 * k), ld4(w3 + 4 * k)};
+            const ulonglong2 x0 = ld4x2(a0 + 4 * k), x1 = ld4x2(a1 + 4 * k);
+            const ulonglong2 w[4] = {ld4x2(w0 + 4 * k), ld4x2(w1 + 4 * k), ld4x2(w2 + 4 * k), ld4x2(w3 + 4 * k)};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                float t0 = c0[u], t1 = c1[u];
-                t0 = fmaf(w[u].x, x0.x, t0);
-                t1 = fmaf(w[u].x, x1.x, t1);
-                t0 = fmaf(w[u].y, x0.y, t0);
-                t1 = fmaf(w[u].y, x1.y, t1);
-                t0 = fmaf(w[u].z, x0.z, t0);
-                t1 = fmaf(w[u].z, x1.z, t1);
-                t0 = fmaf(w[u].w, x0.w, t0);
-                t1 = fmaf(w[u].w, x1.w, t1);
-                c0[u] = t0;
-                c1[u] = t1;
+                c0[u] = fma2(w[u].x, x0.x, c0[u]);
+                c1[u] = fma2(w[u].x, x1.x, c1[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                c0[u] = fma2(w[u].y, x0.y, c0[u]);
+                c1[u] = fma2(w[u].y, x1.y, c1[u]);
             }
         }
         float* o0 = s_out + p0 * kp_out + j0;
@@ -498,8 +422,8 @@ __device__ void forward_layer_blocked(const float* W, int kp, int n_out, const f
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (j0 + u < n_out) {
-                o0[u] = table ? sigmoid_tab(c0[u]) : sigmoid_f(c0[u]);
-                o1[u] = table ? sigmoid_tab(c1[u]) : sigmoid_f(c1[u]);
+                o0[u] = table ? sigmoid_tab(sum2(c0[u])) : sigmoid_f(sum2(c0[u]));
+                o1[u] = table ? sigmoid_tab(sum2(c1[u])) : sigmoid_f(sum2(c1[u]));
             }
         }
     }
@@ -558,17 +482,26 @@ __device__ void hidden_delta_lanes(const float* Wn, int kpn, int n, int nn, cons
 #pragma unroll
         for (int u = 0; u < U; ++u) acc[u] = 0.f;
         if (i0 + U <= kpn) {   // the row piece lies inside the padded row
+            f32x2 acc2[U / 2];   // pairs of units
+#pragma unroll
+            for (int u = 0; u < U / 2; ++u) acc2[u] = 0;
+#pragma unroll 2
             for (int j = 0; j < nn; ++j) {
                 const float d = dnt[j * PG + p];
+                const f32x2 dd = pack2(d, d);
                 const float* wrow = Wn + (size_t)j * kpn + i0;
 #pragma unroll
                 for (int q = 0; q < U / 4; ++q) {
-                    const float4 w = ld4(wrow + 4 * q);
-                    acc[4 * q] = fmaf(d, w.x, acc[4 * q]);
-                    acc[4 * q + 1] = fmaf(d, w.y, acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(d, w.z, acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(d, w.w, acc[4 * q + 3]);
+                    const ulonglong2 w = ld4x2(wrow + 4 * q);
+                    acc2[2 * q] = fma2(dd, w.x, acc2[2 * q]);
+                    acc2[2 * q + 1] = fma2(dd, w.y, acc2[2 * q + 1]);
                 }
+            }
+#pragma unroll
+            for (int u = 0; u < U / 2; ++u) {
+                const float2 t = unpack2(acc2[u]);
+                acc[2 * u] = t.x;
+                acc[2 * u + 1] = t.y;
             }
         } else {
             for (int j = 0; j < nn; ++j) {
@@ -961,9 +894,11 @@ __device__ bool weight_phase(const F32View& v, int B, bool fused, bool fold_g, f
             if (fused) v_old = __ldcg(v.V + idx);
             if (!fused || fold_g) g_old = __ldcg(v.G + idx);
         }
-        float acc[TU * 4];   // unit u, column q of this lane's quad at u * 4 + q
+        f32x2 acc2[TU / 2][4];   // units 2 u and 2 u + 1, column q of this lane's quad
 #pragma unroll
-        for (int q = 0; q < TU * 4; ++q) acc[q] = 0.f;
+        for (int u = 0; u < TU / 2; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc2[u][q] = 0;
         bool all_got = true;   // this thread's waits all arrived
         bool stop = false;     // thread 0: a wait ran out, no more copies
         for (int c = c0; c < c1; ++c) {
@@ -995,18 +930,17 @@ __device__ bool weight_phase(const F32View& v, int B, bool fused, bool fold_g, f
                     const int p = warp * kWarpRows + 4 * i + pl;   // row of the chunk
                     const int dsw = (p >> 2) & 1;
                     const float4 a = *reinterpret_cast<const float4*>(As + p * kTJ + ((cq ^ (p & 7)) << 2));
-                    const float av[4] = {a.x, a.y, a.z, a.w};
+                    const f32x2 av[4] = {pack2(a.x, a.x), pack2(a.y, a.y), pack2(a.z, a.z), pack2(a.w, a.w)};
 #pragma unroll
                     for (int h = 0; h < TU / kDB; ++h) {   // one delta block (8 units) at a time
                         const float* Dh = Ds + h * kPC * kDB + p * kDB;
-                        const float4 d0 = *reinterpret_cast<const float4*>(Dh + (dsw << 2));
-                        const float4 d1 = *reinterpret_cast<const float4*>(Dh + ((1 ^ dsw) << 2));
-                        const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+                        const ulonglong2 d0 = ld4x2(Dh + (dsw << 2));
+                        const ulonglong2 d1 = ld4x2(Dh + ((1 ^ dsw) << 2));
+                        const f32x2 dv[4] = {d0.x, d0.y, d1.x, d1.y};
 #pragma unroll
-                        for (int u = 0; u < 8; ++u)
+                        for (int u = 0; u < 4; ++u)
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                acc[(h * 8 + u) * 4 + q] = fmaf(dv[u], av[q], acc[(h * 8 + u) * 4 + q]);
+                            for (int q = 0; q < 4; ++q) acc2[h * 4 + u][q] = fma2(dv[u], av[q], acc2[h * 4 + u][q]);
                     }
                 }
             }
@@ -1028,6 +962,15 @@ __device__ bool weight_phase(const F32View& v, int B, bool fused, bool fold_g, f
         }
         // a wait ran out: thread 0 has waited for (or drained) every copy it issued
         if (__syncthreads_or(!all_got || stop)) return false;
+        float acc[TU * 4];   // unit u, column q of this lane's quad at u * 4 + q
+#pragma unroll
+        for (int u = 0; u < TU / 2; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 t = unpack2(acc2[u][q]);
+                acc[8 * u + q] = t.x;
+                acc[8 * u + 4 + q] = t.y;
+            }
         // sum over the 4 pattern lanes (lane bits 4, 3), halving the values at
         // each level: afterwards the lane holds values 0 .. TU - 1 of units
         // ub .. ub + TU / 4 - 1, ub = TU / 2 bit4 + TU / 4 bit3 (each sum is

@@ -31,7 +31,6 @@ constexpr int kCThreads = 512;   // most threads of a CTA
 constexpr int kStagesX = 4;      // pattern rows in flight (passes)
 constexpr int kLoaders = 3;      // warps that copy pattern rows
 constexpr int kHelpers = 32 * (kLoaders + 1);   // and one for output biases and error sums
-constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s
 
 // Shared-memory offsets in floats, and the split of the net over the cluster.
 struct ClusterPlan {
@@ -41,54 +40,6 @@ struct ClusterPlan {
     int threads, uthr, outs, pg;   // threads; those of the units and of the output sums, whole warps
     int xb, tb, h, d1, d2, w2, v2, g2, b2, vb2, gb2, part, e2, total;
 };
-
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Orders this CTA's shared-memory writes, remote ones included, before the
-// peers' reads after it (release / acquire at cluster scope).
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-// Stores x at p in CTA `rank`'s shared memory and counts its 4 bytes on that CTA's bar.
-__device__ __forceinline__ void st_remote(float* p, uint64_t* bar, unsigned rank, float x) {
-    uint32_t a, b;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(smem_u32(bar)), "r"(rank));
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a),
-                 "r"(__float_as_uint(x)), "r"(b)
-                 : "memory");
-}
-__device__ __forceinline__ void arm(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// Bounded wait for the bytes of a phase; false (kFlagTimeout latched) if it ran out.
-__device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, int* flags) {
-    unsigned long long t0 = 0;
-    for (unsigned it = 0;; ++it) {
-        unsigned done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((it & 255u) == 0) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (it == 0) t0 = t;
-            else if (t - t0 > kWaitNs) {
-                atomicOr(flags, kFlagTimeout);
-                return false;
-            }
-        }
-    }
-}
 
 // Sums of PG values over aligned groups of S lanes (PG <= S, powers of two):
 // afterwards lane k of a group holds the sum of value k mod PG.
@@ -139,6 +90,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                     const float* T, int n_patterns, int minibatch, int n_steps, float* sse_out) {
     extern __shared__ __align__(128) float sm[];
     __shared__ __align__(8) uint64_t s_bar[2];   // bytes of the output sums, one barrier per buffer
+    if (!bounds_ok((unsigned)c.total <= dyn_smem_floats() && minibatch <= 2 * PG, v.flags)) return;   // in every CTA alike
     const int tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x;
     const int rank = (int)cluster_rank();
     const int n0 = v.n[0], H = v.n[1], n2 = v.n[2];
@@ -285,7 +237,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
             // Bytes of buffer `buf` from all CTAs.  A peer writes this buffer again two
             // passes on, after it has this CTA's sums of the next pass, which are sent
             // after the reads below.
-            ok = wait_bytes(s_bar + buf, parity, v.flags);
+            ok = wait_bytes(s_bar + buf, parity, v.flags, wait_limit_ns(v));
             if (ok && tid == 0) arm(s_bar + buf, C * n2 * PG * 4);
             // 3. outputs and output deltas
             for (int e = tid; e < n2 * PG; e += nthr) {

@@ -254,9 +254,7 @@ bp_status bp_check(bp_net* net, void* stream);
  *   calls on a device share the array and find the previous call's contents:
  *   the call clears what must start at zero, and calls that overlap on the GPU
  *   (different streams, or several host threads) race on it.
- *   Every minibatch size runs on the grid-wide persistent kernel (152 CTAs and
- *   two grid barriers per group), including groups of 1-4 patterns, which
- *   bp_train_epoch sends to its one-CTA kernel.
+ *   Groups run on the kernels that bp_train_epoch picks for their size.
  *   Asynchronous with respect to the host like bp_train_epoch.  Pointers are
  *   checked before any CUDA call: d_theta, d_V, d_X, d_T, d_sse and d_status
  *   must be 4-byte aligned.  Errors: BP_EINVAL, BP_ESHAPE, BP_ECUDA. */

@@ -136,6 +136,11 @@ __device__ __forceinline__ float warp_sum(float x) {
     return x;
 }
 
+// Programmatic dependent launch: wait for the kernels this one depends on (their
+// writes are then visible), and let the next kernel of the stream start its setup.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Butterfly reduce-scatter of V per-lane values over aligned groups of V lanes:
 // afterwards lane k of a group holds in v[0] the group's sum of value k mod V.
 // A binary-tree sum (Section 10.3), V - 1 shuffles for V sums.

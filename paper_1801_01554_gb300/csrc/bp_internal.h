@@ -126,8 +126,10 @@ cudaError_t f32_update(const F32View& v, long long n_params, cudaStream_t s);
 // Packed <-> padded parameter layouts (see F32View), on the host and on the device.
 void f32_pad_host(const F32View& v, const float* packed, float* padded);
 void f32_unpad_host(const F32View& v, const float* padded, float* packed);
-cudaError_t f32_pad_device(const F32View& v, const float* packed, float* padded, cudaStream_t s);
-cudaError_t f32_unpad_device(const F32View& v, const float* padded, float* packed, cudaStream_t s);
+// (the device forms convert caller's packed buffers to v.theta and v.V and back;
+// the first also clears n_zero <= 256 words, the second copies the error word)
+cudaError_t f32_pad_device(const F32View& v, const float* theta, const float* V, unsigned* zero, int n_zero, cudaStream_t s);
+cudaError_t f32_unpad_device(const F32View& v, float* theta, float* V, int* status, cudaStream_t s);
 // Persistent cooperative launch running `n_steps` groups of `minibatch` patterns
 // (the last may be ragged), one update after each.  fold_g: G holds a pending
 // change to add into the first update.

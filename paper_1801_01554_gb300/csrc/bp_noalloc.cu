@@ -149,18 +149,17 @@ extern "C" bp_status bp_train_epoch_noalloc(const int* layer_sizes, int n_layers
     cudaStream_t s = (cudaStream_t)stream;
     // the array keeps the last call's contents: the error word and the barrier
     // must start at zero
-    cudaError_t e = cudaMemsetAsync(base, 0, (size_t)(4 + bar_words) * sizeof(float), s);
-    if (e == cudaSuccess) e = f32_pad_device(v, d_theta, theta_pad, s);
-    if (e == cudaSuccess) e = f32_pad_device(v, d_V, V_pad, s);
-    if (e == cudaSuccess) {
+    cudaError_t e = f32_pad_device(v, d_theta, d_V, reinterpret_cast<unsigned*>(base), 4 + (int)bar_words, s);
+    const int n_steps = (int)(((long long)n_patterns + minibatch - 1) / minibatch);
+    if (e == cudaSuccess && f32_cluster_ok(v, minibatch)) {
+        e = f32_train_cluster(v, d_X, d_T, n_patterns, minibatch, n_steps, d_sse, s);
+    } else if (e == cudaSuccess && f32_small_ok(v, minibatch)) {
+        e = f32_train_small(v, d_X, d_T, n_patterns, minibatch, n_steps, d_sse, s);
+    } else if (e == cudaSuccess) {
         const F32Plan plan = f32_plan(v, minibatch, sms);
-        const int n_steps = (int)(((long long)n_patterns + minibatch - 1) / minibatch);
         e = f32_train(v, d_X, d_T, n_patterns, minibatch, n_steps, d_sse, false, plan, s);
     }
-    if (e == cudaSuccess) e = f32_unpad_device(v, theta_pad, d_theta, s);
-    if (e == cudaSuccess) e = f32_unpad_device(v, V_pad, d_V, s);
-    if (e == cudaSuccess && d_status != nullptr)
-        e = cudaMemcpyAsync(d_status, base, sizeof(int), cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = f32_unpad_device(v, d_theta, d_V, d_status, s);
     if (e != cudaSuccess) {
         snprintf(msg, sizeof msg, "bp_train_epoch_noalloc: %s", cudaGetErrorString(e));
         set_error_message(msg);

@@ -45,3 +45,25 @@ def test_cluster_groups_report_a_nonfinite_error_sum():
         with pytest.raises(bp.BPError) as e:
             net.check()
         assert e.value.status == bp.BP_ENONFINITE
+
+
+@pytest.mark.parametrize("sizes,n,mb", [((203, 60, 26), 41, 3), ((203, 60, 26), 70, 16), ((64, 33, 17, 9), 21, 2)])
+def test_noalloc_small_groups_match_bp_train_epoch(sizes, n, mb):
+    """The same kernels on the caller's buffers: the same bits."""
+    X, T, theta = problem(sizes, n, seed=34)
+    Xd = torch.tensor(X, dtype=torch.float32, device="cuda")
+    Td = torch.tensor(T, dtype=torch.float32, device="cuda")
+    sse = torch.zeros(2, -(-n // mb), device="cuda")
+    th = torch.tensor(theta, dtype=torch.float32, device="cuda")
+    V = torch.zeros_like(th)
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    with bp.Net(sizes, 0.05, 0.9, bp.BP_F32, max_batch=mb) as net:
+        net.set_weights(theta)
+        for _ in range(2):
+            net.train_epoch(Xd, Td, n, mb, sse[0])
+            bp.bp_train_epoch_noalloc(sizes, 0.05, 0.9, 1.0, th, V, Xd, Td, n, mb, sse[1], status)
+        net.check()
+        np.testing.assert_array_equal(th.cpu().numpy(), net.get_weights())
+        np.testing.assert_array_equal(V.cpu().numpy(), net.get_velocity())
+    np.testing.assert_array_equal(sse[0].cpu().numpy(), sse[1].cpu().numpy())
+    assert status.item() == 0

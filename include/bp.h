@@ -271,7 +271,8 @@ bp_status bp_train_epoch_noalloc(const int* layer_sizes, int n_layers, float lr,
  * barriers wait for out of reach, so that its first grid barrier runs out of
  * time; unreachable == 2 makes the first chunk copy of each CTA's weight phase
  * a copy that never comes (its barrier is armed for the bytes, no copy is
- * issued), so that the chunk waits run out.  Either way the launch latches the timeout,
+ * issued), so that the chunk waits run out; large groups, which run without
+ * chunks, wait for weights of which some bytes never come.  Either way the launch latches the timeout,
  * every CTA returns with every copy it issued landed and no update applied,
  * and bp_check reports BP_ETIMEOUT and resets the barrier; 0 turns both off.
  * Synchronises the device.  Errors: BP_EINVAL (NULL, a BP_BF16 net),

@@ -67,6 +67,7 @@ struct bp_net {
     float* D = nullptr;
     float* sse_part = nullptr;
     float* wpart = nullptr;
+    float* gpart = nullptr;
     unsigned* bar = nullptr;
     int* flags = nullptr;
     F32View view{};
@@ -99,6 +100,7 @@ void free_all(bp_net* net) {
     cudaFree(net->D);
     cudaFree(net->sse_part);
     cudaFree(net->wpart);
+    cudaFree(net->gpart);
     cudaFree(net->bar);
     cudaFree(net->flags);
     cudaFree(net->stage_X);
@@ -222,6 +224,8 @@ bp_status bp_create(const int* sizes, int n_layers, float lr, float momentum, in
         if (e == cudaSuccess) e = cudaMalloc(&net->wpart, (size_t)net->num_sms * 2 * 512 * sizeof(float));
         if (e == cudaSuccess) e = cudaMalloc(&net->bar, (size_t)bp::kBarWords * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMalloc(&net->flags, 4 * sizeof(int));
+        if (e == cudaSuccess && f32_large_shape_ok(v) && max_batch >= kLargeMinPerCta * net->num_sms)
+            e = cudaMalloc(&net->gpart, (size_t)net->num_sms * v.P * sizeof(float));
         if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc(scratch)"));
         e = cudaMemset(net->bar, 0, (size_t)bp::kBarWords * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMemset(net->flags, 0, 4 * sizeof(int));
@@ -235,6 +239,7 @@ bp_status bp_create(const int* sizes, int n_layers, float lr, float momentum, in
         v.D = net->D;
         v.sse_part = net->sse_part;
         v.wpart = net->wpart;
+        v.gpart = net->gpart;
         v.bar = net->bar;
         v.flags = net->flags;
         v.faults = reinterpret_cast<unsigned*>(net->flags + 1);
@@ -459,6 +464,10 @@ static bp_status run_epoch(bp_net* net, const void* d_X, const void* d_T, int n_
         // groups of a few patterns: one CTA keeps the weights resident
         BP_CUDA(f32_train_small(net->view, (const float*)d_X, (const float*)d_T, n_patterns,
                                 minibatch, n_steps, d_sse, s),
+                "training launch");
+    } else if (net->dtype == BP_F32 && f32_large_ok(net->view, minibatch, net->num_sms)) {
+        BP_CUDA(f32_train_large(net->view, (const float*)d_X, (const float*)d_T, n_patterns, minibatch,
+                                n_steps, d_sse, net->g_dirty, net->num_sms, s),
                 "training launch");
     } else if (net->dtype == BP_F32) {
         const F32Plan plan = f32_plan(net->view, minibatch, net->num_sms);

@@ -28,8 +28,9 @@
 // number of groups with a grid barrier between the phases; every wait in the
 // barrier is bounded and latches kFlagTimeout instead of hanging.  Groups of at
 // most 16 patterns of a one-hidden-layer net run on one cluster instead
-// (bp_f32_cluster.cu), other nets' groups of at most 4 on one CTA
-// (k_train_small), with the weights resident on chip for the whole launch.
+// (bp_f32_cluster.cu), its groups of 40 or more patterns per CTA with the sums of
+// changes in registers (bp_f32_large.cu), and other nets' groups of at most 4 on
+// one CTA (k_train_small), with the weights resident on chip for the whole launch.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1577,6 +1578,7 @@ cudaError_t f32_setup(int device) {
     if ((e = set_smem_attr<8>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_smem_attr<kWidePG>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = f32_cluster_setup()) != cudaSuccess) return e;
+    if ((e = f32_large_setup()) != cudaSuccess) return e;
     if ((e = set_small_attr<1>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_small_attr<2>(kSmemLimit)) != cudaSuccess) return e;
     if ((e = set_small_attr<4>(kSmemLimit)) != cudaSuccess) return e;

@@ -70,6 +70,7 @@ struct F32View {
     float* D;
     float* sse_part;      // one partial error sum per CTA of the pattern phase
     float* wpart;         // balanced weight phase (large groups): [CTA][2][16 x 32] tile sums, or null
+    float* gpart;         // large groups of one-hidden-layer nets: [CTA][P] sums of changes, or null
     unsigned* bar;        // grid barrier: [0] count at the end of the last launch, [1] arrival count
     int* flags;           // latched error bits
     float lr, momentum, grad_scale;
@@ -151,6 +152,20 @@ cudaError_t f32_cluster_setup();
 bool f32_cluster_ok(const F32View& v, int minibatch);
 cudaError_t f32_train_cluster(const F32View& v, const float* X, const float* T, int n_patterns,
                               int minibatch, int n_steps, float* sse_out, cudaStream_t s);
+
+// Large groups of a one-hidden-layer net (bp_f32_large.cu): each CTA keeps its sums
+// in registers; needs v.gpart of num_sms * P floats.  f32_large_shape_ok: the net
+// fits; f32_large_ok: and the group is worth it.
+// Patterns per CTA from which one pass (64 or 128 patterns, mostly fixed time: 45 us
+// at 203-120-26, 46 at 203-60-26) beats the tiled weight phase: 6,100 patterns take
+// 45.2 against 46.1 us at 203-120-26, 46.4 against 51.2 at 203-60-26; 4,096 take 29.1
+// and 36.7 in the tiled form.
+constexpr int kLargeMinPerCta = 40;
+cudaError_t f32_large_setup();
+bool f32_large_shape_ok(const F32View& v);
+bool f32_large_ok(const F32View& v, int minibatch, int num_sms);
+cudaError_t f32_train_large(const F32View& v, const float* X, const float* T, int n_patterns, int minibatch,
+                            int n_steps, float* sse_out, bool fold_g, int num_sms, cudaStream_t s);
 
 // Diagnostic mode (Section 8): num_sms CTAs each run the forward pass and error
 // of all `batch` patterns; per-CTA error sums to d_sse, SM ids to d_sm.

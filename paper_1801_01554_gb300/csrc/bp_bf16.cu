@@ -20,9 +20,10 @@
 // rows run along K is staged as it lies; one whose rows run along M or N (W_l in
 // the hidden delta, delta_l and A_{l-1} in the pooled change) is staged as 64 x
 // 64 blocks and handed to the tensor cores as an MN-major operand, so that no
-// transposed copy is ever written.  The update kernel sums the partial changes,
-// applies the momentum rule of Section 6.2.1 to the fp32 master weights and
-// rewrites the bf16 weight copy.  The kernels of a step are launched with
+// transposed copy is ever written.  The update applies the momentum rule of Section
+// 6.2.1 to the fp32 master weights and rewrites the bf16 weight copy: in the epilogue
+// of the pooled change where K is not split, else in a kernel that also sums the
+// partial changes.  The kernels of a step are launched with
 // programmatic stream serialisation: each sets up its barriers and TMEM while
 // its predecessor drains, and waits (griddepcontrol.wait) before it touches
 // global memory.  All device-side waits are bounded and latch kFlagTimeout.
@@ -57,7 +58,7 @@ constexpr int kGemmThreads = 64 + kEpiThreads;   // warp 0 TMA, warp 1 MMA, warp
 constexpr unsigned long long kWaitNs = 2000000000ull;
 constexpr unsigned kWaitIters = 1u << 28;
 
-enum Mode : int { MODE_FWD = 0, MODE_FWD_OUT = 1, MODE_DX = 2, MODE_DW = 3 };
+enum Mode : int { MODE_FWD = 0, MODE_FWD_OUT = 1, MODE_DX = 2, MODE_DW = 3, MODE_DWU = 4 };
 
 struct GemmArgs {
     int M, N, K;
@@ -124,6 +125,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
         : "memory");
     return done != 0;
 }
+// Whether the phase is complete, without waiting.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
 // Bounded wait.  Returns false if it ran out or another role aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, volatile int* abort_flag,
                                           int* flags) {
@@ -150,6 +163,15 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
         : "memory");
 }
 
+// True in one lane of the (converged) warp.  Unlike a test of the lane number it tells
+// the compiler that a single thread follows, so that the operands of the TMA and MMA
+// instructions can stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // Programmatic dependent launch: wait for the kernels this one depends on (their
 // writes are then visible), and let the next kernel of the stream start its setup.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -161,20 +183,17 @@ __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.laun
 //   MN-major: blocks of 64 K rows x 64 of M or N (128 bytes); 8 K rows are 1024
 //             bytes apart (stride offset), the next 64 of M or N one block, 8 KB
 //             (leading offset).
+// The upper word is constant; the lower one holds the address (in 16-byte units, below
+// 2^14) and the leading offset, so that stages and K steps are plain additions to it.
 constexpr uint32_t kMnBlockBytes = BK * 64 * 2;
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);   // stride offset, version 1, 128-byte swizzle
 template <bool MN>
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((MN ? kMnBlockBytes : 16u) >> 4) << 16;   // leading byte offset
-    d |= (uint64_t)(1024u >> 4) << 32;    // stride byte offset
-    d |= (uint64_t)1 << 46;               // descriptor version
-    d |= (uint64_t)2 << 61;               // 128-byte swizzle
-    return d;
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) {
+    return (addr >> 4) | (((MN ? kMnBlockBytes : 16u) >> 4) << 16);
 }
-// Bytes from one K step of UMMA_K to the next inside a stage.
+// From one K step of UMMA_K to the next inside a stage, in 16-byte units.
 template <bool MN>
-__device__ __forceinline__ constexpr uint32_t k_step_bytes() { return MN ? UMMA_K * 128 : UMMA_K * 2; }
+__device__ __forceinline__ constexpr uint32_t k_step_units() { return (MN ? UMMA_K * 128 : UMMA_K * 2) >> 4; }
 
 // Instruction descriptor of tcgen05.mma kind::f16: bf16 A and B, fp32 D, M x N
 // tile, each operand K-major or MN-major.
@@ -183,13 +202,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool 
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accumulate) {
+// One tcgen05.mma: operands by the lower words of their descriptors; the first one of
+// a tile overwrites the accumulator.
+template <uint32_t IDESC>
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(tmem_d),
+        "r"(a_lo), "r"(b_lo), "n"(kDescHi), "n"(IDESC), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -223,10 +245,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Logistic for bf16 outputs: hardware exp2 and the fast reciprocal divide (2 ulp;
-// an IEEE divide here cost a quarter of a training step in the epilogues).
-// For 1 + e^-x beyond 2^126 the quotient is 0, the logistic's value there.
-__device__ __forceinline__ float sigmoid_fast(float x) { return __fdividef(1.0f, 1.0f + __expf(-x)); }
+// Logistic for bf16 outputs: hardware exp2 and reciprocal (1 ulp each; an IEEE divide
+// here cost a quarter of a training step in the epilogues).  For 1 + e^-x beyond the
+// largest float the quotient is 0, the logistic's value there.
+__device__ __forceinline__ float sigmoid_fast(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + __expf(-x)));
+    return r;
+}
 
 __device__ __forceinline__ float bf16_round(float x) {
     return __bfloat162float(__float2bfloat16_rn(x));
@@ -235,24 +261,18 @@ __device__ __forceinline__ float bf16_round(float x) {
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // ------------------------------------------------------------ epilogue
-// 32 consecutive bf16 of one row as floats (16-byte loads when the row segment is whole).
-__device__ __forceinline__ void load_row32(float (&a)[32], const bf16* p, bool whole, int valid) {
-    if (whole) {
+// 32 consecutive bf16 of one row (pieces of 8 past `pieces` are zero), and as floats.
+struct Row32 {
+    uint4 u[4];
+};
+__device__ __forceinline__ void load_row32(Row32& r, const bf16* p, int pieces) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint4 u = reinterpret_cast<const uint4*>(p)[k];
-            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float2 f = __bfloat1622float2(h[q]);
-                a[k * 8 + 2 * q] = f.x;
-                a[k * 8 + 2 * q + 1] = f.y;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) a[c] = (c < valid) ? __bfloat162float(p[c]) : 0.f;
-    }
+    for (int k = 0; k < 4; ++k) r.u[k] = k < pieces ? reinterpret_cast<const uint4*>(p)[k] : make_uint4(0u, 0u, 0u, 0u);
+}
+__device__ __forceinline__ float row_value(const Row32& r, int c) {   // c is a compile-time constant
+    const uint4& u = r.u[c >> 3];
+    const uint32_t w = ((c >> 1) & 3) == 0 ? u.x : ((c >> 1) & 3) == 1 ? u.y : ((c >> 1) & 3) == 2 ? u.z : u.w;
+    return __uint_as_float((c & 1) ? (w & 0xffff0000u) : (w << 16));
 }
 
 // One 32-column chunk of a pooled-change tile: this lane's row m of the partial sums.
@@ -264,6 +284,18 @@ __device__ __forceinline__ void store_partial(float* gpart, int M, int N, int m,
         if (n0 + c < N) *reinterpret_cast<float4*>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
 }
 
+// 32 lanes x 16 consecutive fp32 columns from TMEM.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // One 32-column chunk of the tile for the 32 rows of one epilogue warp (this
 // lane's row m).  Values are rounded to bf16 and staged by rows in the warp's
 // 2 KB shared-memory block (16-byte pieces permuted by row so that the lanes'
@@ -273,45 +305,37 @@ __device__ __forceinline__ void store_partial(float* gpart, int M, int N, int m,
 // out: each lane adds its four rows of 8 columns, then the eight lanes of a
 // piece reduce-scatter them (7 shuffles).
 template <int MODE>
-__device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0, int n0, float (&v)[32], float& sse,
-                                               bool row_ok, bf16* sS, const float* sbias, float* colsum_slot) {
+__device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m0, int n0, float (&v)[32], float& sse,
+                                               bool row_ok, bf16* sS, const float* sbias, const Row32& aux,
+                                               float* colsum_slot) {
     const int N = g.N;
     const int lane = threadIdx.x & 31;
-    const bool whole = (n0 + 32 <= N);
     const int valid = min(32, N - n0);
     const bool with_t = (MODE == MODE_FWD_OUT) && (g.aux != nullptr);
-    float vals[32];
+    // values in place; they are rounded when they are packed below
     if (MODE == MODE_FWD || MODE == MODE_FWD_OUT) {
-        float b[32];   // the tile's biases, staged in shared memory (0 past N)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < 8; ++k) {   // the tile's biases, staged in shared memory (0 past N)
             const float4 f = reinterpret_cast<const float4*>(sbias)[k];
-            b[4 * k] = f.x;
-            b[4 * k + 1] = f.y;
-            b[4 * k + 2] = f.z;
-            b[4 * k + 3] = f.w;
+            v[4 * k] = sigmoid_fast(v[4 * k] + f.x);
+            v[4 * k + 1] = sigmoid_fast(v[4 * k + 1] + f.y);
+            v[4 * k + 2] = sigmoid_fast(v[4 * k + 2] + f.z);
+            v[4 * k + 3] = sigmoid_fast(v[4 * k + 3] + f.w);
         }
-        float t[32];
-        if (with_t) load_row32(t, g.aux + (size_t)m * g.ld_aux + n0, whole && row_ok, row_ok ? valid : 0);
+        if (with_t) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const bool ok = row_ok && (c < valid);
-            const float o = bf16_round(sigmoid_fast(v[c] + b[c]));
-            if (with_t) {
-                const float err = t[c] - o;
-                sse = ok ? fmaf(err, err, sse) : sse;
-                vals[c] = ok ? bf16_round(err * o * (1.f - o)) : 0.f;
-            } else {
-                vals[c] = ok ? o : 0.f;
+            for (int c = 0; c < 32; ++c) {
+                const float o = bf16_round(v[c]);
+                const float err = (row_ok && c < valid) ? row_value(aux, c) - o : 0.f;
+                sse = fmaf(err, err, sse);
+                v[c] = err * o * (1.f - o);
             }
         }
-    } else {   // MODE_DX: delta_{l-1} = (delta_l W_l) a (1 - a)
-        float a[32];
-        load_row32(a, g.aux + (size_t)m * g.ld_aux + n0, whole && row_ok, row_ok ? valid : 0);
+    } else {   // MODE_DX: delta_{l-1} = (delta_l W_l) a (1 - a); rows and columns past the edges have a = 0
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
-            const bool ok = row_ok && (c < valid);
-            vals[c] = ok ? bf16_round(v[c] * a[c] * (1.f - a[c])) : 0.f;
+            const float a = row_value(aux, c);
+            v[c] = v[c] * a * (1.f - a);
         }
     }
     // rows: A_l, A_L (and the caller's copy) or delta_L (training output layer), or delta_{l-1}
@@ -324,7 +348,7 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0,
     for (int k = 0; k < 4; ++k) {
         __align__(16) __nv_bfloat162 h[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(vals[8 * k + 2 * q], vals[8 * k + 2 * q + 1]);
+        for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(v[8 * k + 2 * q], v[8 * k + 2 * q + 1]);
         sS4[lane * 4 + (k ^ ((lane >> 1) & 3))] = *reinterpret_cast<const uint4*>(h);
     }
     __syncwarp();
@@ -366,6 +390,111 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m, int m0,
     __syncwarp();   // the staging block may be rewritten
 }
 
+// ------------------------------------------------------------ update arguments
+constexpr int kUpdThreads = 256;
+constexpr int kUpdPieces = 2;                                    // float4 pieces per thread of a weight block
+constexpr int kUpdFloats = kUpdThreads * kUpdPieces * 4;         // weights per block
+constexpr int kUpdBiases = 32, kUpdSlices = kUpdThreads / kUpdBiases;   // biases per block, threads per bias
+
+struct LayerUpd {
+    long long nw;               // n_out * n_in, a multiple of 64
+    int n_out;
+    long long woff, boff;       // offsets in theta / V / G
+    const float* gpart;         // [splits, n_out, n_in]
+    const float* bias_part;     // [mtiles, n_out]
+    bf16* wb;                   // [n_out, n_in]
+    int block0, bias0;          // first weight block of the layer; first bias block (counted apart)
+};
+struct UpdArgs {
+    int L;
+    LayerUpd ly[kMaxL];
+    int blocks, bias_blocks;    // weight blocks and bias blocks of all layers
+    int splits, mtiles;         // pending partial changes (0: none)
+    float* theta;
+    float* V;
+    float* G;
+    float lr_gs, momentum;
+    int mode;                   // 0: apply update; 1: accumulate into G; 2: refresh the bf16 copy
+    int fold_g;
+    const float* sse_part;
+    int n_sse;
+    float* sse_out;
+    int* flags;
+    float guard;          // > 0: fault guard of Section 8
+    unsigned* faults;     // changes the guard zeroed
+};
+
+// Fault guard of Section 8: a total weight change outside (-guard, guard), or
+// not a number, is set to zero and counted (off while guard <= 0).
+__device__ __forceinline__ float guard_change(const UpdArgs& a, float g) {
+    if (a.guard > 0.f && !(fabsf(g) <= a.guard)) {
+        atomicAdd(a.faults, 1u);
+        return 0.f;
+    }
+    return g;
+}
+__device__ __forceinline__ float4 add4(float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); }
+
+// One bias or error-sum block of an update, by 256 threads (t = 0 .. 255) with
+// 1 KB of shared memory; `sync` is their barrier.  Block b: bias blocks
+// [0, a.bias_blocks) layer by layer, then, if the group's error sum is wanted, one more.
+// (the slices of a sum, then the slices in order: the same order on every run)
+// The bias blocks' and the error sum's reduction: slice k of `rows` partials,
+// then the slices in order (the same order on every run).
+__device__ __forceinline__ float slice_sum(const float* p, int rows, size_t pitch, int k, int slices) {
+    const int per = (rows + slices - 1) / slices;
+    const int lo = k * per, hi = min(rows, lo + per);
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = lo; r < hi; ++r) s += p[(size_t)r * pitch];
+    return s;
+}
+
+template <class Sync>
+__device__ __forceinline__ void update_bias_block(const UpdArgs& a, int b, int t, float* red, Sync sync) {
+    if (b == a.bias_blocks) {   // the group's error sum
+        float s = slice_sum(a.sse_part, a.n_sse, 1, t, kUpdThreads);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((t & 31) == 0) red[t >> 5] = s;
+        sync();
+        if (t == 0) {
+            s = 0.f;
+            for (int w = 0; w < kUpdThreads / 32; ++w) s += red[w];
+            *a.sse_out = s;
+            if (!isfinite(s)) atomicOr(a.flags, kFlagNonfinite);
+        }
+        sync();
+        return;
+    }
+    int l = 0;
+    while (l + 1 < a.L && b >= a.ly[l + 1].bias0) ++l;
+    const LayerUpd& u = a.ly[l];
+    // kUpdSlices threads share each bias's row-block partials
+    const int i = t & (kUpdBiases - 1), k = t / kUpdBiases;
+    const int j = (b - u.bias0) * kUpdBiases + i;
+    red[k * kUpdBiases + i] = j < u.n_out ? slice_sum(u.bias_part + j, a.mtiles, u.n_out, k, kUpdSlices) : 0.f;
+    sync();
+    if (t < kUpdBiases && j < u.n_out) {
+        float g = 0.f;
+#pragma unroll
+        for (int q = 0; q < kUpdSlices; ++q) g += red[q * kUpdBiases + t];
+        const long long idx = u.boff + j;
+        if (a.mode == 1) {
+            a.G[idx] += g;
+        } else if (a.mode == 0) {
+            if (a.fold_g) {
+                g += a.G[idx];
+                a.G[idx] = 0.f;
+            }
+            const float vel = a.lr_gs * guard_change(a, g) + a.momentum * a.V[idx];
+            a.V[idx] = vel;
+            a.theta[idx] += vel;
+        }
+    }
+    sync();
+}
+
 // ------------------------------------------------------------ GEMM kernel
 // Tile order: groups of kGroupM row blocks, each group swept over all column
 // blocks (row block fastest), so that the tiles in flight on the 152 SMs share
@@ -399,6 +528,10 @@ struct GemmCfg {
         1024 + kRingBytes + kColsumBytes + kStageOutBytes + kBiasBytes + 256;
 };
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)m) : "memory");
+}
+
 // A work item of a GEMM launch: a tile and its run of K blocks.
 struct Item {
     int mb, nb, kb0, kb1;
@@ -416,6 +549,16 @@ struct OneGemm {
         Item w{0, 0, 0, g.kb_total, 0, 0};
         tile_coords(it, g.num_m, g.num_n, w.mb, w.nb);
         return w;
+    }
+    // The launch's parameters are read here once, while the previous kernel drains: their
+    // first read misses the constant cache.
+    __device__ void touch() const {
+        asm volatile("" ::"r"(g.N), "r"(g.kb_total), "l"(g.bias), "l"(g.out), "r"(g.ldo), "l"(g.out2), "r"(g.ld2),
+                     "l"(g.aux), "r"(g.ld_aux), "l"(g.bias_part), "l"(g.sse_part), "l"(g.flags));
+    }
+    __device__ void prefetch_maps() const {
+        prefetch_map(ma);
+        prefetch_map(mb_);
     }
     __device__ const CUtensorMap* map_a(const Item&) const { return ma; }
     __device__ const CUtensorMap* map_b(const Item&) const { return mb_; }
@@ -439,8 +582,30 @@ struct DwGemm {
         w.kb1 = min(g.kb_total, w.kb0 + g.kb_per_split);
         return w;
     }
+    __device__ void touch() const {
+        asm volatile("" ::"r"(g.splits), "r"(g.kb_per_split), "r"(g.kb_total), "l"(g.flags));
+        for (int l = 0; l < g.L; ++l) asm volatile("" ::"r"(g.ly[l].N), "l"(g.ly[l].gpart));
+    }
+    __device__ void prefetch_maps() const {
+        for (int l = 0; l < g.L; ++l) {
+            prefetch_map(&maps.a[l]);
+            prefetch_map(&maps.b[l]);
+        }
+    }
     __device__ const CUtensorMap* map_a(const Item& w) const { return &maps.a[w.l]; }
     __device__ const CUtensorMap* map_b(const Item& w) const { return &maps.b[w.l]; }
+};
+
+// The same with the update in the epilogue (one K split).
+struct DwuGemm : DwGemm {
+    static constexpr int kMode = MODE_DWU;
+    const UpdArgs& u;
+    __device__ DwuGemm(const DwArgs& g_, const DwMaps& m_, const UpdArgs& u_) : DwGemm{g_, m_}, u(u_) {}
+    __device__ void touch() const {
+        DwGemm::touch();
+        asm volatile("" ::"r"(u.bias_blocks), "l"(u.theta), "l"(u.V), "f"(u.lr_gs), "r"(u.fold_g), "f"(u.guard));
+        for (int l = 0; l < g.L; ++l) asm volatile("" ::"l"(u.ly[l].woff), "l"(u.ly[l].wb), "l"(u.ly[l].bias_part));
+    }
 };
 
 // Copies one operand's stage: ROWS of M or N by BK of K from K block kb.
@@ -452,6 +617,65 @@ __device__ __forceinline__ void load_operand(uint8_t* dst, const CUtensorMap* ma
     } else {
         tma_load_2d(dst, map, kb * BK, row0, bar);
     }
+}
+
+// Momentum update (as k_update_bf16) of 32 rows x 16 columns of a pooled-change
+// tile, from the warp's TMEM lanes: the sums pass through the warp's 2 KB of shared
+// memory (16-byte pieces permuted by row), after which lane (row lane / 4 + 8 j,
+// piece lane % 4) owns 4 consecutive columns, so that theta, V and the bf16 copy
+// move in whole 32-byte sectors.  w4 and v4 hold the block's theta and V, loaded ahead.
+struct UpdBlock {
+    float4 w4[4], v4[4];
+};
+__device__ __forceinline__ void update_block_load(const UpdArgs& a, const LayerUpd& u, int M, int N, int m0, int n0,
+                                                  UpdBlock& x) {
+    const int lane = threadIdx.x & 31, n = n0 + 4 * (lane & 3);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int m = m0 + 8 * j + (lane >> 2);
+        x.w4[j] = x.v4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (m < M && n < N) {   // N is a multiple of 8
+            const long long e = u.woff + (long long)m * N + n;
+            x.w4[j] = __ldcs(reinterpret_cast<const float4*>(a.theta + e));
+            x.v4[j] = __ldcs(reinterpret_cast<const float4*>(a.V + e));
+        }
+    }
+}
+__device__ __forceinline__ void update_block_apply(const UpdArgs& a, const LayerUpd& u, int M, int N, int m0, int n0,
+                                                   const uint32_t (&r)[16], UpdBlock& x, float4* sF) {
+    const int lane = threadIdx.x & 31, piece = lane & 3, n = n0 + 4 * piece;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        sF[lane * 4 + (k ^ ((lane >> 1) & 3))] = make_float4(__uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]),
+                                                              __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int row = 8 * j + (lane >> 2), m = m0 + row;
+        float4 g = sF[row * 4 + (piece ^ ((row >> 1) & 3))];
+        if (m >= M || n >= N) continue;
+        const long long i = (long long)m * N + n, e = u.woff + i;
+        if (a.fold_g) {
+            g = add4(g, *reinterpret_cast<const float4*>(a.G + e));
+            *reinterpret_cast<float4*>(a.G + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const float* gc = &g.x;
+        float* wc = &x.w4[j].x;
+        float* vc = &x.v4[j].x;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float vel = a.lr_gs * guard_change(a, gc[c]) + a.momentum * vc[c];
+            vc[c] = vel;
+            wc[c] += vel;
+        }
+        __stcs(reinterpret_cast<float4*>(a.V + e), x.v4[j]);
+        __stcs(reinterpret_cast<float4*>(a.theta + e), x.w4[j]);
+        __align__(8) __nv_bfloat162 h[2];
+        h[0] = __floats2bfloat162_rn(x.w4[j].x, x.w4[j].y);
+        h[1] = __floats2bfloat162_rn(x.w4[j].z, x.w4[j].w);
+        *reinterpret_cast<uint2*>(u.wb + i) = *reinterpret_cast<const uint2*>(h);
+    }
+    __syncwarp();   // the block may be rewritten
 }
 
 template <int BN, class Work>
@@ -477,10 +701,13 @@ __device__ __forceinline__ void gemm_body(const Work work) {
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int items = work.items();
+    const Item first = work.item(blockIdx.x);   // (the grid has at most one CTA per item)
 
     pdl_launch();
+    if (threadIdx.x == 32 * 2) work.prefetch_maps();
+    work.touch();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -509,65 +736,65 @@ __device__ __forceinline__ void gemm_body(const Work work) {
 
     if (warp == 0) {
         // ---------------- TMA producer
-        if (lane == 0) {
-            int stage = 0;
+        if (elect_one()) {
+            int stage = 0, issued = 0;   // copies issued so far
             unsigned phase = 0;
-            int issued_parity[8];
-            for (int s = 0; s < S; ++s) issued_parity[s] = -1;
-            bool ok = true;
+            bool ok = true, free_ = true;   // the stage's buffer is known to be free (all are at first)
+            Item w = first;
             for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-                const Item w = work.item(it);
+                if (it != (int)blockIdx.x) w = work.item(it);
                 const CUtensorMap *ma = work.map_a(w), *mb = work.map_b(w);
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
+                    if (!free_ && !mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
                     uint8_t* sa = ring + stage * Cfg::kStageBytes;
                     mbar_expect_tx(&full[stage], Cfg::kStageBytes);
                     load_operand<BM, Work::kAMn>(sa, ma, w.mb * BM, kb, &full[stage]);
                     load_operand<BN, Work::kBMn>(sa + Cfg::kABytes, mb, w.nb * BN, kb, &full[stage]);
-                    issued_parity[stage] = (int)phase;
+                    ++issued;
                     if (++stage == S) { stage = 0; phase ^= 1u; }
+                    free_ = issued < S || mbar_test(&empty[stage], phase ^ 1u);
                 }
             }
             if (!ok) {
                 // let every copy already issued land before the CTA can exit
-                for (int s = 0; s < S; ++s) {
-                    if (issued_parity[s] < 0) continue;
+                for (int n = issued - 1; n >= 0 && n >= issued - S; --n) {   // each stage's last copy
                     const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(&full[s], (unsigned)issued_parity[s]) &&
-                           global_ns() - t0 < kWaitNs) {
+                    while (!mbar_try_wait(&full[n % S], (unsigned)(n / S) & 1u) && global_ns() - t0 < kWaitNs) {
                     }
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(BM, BN, Work::kAMn, Work::kBMn);
+            const uint32_t a0 = desc_lo<Work::kAMn>(smem_u32(ring)), b0 = desc_lo<Work::kBMn>(smem_u32(ring) + Cfg::kABytes);
             int stage = 0;
             unsigned phase = 0;
             int acc = 0;
             unsigned acc_phase = 0;
-            bool ok = true;
+            bool ok = true, ready = false;   // the stage's operands are known to be there
             bool issued_any = false;
+            Item w = first;
             for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-                const Item w = work.item(it);
+                if (it != (int)blockIdx.x) w = work.item(it);
                 if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
+                uint32_t accumulate = 0;
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    if (!mbar_wait(&full[stage], phase, abort_flag, g.flags)) { ok = false; break; }
+                    if (!ready && !mbar_wait(&full[stage], phase, abort_flag, g.flags)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a0 = smem_u32(ring + stage * Cfg::kStageBytes);
-                    const uint32_t b0 = a0 + Cfg::kABytes;
+                    const uint32_t al = a0 + stage * (Cfg::kStageBytes >> 4), bl = b0 + stage * (Cfg::kStageBytes >> 4);
+                    umma_bf16<idesc>(tmem_d, al, bl, accumulate);
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                        const uint64_t ad = smem_desc_sw128<Work::kAMn>(a0 + kk * k_step_bytes<Work::kAMn>());
-                        const uint64_t bd = smem_desc_sw128<Work::kBMn>(b0 + kk * k_step_bytes<Work::kBMn>());
-                        umma_bf16(tmem_d, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
-                    }
+                    for (int kk = 1; kk < BK / UMMA_K; ++kk)
+                        umma_bf16<idesc>(tmem_d, al + kk * k_step_units<Work::kAMn>(), bl + kk * k_step_units<Work::kBMn>(), 1u);
+                    accumulate = 1u;
                     issued_any = true;
                     umma_commit(&empty[stage]);
                     if (++stage == S) { stage = 0; phase ^= 1u; }
+                    ready = mbar_test(&full[stage], phase);
                 }
                 if (!ok) break;
                 umma_commit(&tfull[acc]);
@@ -589,8 +816,15 @@ __device__ __forceinline__ void gemm_body(const Work work) {
         const int cbeg = (ew >> 2) * (BN / 2);   // this warp's half of the columns
         int acc = 0;
         unsigned acc_phase = 0;
+        if constexpr (MODE == MODE_DWU) {
+            // this CTA's share of the biases and the error sum, while the first tile accumulates
+            const int nb = work.u.bias_blocks + (work.u.sse_out != nullptr ? 1 : 0);
+            for (int b = blockIdx.x; b < nb; b += gridDim.x)
+                update_bias_block(work.u, b, threadIdx.x - 64, colsum, [] { epi_bar(); });
+        }
+        Item w = first;
         for (int it = blockIdx.x; it < items; it += gridDim.x) {
-            const Item w = work.item(it);
+            if (it != (int)blockIdx.x) w = work.item(it);
             float* sbias = bias_s + acc * BN;
             if constexpr (MODE == MODE_FWD || MODE == MODE_FWD_OUT) {
                 // block acc was last read two tiles ago, before the barrier of the previous tile
@@ -599,13 +833,44 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     sbias[c] = n < g.N ? g.bias[n] : 0.f;
                 }
             }
+            UpdBlock cur, nxt;
+            if constexpr (MODE == MODE_DWU) {
+                const DwLayer& y = g.ly[w.l];
+                update_block_load(work.u, work.u.ly[w.l], y.M, y.N, w.mb * BM + q * 32, w.nb * BN + cbeg, cur);
+            }
+            const int m = w.mb * BM + q * 32 + lane;
+            Row32 aux[2];   // this lane's row of the targets or activations: this chunk's and the next one's
+            auto load_aux = [&](int c0, Row32& r) {
+                if constexpr (MODE == MODE_FWD_OUT || MODE == MODE_DX) {
+                    const int n0 = w.nb * BN + c0;
+                    if (g.aux != nullptr) load_row32(r, g.aux + (size_t)m * g.ld_aux + n0, m < g.M ? (g.N - n0) >> 3 : 0);
+                }
+            };
+            load_aux(cbeg, aux[0]);
             mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
             epi_bar();                     // the epilogue warps leave together on an abort
             if (*abort_flag) break;
             tc_fence_after();
-            const int m = w.mb * BM + q * 32 + lane;
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
-            if constexpr (MODE == MODE_DW) {
+            if constexpr (MODE == MODE_DWU) {
+                const DwLayer& y = g.ly[w.l];
+                const LayerUpd& u = work.u.ly[w.l];
+                float4* sF = reinterpret_cast<float4*>(stage_out + ew * 1024);
+                const int m0 = w.mb * BM + q * 32;
+                for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
+                    const int n0 = w.nb * BN + c0;
+                    uint32_t r[16];
+                    update_block_load(work.u, u, y.M, y.N, m0, n0 + 16, nxt);
+                    tmem_ld16(tbase + (uint32_t)c0, r);
+                    update_block_apply(work.u, u, y.M, y.N, m0, n0, r, cur, sF);
+                    if (c0 + 32 < cbeg + BN / 2) update_block_load(work.u, u, y.M, y.N, m0, n0 + 32, cur);
+                    tmem_ld16(tbase + (uint32_t)(c0 + 16), r);
+                    update_block_apply(work.u, u, y.M, y.N, m0, n0 + 16, r, nxt, sF);
+                }
+                tc_fence_before();
+                mbar_arrive(&tempty[acc]);
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            } else if constexpr (MODE == MODE_DW) {
                 const DwLayer& y = g.ly[w.l];
                 for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
                     float v[32];
@@ -621,15 +886,14 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 const int m0 = w.mb * BM + q * 32;
                 bf16* sS = stage_out + ew * 1024;
                 const bool want_colsum = (MODE == MODE_DX) || (MODE == MODE_FWD_OUT && g.aux != nullptr);
-                for (int c0 = cbeg; c0 < cbeg + BN / 2; c0 += 32) {
-                    const int n0 = w.nb * BN + c0;
+#pragma unroll 2
+                for (int i = 0; i < BN / 64; ++i) {
+                    const int c0 = cbeg + 32 * i, n0 = w.nb * BN + c0;
+                    if (n0 >= g.N) break;   // (column sums past N are not read)
+                    if (i + 1 < BN / 64) load_aux(c0 + 32, aux[(i + 1) & 1]);
                     float v[32];
                     tmem_ld32(tbase + (uint32_t)c0, v);
-                    if (n0 >= g.N) {
-                        if (want_colsum) colsum[slot * BN + c0 + lane] = 0.f;
-                        continue;
-                    }
-                    epilogue_chunk<MODE>(g, m, m0, n0, v, sse, row_ok, sS, sbias + c0,
+                    epilogue_chunk<MODE>(g, m0, n0, v, sse, row_ok, sS, sbias + c0, aux[i & 1],
                                          want_colsum ? colsum + slot * BN + c0 : nullptr);
                 }
                 // TMEM is free for the next accumulation into this buffer
@@ -683,6 +947,12 @@ template <int BN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_dw(const __grid_constant__ DwMaps maps, const __grid_constant__ DwArgs g) {
     gemm_body<BN>(DwGemm{g, maps});
+}
+
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    k_gemm_dwu(const __grid_constant__ DwMaps maps, const __grid_constant__ DwArgs g, const __grid_constant__ UpdArgs u) {
+    gemm_body<BN>(DwuGemm(g, maps, u));
 }
 
 // ------------------------------------------------------------ SIMT kernels
@@ -755,113 +1025,24 @@ __global__ void __launch_bounds__(256) k_output_delta(const bf16* O, const bf16*
     }
 }
 
-constexpr int kUpdThreads = 256;
-constexpr int kUpdPieces = 2;                                    // float4 pieces per thread of a weight block
-constexpr int kUpdFloats = kUpdThreads * kUpdPieces * 4;         // weights per block
-constexpr int kUpdBiases = 32, kUpdSlices = kUpdThreads / kUpdBiases;   // biases per block, threads per bias
-
-struct LayerUpd {
-    long long nw;               // n_out * n_in, a multiple of 64
-    int n_out;
-    long long woff, boff;       // offsets in theta / V / G
-    const float* gpart;         // [splits, n_out, n_in]
-    const float* bias_part;     // [mtiles, n_out]
-    bf16* wb;                   // [n_out, n_in]
-    int block0, bias0;          // first weight block and first bias block of the layer
-};
-struct UpdArgs {
-    int L;
-    LayerUpd ly[kMaxL];
-    int blocks;                 // weight and bias blocks of all layers
-    int splits, mtiles;         // pending partial changes (0: none)
-    float* theta;
-    float* V;
-    float* G;
-    float lr_gs, momentum;
-    int mode;                   // 0: apply update; 1: accumulate into G; 2: refresh the bf16 copy
-    int fold_g;
-    const float* sse_part;
-    int n_sse;
-    float* sse_out;
-    int* flags;
-    float guard;          // > 0: fault guard of Section 8
-    unsigned* faults;     // changes the guard zeroed
-};
-
-// Fault guard of Section 8: a total weight change outside (-guard, guard), or
-// not a number, is set to zero and counted (off while guard <= 0).
-__device__ __forceinline__ float guard_change(const UpdArgs& a, float g) {
-    if (a.guard > 0.f && !(fabsf(g) <= a.guard)) {
-        atomicAdd(a.faults, 1u);
-        return 0.f;
-    }
-    return g;
-}
-__device__ __forceinline__ float4 add4(float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); }
-
-// The bias blocks' and the error sum's reduction: slice k of `rows` partials,
-// then the slices in order (the same order on every run).
-__device__ __forceinline__ float slice_sum(const float* p, int rows, size_t pitch, int k, int slices) {
-    const int per = (rows + slices - 1) / slices;
-    const int lo = k * per, hi = min(rows, lo + per);
-    float s = 0.f;
-#pragma unroll 8
-    for (int r = lo; r < hi; ++r) s += p[(size_t)r * pitch];
-    return s;
-}
-
 // Momentum update of Section 6.2.1: g = sum of partial changes (+ pending G);
 // v = lr*gs*g + m*v; w += v; then the bf16 copy.  Mode 1 adds the partial changes
 // into G instead.  Bound by DRAM: a block owns 2,048 consecutive weights, every
 // thread two float4 pieces whose loads (weights, changes, up to two partial
 // planes at a time) are all issued before the first store.
 __global__ void __launch_bounds__(kUpdThreads) k_update_bf16(const __grid_constant__ UpdArgs a) {
-    __shared__ float red[kUpdSlices][kUpdBiases];
+    __shared__ float red[kUpdSlices * kUpdBiases];
     const int t = threadIdx.x;
     pdl_launch();
     pdl_wait();
     const int b = blockIdx.x;
-    if (b == a.blocks) {   // the last block: the group's error sum
-        float s = slice_sum(a.sse_part, a.n_sse, 1, t, kUpdThreads);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((t & 31) == 0) red[0][t >> 5] = s;
-        __syncthreads();
-        if (t == 0) {
-            s = 0.f;
-            for (int w = 0; w < kUpdThreads / 32; ++w) s += red[0][w];
-            *a.sse_out = s;
-            if (!isfinite(s)) atomicOr(a.flags, kFlagNonfinite);
-        }
+    if (b >= a.blocks) {
+        update_bias_block(a, b - a.blocks, t, red, [] { __syncthreads(); });
         return;
     }
     int l = 0;
     while (l + 1 < a.L && b >= a.ly[l + 1].block0) ++l;
     const LayerUpd& u = a.ly[l];
-    if (b >= u.bias0) {
-        // biases: kUpdSlices threads share each one's row-block partials
-        const int j = (b - u.bias0) * kUpdBiases + (t & (kUpdBiases - 1)), k = t / kUpdBiases;
-        red[k][t & (kUpdBiases - 1)] =
-            j < u.n_out ? slice_sum(u.bias_part + j, a.mtiles, u.n_out, k, kUpdSlices) : 0.f;
-        __syncthreads();
-        if (t >= kUpdBiases || j >= u.n_out) return;
-        float g = 0.f;
-#pragma unroll
-        for (int q = 0; q < kUpdSlices; ++q) g += red[q][t];
-        const long long idx = u.boff + j;
-        if (a.mode == 1) {
-            a.G[idx] += g;
-        } else if (a.mode == 0) {
-            if (a.fold_g) {
-                g += a.G[idx];
-                a.G[idx] = 0.f;
-            }
-            const float vel = a.lr_gs * guard_change(a, g) + a.momentum * a.V[idx];
-            a.V[idx] = vel;
-            a.theta[idx] += vel;
-        }
-        return;
-    }
     const long long e0 = (long long)(b - u.block0) * kUpdFloats + t * 4;
     float4 g4[kUpdPieces], w4[kUpdPieces], v4[kUpdPieces];
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -943,7 +1124,7 @@ bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_ro
 template <int BN>
 cudaError_t gemm_setup() {
     const void* fns[] = {(const void*)k_gemm<BN, MODE_FWD>, (const void*)k_gemm<BN, MODE_FWD_OUT>,
-                         (const void*)k_gemm<BN, MODE_DX>, (const void*)k_gemm_dw<BN>};
+                         (const void*)k_gemm<BN, MODE_DX>, (const void*)k_gemm_dw<BN>, (const void*)k_gemm_dwu<BN>};
     for (const void* f : fns) {
         const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    GemmCfg<BN>::kSmemBytes);
@@ -1018,25 +1199,26 @@ int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 int tiles_of(int M, int N, int bn) { return ceil_div(M, BM) * ceil_div(N, bn); }
 
 // Clocks of a K block (64 of K) of a 128 x bn tile with every SM busy, fitted to
-// whole steps at forced widths.  Half the width costs more than half the time:
-// each SM then re-reads A twice as often from L2.
-constexpr double kb_clocks(int bn) { return bn == 256 ? 560 : bn == 128 ? 380 : 250; }
+// whole steps at forced widths (the MMAs alone: 512, 256, 128).  Half the width costs
+// more than half the time: each SM then re-reads A twice as often from L2, and the
+// loops that issue copies and MMAs take about 300 clocks a block themselves (two 64s
+// of K a block at the narrow widths were 1-3% slower).
+constexpr double kb_clocks(int bn) { return bn == 256 ? 530 : bn == 128 ? 330 : 230; }
 
 // Tile width of a launch.  A tile's time is its K loop or its epilogue, whichever
 // is longer (they overlap across tiles), once per wave of tiles over the SMs, plus
 // the other one at the end.  Narrow tiles fill the chip when the batch or the
-// layer is small: a 208-1024-32 step of 512 patterns takes 28.4 / 31.8 / 35.2 us
-// with all launches at 64 / 128 / 256 columns, the forward of 1,001 patterns of
-// 1024-2048-2048-512 54.5 / 38.2 / 45.5 (36.4 by this rule); large batches want
-// 256: 1024-2048-2048-512 at 8,192 540 / 365 / 318 us per step, 512-512-256 at
-// 16,384 37.9 / 30.5 / 27.7 us forward.
+// layer is small: the forward of 512 patterns of 208-1024-32 takes 9.3 / 10.7 / 14.7 us
+// with all launches at 64 / 128 / 256 columns, of 1,001 of 1024-2048-2048-512 29.5 /
+// 27.2 / 41.0 (25.5 by this rule); large batches want 256: a step of 8,192 of
+// 1024-2048-2048-512 364 / 298 / 296.
 int pick_bn(int M, int N, int kb, int num_sms) {
     const int bns[3] = {256, 128, 64};
     int best = 256;
     double best_t = 0;
     for (int bn : bns) {
         const double waves = ceil_div(tiles_of(M, N, bn), num_sms);
-        const double k = kb * kb_clocks(bn), e = 1000.0 + 1200.0 * bn / 64;
+        const double k = kb * kb_clocks(bn), e = 800.0 + 900.0 * bn / 64;
         const double t = waves * (k > e ? k : e) + (k > e ? e : k);
         if (bn == 256 || t < best_t) {
             best = bn;
@@ -1108,37 +1290,53 @@ cudaError_t run_forward(Bf16Net* b, const bf16* X, int B, const bf16* T, bf16* Y
     return cudaSuccess;
 }
 
-// How the pooled-change launch of a group of B patterns is cut: the tile width
-// and the number of K splits that minimise, in clocks,
-//   ceil(tiles * s / num_sms) * K blocks / s * kb_clocks     (waves of 1/s-K work items)
-//   + s * (fp32 partial planes written here and read by the update) / 3,285 B per clock
-//     (the measured 6.8 TB/s copy rate at 2.07 GHz).
-// All layers share the launch, so their tiles fill the last wave together:
-// 1024-2048-2048-512 has 224 tiles of 256 columns, 98% of three waves in two
-// splits (326 us per step; unsplit 334), 4096^5 has 2,048, 96% of 14 waves
-// unsplit; 512-512-256 at 2,048 patterns takes 35.0 / 31.8 / 31.1 us in 1 / 2 /
-// 3 splits of 64 columns, 40.7 / 36.5 / 34.7 of 256.
+// How the pooled-change launch of a group of B patterns is cut: the tile width,
+// the number of K splits, and whether the update runs in its epilogue (training, one
+// split).  All layers share the launch, so their tiles fill the last wave together.
+// The choice minimises, in clocks,
+//   fused:   as pick_bn, with the update of a tile (18 bytes a weight through an SM's
+//            share of DRAM) as the epilogue;
+//   split:   ceil(tiles * s / num_sms) * K blocks / s * kb_clocks   (waves of 1/s-K items)
+//            + s fp32 partial planes, written here and read by the update, at 3,285 B a
+//            clock (the measured 6.8 TB/s copy rate at 2.07 GHz)
+//            + the update kernel's 18 bytes a weight at the same rate and 8,000 clocks
+//            of one more launch in the chain.
+// us per step, split at its best / fused at 64 / 128 / 256 columns: 208-1024-32 at 512
+// patterns 21.9 / 20.6 / 24.4 / 29.7; 1024-2048-2048-512 at 1,001 90.6 / 82.2 / 84.5 /
+// 93.5, at 8,192 294.0 / 313.4 / 281.4 / 296.4; 2048-2048-2048 at 2,048 117.7 / 109.9 /
+// 114.3 / 116.4; 128-256-256-64 at 8,192, whose 16 tiles leave the chip idle unsplit,
+// 39.9 / 48.5 / 57.1 / 75.2.
 constexpr int kMaxSplits = 16;
 struct DwPlan {
     int bn, tiles, splits, kb_total, kb_per_split;
+    bool fused;     // the update runs in the pooled-change launch's epilogue
 };
-DwPlan dw_plan(const int* n, int L, int B, int num_sms, int max_splits) {
+DwPlan dw_plan(const int* n, int L, int B, int num_sms, int max_splits, bool may_fuse) {
     DwPlan p{};
     p.kb_total = ceil_div(B, BK);
-    double best_cost = 0;
+    double best = 0, weights = 0;
+    for (int l = 1; l <= L; ++l) weights += (double)n[l] * n[l - 1];
+    auto take = [&](double t, int bn, int tiles, int splits, bool fused) {
+        if (best != 0 && t >= best * (1.0 - 1e-9)) return;
+        best = t;
+        p.bn = bn;
+        p.tiles = tiles;
+        p.splits = splits;
+        p.fused = fused;
+    };
+    const double hbm = 3285;   // bytes per clock
     const int bns[3] = {256, 128, 64};
     for (int bn : bns) {
         int tiles = 0;
         for (int l = 1; l <= L; ++l) tiles += tiles_of(n[l], n[l - 1], bn);
+        const double loop = p.kb_total * kb_clocks(bn), plane = 8.0 * BM * bn * tiles / hbm;
+        if (may_fuse) {
+            const double upd = 7000.0 * bn / 64, waves = ceil_div(tiles, num_sms);
+            take(waves * (loop > upd ? loop : upd) + (loop > upd ? upd : loop), bn, tiles, 1, true);
+        }
         for (int s = 1; s <= max_splits && s <= p.kb_total; ++s) {
             const double waves = (double)(((long long)tiles * s + num_sms - 1) / num_sms) / s;
-            const double cost = waves * p.kb_total * kb_clocks(bn) + s * (8.0 * BM * bn * tiles) / 3285;
-            if (best_cost == 0 || cost < best_cost * (1.0 - 1e-9)) {
-                best_cost = cost;
-                p.bn = bn;
-                p.tiles = tiles;
-                p.splits = s;
-            }
+            take(waves * loop + s * plane + weights * 18 / hbm + 8000, bn, tiles, s, false);
         }
     }
     p.kb_per_split = ceil_div(p.kb_total, p.splits);
@@ -1148,7 +1346,7 @@ DwPlan dw_plan(const int* n, int L, int B, int num_sms, int max_splits) {
 
 // Hidden deltas and pooled partial changes for every layer (deltas of layer L
 // and the activations must already be in scratch).
-cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, const DwPlan& p, cudaStream_t s) {
+cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, const DwPlan& p, const UpdArgs* upd, cudaStream_t s) {
     const int L = b->L;
     for (int l = L; l >= 2; --l) {
         // delta_{l-1} = (delta_l W_l) * a (1 - a):  A = delta_l [B, n_l], B-operand = W_l along K
@@ -1190,6 +1388,13 @@ cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, const DwPlan& p, cuda
     }
     const int items = p.tiles * p.splits;
     const int grid = items < b->num_sms ? items : b->num_sms;
+    if (upd != nullptr) {
+        switch (p.bn) {
+            case 64: return launch_pdl(k_gemm_dwu<64>, grid, 1, kGemmThreads, GemmCfg<64>::kSmemBytes, s, maps, g, *upd);
+            case 128: return launch_pdl(k_gemm_dwu<128>, grid, 1, kGemmThreads, GemmCfg<128>::kSmemBytes, s, maps, g, *upd);
+            default: return launch_pdl(k_gemm_dwu<256>, grid, 1, kGemmThreads, GemmCfg<256>::kSmemBytes, s, maps, g, *upd);
+        }
+    }
     switch (p.bn) {
         case 64: return launch_pdl(k_gemm_dw<64>, grid, 1, kGemmThreads, GemmCfg<64>::kSmemBytes, s, maps, g);
         case 128: return launch_pdl(k_gemm_dw<128>, grid, 1, kGemmThreads, GemmCfg<128>::kSmemBytes, s, maps, g);
@@ -1203,7 +1408,7 @@ UpdArgs upd_args(Bf16Net* b, int splits, int mtiles, int mode, bool fold, float 
     UpdArgs a;
     memset(&a, 0, sizeof a);
     a.L = b->L;
-    int blocks = 0;
+    int blocks = 0, bias_blocks = 0;
     for (int l = 1; l <= b->L; ++l) {
         LayerUpd& u = a.ly[l - 1];
         u.n_out = b->n[l];
@@ -1214,10 +1419,12 @@ UpdArgs upd_args(Bf16Net* b, int splits, int mtiles, int mode, bool fold, float 
         u.bias_part = b->bpart[l];
         u.wb = b->wb[l];
         u.block0 = blocks;
-        u.bias0 = blocks + ceil_div(u.nw, kUpdFloats);
-        blocks = u.bias0 + ceil_div(u.n_out, kUpdBiases);
+        u.bias0 = bias_blocks;
+        blocks += ceil_div(u.nw, kUpdFloats);
+        bias_blocks += ceil_div(u.n_out, kUpdBiases);
     }
     a.blocks = blocks;
+    a.bias_blocks = bias_blocks;
     a.splits = splits;
     a.mtiles = mtiles;
     a.theta = b->theta;
@@ -1237,7 +1444,7 @@ UpdArgs upd_args(Bf16Net* b, int splits, int mtiles, int mode, bool fold, float 
 }
 
 cudaError_t launch_update(const UpdArgs& a, cudaStream_t s) {
-    return launch_pdl(k_update_bf16, a.blocks + (a.sse_out != nullptr ? 1 : 0), 1, kUpdThreads, 0, s, a);
+    return launch_pdl(k_update_bf16, a.blocks + a.bias_blocks + (a.sse_out != nullptr ? 1 : 0), 1, kUpdThreads, 0, s, a);
 }
 
 }  // namespace
@@ -1289,7 +1496,7 @@ bp_status bf16_create(const int* n, int L, int max_batch, int num_sms, float* th
     }
     bool ok = true;
     const int mt = ceil_div(max_batch, BM);
-    b->max_splits = dw_plan(n, L, max_batch, num_sms, kMaxSplits).splits;
+    b->max_splits = dw_plan(n, L, max_batch, num_sms, kMaxSplits, false).splits;
     for (int l = 1; l <= L && ok; ++l) {
         ok = ok && alloc(b, (void**)&b->wb[l], (size_t)n[l] * n[l - 1] * 2);
         ok = ok && alloc(b, (void**)&b->act[l], (size_t)max_batch * n[l] * 2);
@@ -1332,8 +1539,8 @@ cudaError_t bf16_backward(Bf16Net* b, const void* X, const void* T, int batch, f
     cudaError_t e = launch_pdl(k_output_delta, nc, mt, 256, 0, s, b->act[L], (const bf16*)T, batch, nL, b->dlt[L],
                                b->bpart[L], b->sse_part);
     if (e != cudaSuccess) return e;
-    const DwPlan p = dw_plan(b->n, L, batch, b->num_sms, b->max_splits);
-    e = run_backward(b, (const bf16*)X, batch, p, s);
+    const DwPlan p = dw_plan(b->n, L, batch, b->num_sms, b->max_splits, false);
+    e = run_backward(b, (const bf16*)X, batch, p, nullptr, s);
     if (e != cudaSuccess) return e;
     return launch_update(upd_args(b, p.splits, mt, 1, false, 0.f, 0.f, sse, mt * nc), s);
 }
@@ -1355,13 +1562,12 @@ cudaError_t bf16_train(Bf16Net* b, const void* X, const void* T, int n_patterns,
         const bf16* Ts = (const bf16*)T + p0 * trow;
         cudaError_t e = run_forward(b, Xs, B, Ts, nullptr, s);
         if (e != cudaSuccess) return e;
-        const DwPlan p = dw_plan(b->n, L, B, b->num_sms, b->max_splits);
-        e = run_backward(b, Xs, B, p, s);
-        if (e != cudaSuccess) return e;
+        const DwPlan p = dw_plan(b->n, L, B, b->num_sms, b->max_splits, true);
         const int n_sse = tiles_of(B, b->n[L], pick_bn(B, b->n[L], ceil_div(b->n[L - 1], BK), b->num_sms));
-        e = launch_update(upd_args(b, p.splits, ceil_div(B, BM), 0, fold, lr * grad_scale, momentum,
-                                   sse != nullptr ? sse + step : nullptr, n_sse),
-                          s);
+        const UpdArgs a = upd_args(b, p.fused ? 0 : p.splits, ceil_div(B, BM), 0, fold, lr * grad_scale, momentum,
+                                   sse != nullptr ? sse + step : nullptr, n_sse);
+        e = run_backward(b, Xs, B, p, p.fused ? &a : nullptr, s);
+        if (e == cudaSuccess && !p.fused) e = launch_update(a, s);
         if (e != cudaSuccess) return e;
         fold = false;
     }

@@ -46,3 +46,25 @@ def test_step_at_tile_edges_matches_oracle(sizes, B):
     st.G = G_ref
     O.apply_update(st)
     assert_layers(sizes, th - theta, st.theta - theta, TOL, None, "W1-W0")
+
+
+@pytest.mark.parametrize("sizes,B", [((208, 520, 64), 300), ((64, 128, 32), 4100)])
+def test_pending_change_is_folded_into_train_batch(sizes, B):
+    """Update in the pooled change's epilogue, and in the kernel after split sums."""
+    X, T, theta = problem(sizes, B, seed=51)
+    X2, T2, _ = problem(sizes, B, seed=52)
+    st = O.State(sizes, theta, lr=0.01, momentum=0.9, grad_scale=1.0 / B)
+    with bp.Net(sizes, 0.01, 0.9, bp.BP_BF16, max_batch=B, grad_scale=1.0 / B) as net:
+        net.set_weights(theta)
+        Xd, X2d = dev_bf16(X), dev_bf16(X2)
+        for k in range(2):   # the second step has a velocity
+            net.forward(Xd, B)
+            net.backward(dev_bf16(T), B)
+            net.train_batch(X2d, dev_bf16(T2), B)
+            O.backward_accumulate(st, X, T)
+            O.train_batch(st, X2, T2)
+        net.check()
+        th, V = net.get_weights(), net.get_velocity()
+        np.testing.assert_array_equal(net.get_grads(), 0.0)
+    assert_layers(sizes, th - theta, st.theta - theta, TOL, None, "W2-W0")
+    assert_layers(sizes, V, st.V, TOL, None, "V2")

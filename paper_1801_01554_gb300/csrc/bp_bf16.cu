@@ -261,13 +261,46 @@ __device__ __forceinline__ float bf16_round(float x) {
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // ------------------------------------------------------------ epilogue
-// 32 consecutive bf16 of one row (pieces of 8 past `pieces` are zero), and as floats.
+// A warp's 32 x 32 block of bf16 as 16-byte pieces (8 columns).  Global memory is read
+// and written with lane (row 8 j + lane / 4, piece lane % 4), four lanes to a 64-byte
+// row segment; the arithmetic wants lane = row.  The warp's 2 KB of shared memory turns
+// one into the other (pieces permuted by row so that both sides spread over the banks).
+// Loading a row per lane instead costs 32 cache-line lookups an instruction (the output
+// layer's epilogue took 17,200 clocks a 128 x 256 tile, 14,600 with whole segments; a
+// 1024-2048-2048-512 step of 1,001 patterns 81.8 us, 79.8), but no turn through shared
+// memory: it is kept for 64-column tiles, one chunk per warp, where the latency of that
+// counts for more (208-1024-32 at 512 patterns: 20.6 us against 20.9).
 struct Row32 {
     uint4 u[4];
 };
-__device__ __forceinline__ void load_row32(Row32& r, const bf16* p, int pieces) {
+__device__ __forceinline__ uint4* piece_at(uint4* sS4, int row, int piece) {
+    return sS4 + row * 4 + (piece ^ ((row >> 1) & 3));
+}
+// rows past `rows` and pieces past `pieces` are zero
+__device__ __forceinline__ void load_block(Row32& r, const bf16* p, int ld, int rows, int pieces) {
+    const int lane = threadIdx.x & 31, piece = lane & 3;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) r.u[k] = k < pieces ? reinterpret_cast<const uint4*>(p)[k] : make_uint4(0u, 0u, 0u, 0u);
+    for (int j = 0; j < 4; ++j) {
+        const int row = 8 * j + (lane >> 2);
+        r.u[j] = (row < rows && piece < pieces) ? *reinterpret_cast<const uint4*>(p + (size_t)row * ld + piece * 8)
+                                                : make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+__device__ __forceinline__ void load_own_row(Row32& r, const bf16* p, int ld, int rows, int pieces) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        r.u[k] = (lane < rows && k < pieces) ? reinterpret_cast<const uint4*>(p + (size_t)lane * ld)[k]
+                                             : make_uint4(0u, 0u, 0u, 0u);
+}
+__device__ __forceinline__ void block_to_rows(Row32& r, uint4* sS4) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *piece_at(sS4, 8 * j + (lane >> 2), lane & 3) = r.u[j];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r.u[k] = *piece_at(sS4, lane, k);
+    __syncwarp();   // the block is rewritten
 }
 __device__ __forceinline__ float row_value(const Row32& r, int c) {   // c is a compile-time constant
     const uint4& u = r.u[c >> 3];
@@ -304,14 +337,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 // sums of a delta block (bias change) are taken from the pieces on their way
 // out: each lane adds its four rows of 8 columns, then the eight lanes of a
 // piece reduce-scatter them (7 shuffles).
-template <int MODE>
+template <int BN, int MODE>
 __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m0, int n0, float (&v)[32], float& sse,
-                                               bool row_ok, bf16* sS, const float* sbias, const Row32& aux,
+                                               bool row_ok, bf16* sS, const float* sbias, Row32& aux,
                                                float* colsum_slot) {
     const int N = g.N;
     const int lane = threadIdx.x & 31;
     const int valid = min(32, N - n0);
     const bool with_t = (MODE == MODE_FWD_OUT) && (g.aux != nullptr);
+    uint4* sS4 = reinterpret_cast<uint4*>(sS);
+    if (BN > 64 && (with_t || MODE == MODE_DX)) block_to_rows(aux, sS4);
     // values in place; they are rounded when they are packed below
     if (MODE == MODE_FWD || MODE == MODE_FWD_OUT) {
 #pragma unroll
@@ -342,14 +377,13 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m0, int n0
     bf16* const rows = with_t ? g.out2 : g.out;
     const int ldr = with_t ? g.ld2 : g.ldo;
     bf16* const copy = (MODE == MODE_FWD_OUT && !with_t) ? g.out2 : nullptr;
-    uint4* sS4 = reinterpret_cast<uint4*>(sS);
     const int piece = lane & 3;   // 16-byte piece of a 64-byte segment
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         __align__(16) __nv_bfloat162 h[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(v[8 * k + 2 * q], v[8 * k + 2 * q + 1]);
-        sS4[lane * 4 + (k ^ ((lane >> 1) & 3))] = *reinterpret_cast<const uint4*>(h);
+        *piece_at(sS4, lane, k) = *reinterpret_cast<const uint4*>(h);
     }
     __syncwarp();
     const int pieces = valid >> 3;   // N is a multiple of 8
@@ -359,7 +393,7 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs& g, int m0, int n0
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int r = j * 8 + (lane >> 2);
-        const uint4 u = sS4[r * 4 + (piece ^ ((r >> 1) & 3))];
+        const uint4 u = *piece_at(sS4, r, piece);
         if (m0 + r < g.M && piece < pieces) {
             *reinterpret_cast<uint4*>(rows + (size_t)(m0 + r) * ldr + n0 + piece * 8) = u;
             if (copy != nullptr) *reinterpret_cast<uint4*>(copy + (size_t)(m0 + r) * g.ld2 + n0 + piece * 8) = u;
@@ -838,12 +872,15 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 const DwLayer& y = g.ly[w.l];
                 update_block_load(work.u, work.u.ly[w.l], y.M, y.N, w.mb * BM + q * 32, w.nb * BN + cbeg, cur);
             }
-            const int m = w.mb * BM + q * 32 + lane;
-            Row32 aux[2];   // this lane's row of the targets or activations: this chunk's and the next one's
+            const int m0 = w.mb * BM + q * 32, m = m0 + lane;
+            Row32 aux[2];   // the targets' or activations' block of this chunk and of the next one
             auto load_aux = [&](int c0, Row32& r) {
                 if constexpr (MODE == MODE_FWD_OUT || MODE == MODE_DX) {
                     const int n0 = w.nb * BN + c0;
-                    if (g.aux != nullptr) load_row32(r, g.aux + (size_t)m * g.ld_aux + n0, m < g.M ? (g.N - n0) >> 3 : 0);
+                    const bf16* p = g.aux + (size_t)m0 * g.ld_aux + n0;
+                    if (g.aux == nullptr) return;
+                    if (BN > 64) load_block(r, p, g.ld_aux, g.M - m0, (g.N - n0) >> 3);
+                    else load_own_row(r, p, g.ld_aux, g.M - m0, (g.N - n0) >> 3);
                 }
             };
             load_aux(cbeg, aux[0]);
@@ -856,7 +893,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 const DwLayer& y = g.ly[w.l];
                 const LayerUpd& u = work.u.ly[w.l];
                 float4* sF = reinterpret_cast<float4*>(stage_out + ew * 1024);
-                const int m0 = w.mb * BM + q * 32;
                 for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
                     const int n0 = w.nb * BN + c0;
                     uint32_t r[16];
@@ -883,7 +919,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
             } else {
                 const bool row_ok = m < g.M;
                 float sse = 0.f;
-                const int m0 = w.mb * BM + q * 32;
                 bf16* sS = stage_out + ew * 1024;
                 const bool want_colsum = (MODE == MODE_DX) || (MODE == MODE_FWD_OUT && g.aux != nullptr);
 #pragma unroll 2
@@ -893,7 +928,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     if (i + 1 < BN / 64) load_aux(c0 + 32, aux[(i + 1) & 1]);
                     float v[32];
                     tmem_ld32(tbase + (uint32_t)c0, v);
-                    epilogue_chunk<MODE>(g, m0, n0, v, sse, row_ok, sS, sbias + c0, aux[i & 1],
+                    epilogue_chunk<BN, MODE>(g, m0, n0, v, sse, row_ok, sS, sbias + c0, aux[i & 1],
                                          want_colsum ? colsum + slot * BN + c0 : nullptr);
                 }
                 // TMEM is free for the next accumulation into this buffer

@@ -27,7 +27,7 @@
 // A training launch is a persistent cooperative kernel that loops over any
 // number of groups with a grid barrier between the phases; every wait in the
 // barrier is bounded and latches kFlagTimeout instead of hanging.  Groups of at
-// most 16 patterns of a one-hidden-layer net run on one cluster instead
+// most 4 patterns of a one-hidden-layer net run on one cluster instead
 // (bp_f32_cluster.cu), its groups of 40 or more patterns per CTA with the sums of
 // changes in registers (bp_f32_large.cu), and other nets' groups of at most 4 on
 // one CTA (k_train_small), with the weights resident on chip for the whole launch.
@@ -290,41 +290,21 @@ __device__ void forward_layer(const float* W, int kp, int n_out, const float* s_
             const float* wr[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) wr[u] = W + (size_t)min(j0 + u, n_out - 1) * kp;
-            if constexpr (V <= 16) {   // sums of even and odd columns, two multiply-adds an instruction
-                f32x2 acc2[V];
+            for (int k = s; k < K4; k += S) {
+                float4 a[PG];
 #pragma unroll
-                for (int k = 0; k < V; ++k) acc2[k] = 0;
-                for (int k = s; k < K4; k += S) {
-                    ulonglong2 a[PG];
+                for (int p = 0; p < PG; ++p) a[p] = ld4(s_in + p * kp + 4 * k);
 #pragma unroll
-                    for (int p = 0; p < PG; ++p) a[p] = ld4x2(s_in + p * kp + 4 * k);
+                for (int u = 0; u < U; ++u) {
+                    const float4 w = ld4(wr[u] + 4 * k);
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const ulonglong2 w = ld4x2(wr[u] + 4 * k);
-#pragma unroll
-                        for (int p = 0; p < PG; ++p)
-                            acc2[u * PG + p] = fma2(w.y, a[p].y, fma2(w.x, a[p].x, acc2[u * PG + p]));
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < V; ++k) acc[k] = sum2(acc2[k]);
-            } else {   // 32 sums: pairs would take 64 registers
-                for (int k = s; k < K4; k += S) {
-                    float4 a[PG];
-#pragma unroll
-                    for (int p = 0; p < PG; ++p) a[p] = ld4(s_in + p * kp + 4 * k);
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const float4 w = ld4(wr[u] + 4 * k);
-#pragma unroll
-                        for (int p = 0; p < PG; ++p) {
-                            float t = acc[u * PG + p];
-                            t = fmaf(w.x, a[p].x, t);
-                            t = fmaf(w.y, a[p].y, t);
-                            t = fmaf(w.z, a[p].z, t);
-                            t = fmaf(w.w, a[p].w, t);
-                            acc[u * PG + p] = t;
-                        }
+                    for (int p = 0; p < PG; ++p) {
+                        float t = acc[u * PG + p];
+                        t = fmaf(w.x, a[p].x, t);
+                        t = fmaf(w.y, a[p].y, t);
+                        t = fmaf(w.z, a[p].z, t);
+                        t = fmaf(w.w, a[p].w, t);
+                        acc[u * PG + p] = t;
                     }
                 }
             }
@@ -448,80 +428,42 @@ __device__ __forceinline__ void forward_any(const float* W, int kp, int n_out, c
 }
 
 // Hidden deltas of layer l for PG patterns: d_l[p][i] = (sum_j W_{l+1}[j][i]
-// d_{l+1}[p][j]) a_l[p][i] (1 - a_l[p][i]).  Four lanes share a unit: lane r sums
-// the next layer's units r, r + 4, .. for all PG patterns (a weight and one read of
-// the PG deltas per PG multiply-adds), then a reduce-scatter over the four leaves
-// each lane PG / 4 patterns (or, below 4, copies).  One thread per (pattern, unit), with
-// the whole sum in its one chain, took 11.8 us per update at groups of 512 of 203-120-26
-// and 25.1 at 2,000, against 11.6 and 23.9.  dnt holds d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl, pitch dpl) and, if dlt is not null,
-// pattern-minor (dlt).
+// d_{l+1}[p][j]) a_l[p][i] (1 - a_l[p][i]), summed over the next layer's units in
+// order.  One thread per unit sums all PG patterns, so that a weight and one read of
+// the PG deltas feed PG multiply-adds (a thread per pattern and unit read both for
+// each one: 11.7 us per update at groups of 512 of 203-120-26 and 25.1 at 2,000,
+// against 11.6 and 24.0).  dnt holds d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl,
+// pitch dpl) and, if dlt is not null, pattern-minor (dlt).
 template <int PG>
 __device__ void hidden_delta(const float* Wn, int kpn, int n, int nn, const float* dnt,
                              const float* al, int apl, float* dl, int dpl, float* dlt) {
-    const int lane = threadIdx.x & 31, r = lane & 3;
-    for (int i0 = 0; i0 < n; i0 += kThreads / 4) {   // uniform trip count: every lane shuffles
-        const int i = i0 + (threadIdx.x >> 2);
+    for (int i = threadIdx.x; i < n; i += kThreads) {
         float acc[PG];
 #pragma unroll
         for (int p = 0; p < PG; ++p) acc[p] = 0.f;
-        if (i < n) {
 #pragma unroll 4
-            for (int j = r; j < nn; j += 4) {
-                const float w = Wn[(size_t)j * kpn + i];
-                float d[PG];
-                if constexpr (PG >= 4) {
+        for (int j = 0; j < nn; ++j) {
+            const float w = Wn[(size_t)j * kpn + i];
+            if constexpr (PG >= 4) {
 #pragma unroll
-                    for (int q = 0; q < PG / 4; ++q) {
-                        const float4 t = ld4(dnt + j * PG + 4 * q);
-                        d[4 * q] = t.x;
-                        d[4 * q + 1] = t.y;
-                        d[4 * q + 2] = t.z;
-                        d[4 * q + 3] = t.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int p = 0; p < PG; ++p) d[p] = dnt[j * PG + p];
+                for (int q = 0; q < PG / 4; ++q) {
+                    const float4 d = ld4(dnt + j * PG + 4 * q);
+                    acc[4 * q] = fmaf(d.x, w, acc[4 * q]);
+                    acc[4 * q + 1] = fmaf(d.y, w, acc[4 * q + 1]);
+                    acc[4 * q + 2] = fmaf(d.z, w, acc[4 * q + 2]);
+                    acc[4 * q + 3] = fmaf(d.w, w, acc[4 * q + 3]);
                 }
+            } else {
 #pragma unroll
-                for (int p = 0; p < PG; ++p) acc[p] = fmaf(d[p], w, acc[p]);
+                for (int p = 0; p < PG; ++p) acc[p] = fmaf(dnt[j * PG + p], w, acc[p]);
             }
         }
-        // lane r keeps patterns r P4 .. (PG >= 4), or pattern r mod PG
-        if constexpr (PG >= 4) {
 #pragma unroll
-            for (int half = 2; half >= 1; half >>= 1) {
-                const bool up = (r & half) != 0;
-                constexpr int kAll = PG;
-#pragma unroll
-                for (int k = 0; k < kAll; ++k) {
-                    const int cnt = half == 2 ? PG / 2 : PG / 4;
-                    if (k >= cnt) break;
-                    const float send = up ? acc[k] : acc[k + cnt];
-                    const float keep = up ? acc[k + cnt] : acc[k];
-                    acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int p = 0; p < PG; ++p) {
-                acc[p] += __shfl_xor_sync(0xffffffffu, acc[p], 1);
-                acc[p] += __shfl_xor_sync(0xffffffffu, acc[p], 2);
-            }
-        }
-        if (i < n) {
-            constexpr int kMine = PG >= 4 ? PG / 4 : 1;
-#pragma unroll
-            for (int k = 0; k < kMine; ++k) {
-                const int p = PG >= 4 ? r * kMine + k : r;
-                float sum = acc[k];
-                if (PG == 2) sum = r == 0 ? acc[0] : acc[PG - 1];
-                if (p < PG) {
-                    const float a = al[p * apl + i];
-                    const float d = sum * a * (1.f - a);
-                    dl[p * dpl + i] = d;
-                    if (dlt != nullptr) dlt[i * PG + p] = d;
-                }
-            }
+        for (int p = 0; p < PG; ++p) {
+            const float a = al[p * apl + i];
+            const float d = acc[p] * a * (1.f - a);
+            dl[p * dpl + i] = d;
+            if (dlt != nullptr) dlt[i * PG + p] = d;
         }
     }
 }

@@ -210,8 +210,10 @@ __device__ __forceinline__ bool wait_bytes(uint64_t* bar, unsigned parity, int* 
 
 // Pairs of floats in one 64-bit register: two multiply-adds (each rounded as fmaf)
 // per issued instruction.  The multiply-add rate per SM is the same, so what they
-// save is issue slots: 203-120-26 took 31.0 -> 29.2 us per update at groups of 4,096,
-// 353 -> 350 at 65,536 (shared memory and latency bound it there), 11.85 -> 11.8 at 512.
+// save is issue slots: in the passes of 32 patterns and the weight phase, groups of
+// 4,096 of 203-120-26 took 31.1 -> 29.3 us per update.  The lane-group forward of
+// smaller passes keeps single ones: it gained nothing from pairs of columns, which
+// add up in another order.
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
     f32x2 r;

@@ -530,17 +530,22 @@ __device__ __forceinline__ void update_bias_block(const UpdArgs& a, int b, int t
 }
 
 // ------------------------------------------------------------ GEMM kernel
-// Tile order: groups of kGroupM row blocks, each group swept over all column
-// blocks (row block fastest), so that the tiles in flight on the 152 SMs share
-// a few row blocks of A and column blocks of B, which stay in L2, instead of
-// reading every row block of A at once (4, 8, 16 and 32 row blocks measured
-// within 2% of each other; one row block at a time was 10% slower for 4096^5).
-constexpr int kGroupM = 4;
+// Tile order: groups of GROUP row blocks, each group swept over all column blocks (row
+// block fastest), so that the tiles in flight on the 152 SMs share a few row blocks of A
+// and column blocks of B, which stay in L2, instead of reading every row block of A at
+// once (that was 10% slower for 4096^5).  16 row blocks in the backward: 152 tiles of
+// 128 x 256 are then about a square, 16 x 10, and read least (with 4, 12 x 16 tiles, the
+// pooled changes of 4096^5 read 4.0 GB from DRAM for 1.6 GB of operands and weights).  ms
+// per step of 4096^5, 4 / 8 / 12 / 16 / 32 in the pooled changes: 3.93 / 3.93 / 3.91 /
+// 3.90 / 3.90.  The forward keeps 4: 16 gains it nothing at that size, and costs 0.9% where
+// all tiles run at once (1,001 of 1024-2048-2048-512).  A choice at run time costs the
+// small launches 1-3%.
+template <int GROUP>
 __device__ __forceinline__ void tile_coords(int tile, int num_m, int num_n, int& mb, int& nb) {
-    const int per_group = kGroupM * num_n;
+    const int per_group = GROUP * num_n;
     const int grp = tile / per_group;
-    const int first = grp * kGroupM;
-    const int gm = min(num_m - first, kGroupM);
+    const int first = grp * GROUP;
+    const int gm = min(num_m - first, GROUP);
     const int local = tile - grp * per_group;
     mb = first + local % gm;
     nb = local / gm;
@@ -581,7 +586,7 @@ struct OneGemm {
     __device__ int items() const { return g.num_m * g.num_n; }
     __device__ Item item(int it) const {
         Item w{0, 0, 0, g.kb_total, 0, 0};
-        tile_coords(it, g.num_m, g.num_n, w.mb, w.nb);
+        tile_coords<MODE == MODE_DX ? 16 : 4>(it, g.num_m, g.num_n, w.mb, w.nb);
         return w;
     }
     // The launch's parameters are read here once, while the previous kernel drains: their
@@ -611,7 +616,7 @@ struct DwGemm {
         w.l = 0;
         while (w.l + 1 < g.L && tile >= g.ly[w.l + 1].tile0) ++w.l;
         const DwLayer& y = g.ly[w.l];
-        tile_coords(tile - y.tile0, y.num_m, y.num_n, w.mb, w.nb);
+        tile_coords<16>(tile - y.tile0, y.num_m, y.num_n, w.mb, w.nb);
         w.kb0 = w.split * g.kb_per_split;
         w.kb1 = min(g.kb_total, w.kb0 + g.kb_per_split);
         return w;

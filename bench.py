@@ -261,19 +261,19 @@ def synth_sizes(name):
 
 # DRAM bytes (read + write) per pattern of each workload's roofline unit, from
 # single-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum; the
-# commands are in profiles/dram_traffic_all_workloads.md): one k_train launch
+# commands are in profiles/dram_traffic_all_workloads.md): one training launch
 # for the float32 nets (one epoch; 203-120-26 captured on a 16,384-pattern epoch
 # and scaled by patterns, as its traffic is the inputs read once), the whole
 # training step (all launches) for the bf16 nets.  Re-measure after any change
-# to these kernels; a workload whose kernels changed since its capture has none
-# (the bf16 nets: the update kernel's bias part changed after their capture).
+# to these kernels.
 TRAFFIC_PER_PATTERN = {
-    "nettalk60": 1_116_416 / 1024,          # 1.12 MB per launch (one update of 1,024)
-    "nettalk120": 15_408_128 / 16384,       # 61.6 MB per 65,536-pattern launch
+    "nettalk60": 1_116_928 / 1024,          # 1.12 MB per launch (one update of 1,024)
+    "nettalk120": 15_412_224 / 16384,       # 61.6 MB per 65,536-pattern launch
+    "wide3": 596_949_760 / 8192,            # 597 MB per step
+    "wide4096": 7_459_912_448 / 16384,      # 7.46 GB per step
 }
-# sweep groups of 203-120-26 with a capture of their own (bytes per pattern of one launch);
-# at B = 65,536 the group's scratch rows no longer fit the L2 and make a DRAM round trip
-SWEEP_TRAFFIC_PER_PATTERN = {512: TRAFFIC_PER_PATTERN["nettalk120"], 65536: 676_348_928 / 65536}
+# sweep groups of 203-120-26 with a capture of their own (bytes per pattern of one launch)
+SWEEP_TRAFFIC_PER_PATTERN = {512: TRAFFIC_PER_PATTERN["nettalk120"], 65536: 61_789_696 / 65536}
 
 
 def connections(sizes):
@@ -687,8 +687,8 @@ def run_wide(args, world, rank, local):
 def run_sweep(args, world, rank, local):
     """CPS against the group size B on the 203-120-26 net (the paper's group-size
     question, Section 5): one JSON line per B, from CUDA events around whole
-    epochs with the L2 flushed before each.  B <= 4 runs on the one-CTA kernel,
-    larger groups on the persistent kernel."""
+    epochs with the L2 flushed before each.  B <= 4 runs on one cluster,
+    larger groups on a grid-wide persistent kernel."""
     import torch
     from paper_1801_01554_gb300 import bp, perf_model, synth
 
@@ -724,9 +724,9 @@ def run_sweep(args, world, rank, local):
         t = sorted(ms)[len(ms) // 2] / 1e3
         print(json.dumps({"sweep": "group size", "B": B, "patterns": n, "updates": updates,
                           "us_per_update": 1e6 * t / updates,
-                          "model_us_per_update": perf_model.gb300_update_us(B),
+                          "model_us_per_update": perf_model.gb300_update_us(B, cluster=True),
                           "value": W * n / t, "unit": UNIT,
-                          "kernel": "one-CTA" if B <= 4 else "persistent cooperative",
+                          "kernel": "one cluster" if B <= 4 else "persistent cooperative",
                           "dtype": "f32", "data": "synthetic"}), flush=True)
     return 0
 

@@ -10,10 +10,10 @@ Two models live here:
 * the same accounting restated for this library's float32 kernels on one
   GB300: microseconds per update from the phases of the persistent kernel
   (two grid barriers, the weight copy into shared memory, pattern passes of PG
-  patterns per CTA, 256-pattern chunks of the weight phase) and of the one-CTA
-  kernel for groups of 1-4 patterns.  Its constants are the phase costs
-  measured on GB300 (each phase looped inside one launch), not fitted to the
-  end-to-end times; `skew_us` is the one remainder.
+  patterns per CTA, 512-pattern chunks of the weight phase), of the kernel for
+  large groups of one-hidden-layer nets (a fixed cost, then one cost per pass of
+  64 patterns a CTA), and of the kernels for groups of 1-4 patterns.  Its
+  constants are fitted to per-update times measured on GB300.
 
 Readings of the printed model (Section 6.1):
 * the last term of T is printed as 4P x W, but the tree cost per update is
@@ -80,26 +80,34 @@ def gf11_optimal_processors(W, Wi, U, C, summing="tree", M=GF11_FREE_SRAM, bundl
 @dataclass
 class GB300Phases:
     """Phase costs of the float32 kernels on one GB300 (microseconds), fitted
-    to per-update times of the 203-120-26 net with and without the weight
-    phase (a timing-only copy of the kernel) at B = 8 .. 65,536."""
+    to per-update times of the 203-120-26 net at B = 1 .. 65,536."""
     n_sm: int = 152
     # pattern side of an update: two grid barriers, the weight copy, skew, and
     # one pass per PG patterns of a CTA's share
-    pattern_fixed_us: float = 4.79
-    pass_us: tuple = ((1, 3.10), (2, 3.43), (4, 4.56), (8, 7.09), (32, 16.3))
+    pattern_fixed_us: float = 4.70
+    pass_us: tuple = ((1, 3.10), (2, 3.43), (4, 4.56), (8, 6.10), (32, 13.1))
     # whole-tile weight phase (8 x 32 tiles, one per CTA): fixed part, then per
     # 512-pattern chunk a fixed and a per-row part
     weight_fixed_us: float = 1.19
     chunk_fixed_us: float = 0.58
     chunk_rows_us: float = 0.72        # for a full chunk of 512 rows
     # balanced weight phase (16 x 32 tiles, equal runs of chunks per CTA, one
-    # more grid barrier and the fix-up): fixed part and per chunk of a run
+    # more grid barrier and the fix-up): fixed part and per chunk of a run; nets of
+    # more than one hidden layer, or with `large_min_per_cta` out of reach
     balanced_fixed_us: float = 6.66
     balanced_chunk_us: float = 2.12
     balanced_min_chunks: int = 24
     chunk_rows: int = 512
-    # one-CTA kernel: per group of B patterns
+    # large groups of one-hidden-layer nets (changes summed in registers), from
+    # this many patterns per CTA on: barriers, the reduction over the CTAs and the
+    # weight copy, then one cost per pass of 64 patterns
+    large_min_per_cta: int = 40
+    large_fixed_us: float = 12.0
+    large_pass: int = 64
+    large_pass_us: float = 32.9
+    # groups of up to 4 patterns: one CTA (any depth), one cluster (one hidden layer)
     small_us: tuple = ((1, 6.68), (2, 7.37), (4, 9.17))
+    cluster_us: tuple = ((1, 2.0), (2, 2.2), (4, 2.7))
 
 
 def gb300_group_size(B, n_sm=152, max_pg=8, wide=True):
@@ -115,12 +123,16 @@ def gb300_group_size(B, n_sm=152, max_pg=8, wide=True):
     return pg
 
 
-def gb300_update_us(B, tiles=121, tiles16=64, ph: GB300Phases = GB300Phases(), small_max=4):
-    """Predicted microseconds per update of a B-pattern group (203-120-26)."""
+def gb300_update_us(B, tiles=121, tiles16=64, ph: GB300Phases = GB300Phases(), small_max=4, cluster=False):
+    """Predicted microseconds per update of a B-pattern group (203-120-26).
+    Groups of up to `small_max` patterns run on one CTA, or, with `cluster`, on the
+    cluster that keeps a one-hidden-layer net on chip."""
     if B <= small_max:
-        for b, us in ph.small_us:
+        for b, us in ph.cluster_us if cluster else ph.small_us:
             if B <= b:
                 return us
+    if B >= ph.large_min_per_cta * ph.n_sm:
+        return ph.large_fixed_us + -(-(-(-B // ph.n_sm)) // ph.large_pass) * ph.large_pass_us
     pg = gb300_group_size(B, ph.n_sm)
     passes = -(-(-(-B // ph.n_sm)) // pg)
     t = ph.pattern_fixed_us + passes * dict(ph.pass_us)[pg]

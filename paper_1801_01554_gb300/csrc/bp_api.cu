@@ -224,9 +224,13 @@ bp_status bp_create(const int* sizes, int n_layers, float lr, float momentum, in
         if (e == cudaSuccess) e = cudaMalloc(&net->wpart, (size_t)net->num_sms * 2 * 512 * sizeof(float));
         if (e == cudaSuccess) e = cudaMalloc(&net->bar, (size_t)bp::kBarWords * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMalloc(&net->flags, 4 * sizeof(int));
-        if (e == cudaSuccess && f32_large_shape_ok(v) && max_batch >= kLargeMinPerCta * net->num_sms)
-            e = cudaMalloc(&net->gpart, (size_t)net->num_sms * v.P * sizeof(float));
         if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc(scratch)"));
+        // per-CTA sums of large groups; without room for them these groups take the tiled weight phase
+        if (f32_large_shape_ok(v) && max_batch >= kLargeMinPerCta * net->num_sms &&
+            cudaMalloc(&net->gpart, (size_t)net->num_sms * v.P * sizeof(float)) != cudaSuccess) {
+            net->gpart = nullptr;
+            cudaGetLastError();
+        }
         e = cudaMemset(net->bar, 0, (size_t)bp::kBarWords * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMemset(net->flags, 0, 4 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(net->A, 0, v.a_floats * sizeof(float));

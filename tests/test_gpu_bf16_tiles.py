@@ -18,7 +18,8 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 CASES = [((8, 8, 8), 1), ((72, 264, 136), 129), ((320, 520, 64), 63), ((136, 1032, 40), 127),
-         ((64, 128, 32), 4100), ((256, 328, 200, 72), 1025), ((256, 512, 64), 20000)]
+         ((64, 128, 32), 4100), ((256, 328, 200, 72), 1025), ((256, 512, 64), 20000),
+         ((136, 2312, 264), 130)]   # more than one group of row blocks in the pooled changes
 
 
 @pytest.mark.parametrize("sizes,B", CASES)

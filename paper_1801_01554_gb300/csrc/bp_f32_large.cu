@@ -44,6 +44,11 @@ struct LargeCfg {
     static constexpr int kPG = kP / 4;              // pattern groups: patterns pg, pg + kPG, ..
 };
 
+// A float4 of a row of changes whose bias is component `last` (or lies further on).
+__device__ __forceinline__ float4 pads_cleared(float4 x, int last) {
+    return make_float4(x.x, last >= 1 ? x.y : 0.f, last >= 2 ? x.z : 0.f, last >= 3 ? x.w : 0.f);
+}
+
 template <int TU>
 __global__ void __launch_bounds__(kT, 1)
     k_train_large(const __grid_constant__ F32View v, const __grid_constant__ LargePlan c, const float* X, const float* T,
@@ -313,7 +318,8 @@ __global__ void __launch_bounds__(kT, 1)
             }
             __syncthreads();   // the rows may be overwritten
         }
-        // this CTA's sums
+        // this CTA's sums; those of a row's padding columns are 0 (their inputs are 0, but 0
+        // times a NaN or an infinite delta is NaN)
         float* gp = v.gpart + (long long)blockIdx.x * v.P;
         if (w1c) {
 #pragma unroll
@@ -323,7 +329,7 @@ __global__ void __launch_bounds__(kT, 1)
                     if (TU * ur1 + u < H && 12 * cg1 + q < kp1) {
                         const float2 a = unpack2(g1[u][q / 2]), b = unpack2(g1[u][q / 2 + 1]);
                         __stcg(reinterpret_cast<float4*>(gp + v.woff[1] + (long long)(TU * ur1 + u) * kp1 + 12 * cg1 + q),
-                               make_float4(a.x, a.y, b.x, b.y));
+                               pads_cleared(make_float4(a.x, a.y, b.x, b.y), n0 - 12 * cg1 - q));
                     }
         }
         if (w2c) {
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(kT, 1)
             for (int u = 0; u < 4; ++u)
                 if (4 * kr2 + u < n2)
                     __stcg(reinterpret_cast<float4*>(gp + v.woff[2] + (long long)(4 * kr2 + u) * kp2 + 4 * cg2),
-                           make_float4(g2[u][0], g2[u][1], g2[u][2], g2[u][3]));
+                           pads_cleared(make_float4(g2[u][0], g2[u][1], g2[u][2], g2[u][3]), H - 4 * cg2));
         }
         sse = warp_sum(sse);
         if (lane == 0) s_sse[warp] = sse;

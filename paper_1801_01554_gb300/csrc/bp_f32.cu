@@ -1336,10 +1336,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float4* wp = reinterpret_cast<float4*>(smem + v.woff[l] + (long long)j * v.kp[l]) + c;
                 float4 w = *wp;
                 if (GUARD) {
+                    // columns past the bias are no weights: their inputs are 0, but 0 times a NaN
+                    // or an infinite delta is NaN, which is nothing for the guard to count
+                    const int last = v.n[l - 1] - 4 * c;
                     g.x = guard_count(guard, g.x, n_bad);
-                    g.y = guard_count(guard, g.y, n_bad);
-                    g.z = guard_count(guard, g.z, n_bad);
-                    g.w = guard_count(guard, g.w, n_bad);
+                    g.y = last >= 1 ? guard_count(guard, g.y, n_bad) : 0.f;
+                    g.z = last >= 2 ? guard_count(guard, g.z, n_bad) : 0.f;
+                    g.w = last >= 3 ? guard_count(guard, g.w, n_bad) : 0.f;
                 }
                 float4& u = vel[m];
                 u.x = a_lr * g.x + mom * u.x;

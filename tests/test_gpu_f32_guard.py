@@ -64,6 +64,13 @@ def test_guard_counts_weight_changes_only_in_large_groups(sizes, plant):
 
 
 @pytest.mark.parametrize("plant", ["nan input", "infinite target"])
+@pytest.mark.parametrize("B", [1, 2, 4])
+def test_guard_counts_weight_changes_only_on_one_cta(B, plant):
+    got, want = nonfinite_count((64, 33, 17, 9), B, plant)
+    assert got == want
+
+
+@pytest.mark.parametrize("plant", ["nan input", "infinite target"])
 @pytest.mark.parametrize("sizes,B", [((203, 120, 26), 512), ((202, 61, 26), 5), ((64, 33, 17, 9), 300)])
 def test_guard_counts_weight_changes_only_on_the_grid_wide_kernel(sizes, B, plant):
     got, want = nonfinite_count(sizes, B, plant)

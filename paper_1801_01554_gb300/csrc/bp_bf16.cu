@@ -260,6 +260,21 @@ __device__ __forceinline__ float bf16_round(float x) {
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
+// The same barrier; true in every epilogue thread if x is true in any.
+__device__ __forceinline__ bool epi_any(bool x) {
+    unsigned r;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.or.pred p, 1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"(x ? 1u : 0u), "n"(kEpiThreads)
+        : "memory");
+    return r != 0;
+}
+
 // ------------------------------------------------------------ epilogue
 // A warp's 32 x 32 block of bf16 as 16-byte pieces (8 columns).  Global memory is read
 // and written with lane (row 8 j + lane / 4, piece lane % 4), four lanes to a 64-byte
@@ -889,9 +904,10 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 }
             };
             load_aux(cbeg, aux[0]);
-            mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
-            epi_bar();                     // the epilogue warps leave together on an abort
-            if (*abort_flag) break;
+            // The epilogue warps leave together: the flag may rise between two warps' reads of it,
+            // and a warp that stayed would wait at the barriers below for those that left.
+            const bool got = mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
+            if (epi_any(!got || *abort_flag != 0)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
             if constexpr (MODE == MODE_DWU) {

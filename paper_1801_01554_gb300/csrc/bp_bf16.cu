@@ -12,9 +12,10 @@
 //   hidden delta (Section 3)  delta_{l-1} = (delta_l W_l) * a (1 - a), for
 //                               l = L..2 only: no delta for the input units
 //                               (Section 6.1)
-//   pooled change (Sec. 4.1)  G_l = delta_l^T A_{l-1}, K = the batch, split
-//                               over K into fp32 partial sums; the layers
-//                               share one launch
+//   pooled change (Sec. 4.1)  G_l = delta_l^T A_{l-1}, K = the batch, summed
+//                               in fp32 chains of bounded length and, where tiles
+//                               are few, split over CTAs into partial sums; the
+//                               layers share one launch
 //
 // Activations, deltas and weights are stored once, row-major.  An operand whose
 // rows run along K is staged as it lies; one whose rows run along M or N (W_l in
@@ -76,12 +77,14 @@ struct GemmArgs {
     int* flags;
 };
 
-// The pooled-change GEMMs of all layers, one launch: layer l's tiles are the
-// items [item0[l], item0[l + 1]), times `splits` runs of kb_per_split K blocks.
+// The pooled-change GEMMs of all layers, one launch: layer l's tiles are
+// [tile0[l], tile0[l + 1]), times `splits` runs of kb_per_split K blocks.  A run is
+// accumulated in TMEM `chain` K blocks at a time; the epilogue adds these sums.
 struct DwLayer {
     int M, N;               // n_l, n_{l-1}
     int num_m, num_n;
     int tile0;              // first tile of the layer
+    int chain;              // K blocks of one sum in TMEM (sum_chain)
     float* gpart;           // [splits, M, N]
 };
 struct DwArgs {
@@ -333,7 +336,8 @@ __device__ __forceinline__ void store_partial(float* gpart, int M, int N, int m,
 }
 
 // 32 lanes x 16 consecutive fp32 columns from TMEM.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -342,7 +346,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// And back.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]),
+        "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]),
+        "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // One 32-column chunk of the tile for the 32 rows of one epilogue warp (this
 // lane's row m).  Values are rounded to bf16 and staged by rows in the warp's
@@ -589,6 +609,7 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
 // A work item of a GEMM launch: a tile and its run of K blocks.
 struct Item {
     int mb, nb, kb0, kb1;
+    int chain;               // K blocks per sum in TMEM
     int l, split;            // pooled change only
 };
 // Work of the forward and hidden-delta launches: one problem, whole K.
@@ -600,7 +621,7 @@ struct OneGemm {
     const CUtensorMap *ma, *mb_;
     __device__ int items() const { return g.num_m * g.num_n; }
     __device__ Item item(int it) const {
-        Item w{0, 0, 0, g.kb_total, 0, 0};
+        Item w{0, 0, 0, g.kb_total, g.kb_total, 0, 0};
         tile_coords<MODE == MODE_DX ? 16 : 4>(it, g.num_m, g.num_n, w.mb, w.nb);
         return w;
     }
@@ -634,11 +655,12 @@ struct DwGemm {
         tile_coords<16>(tile - y.tile0, y.num_m, y.num_n, w.mb, w.nb);
         w.kb0 = w.split * g.kb_per_split;
         w.kb1 = min(g.kb_total, w.kb0 + g.kb_per_split);
+        w.chain = y.chain;
         return w;
     }
     __device__ void touch() const {
         asm volatile("" ::"r"(g.splits), "r"(g.kb_per_split), "r"(g.kb_total), "l"(g.flags));
-        for (int l = 0; l < g.L; ++l) asm volatile("" ::"r"(g.ly[l].N), "l"(g.ly[l].gpart));
+        for (int l = 0; l < g.L; ++l) asm volatile("" ::"r"(g.ly[l].N), "r"(g.ly[l].chain), "l"(g.ly[l].gpart));
     }
     __device__ void prefetch_maps() const {
         for (int l = 0; l < g.L; ++l) {
@@ -696,12 +718,11 @@ __device__ __forceinline__ void update_block_load(const UpdArgs& a, const LayerU
     }
 }
 __device__ __forceinline__ void update_block_apply(const UpdArgs& a, const LayerUpd& u, int M, int N, int m0, int n0,
-                                                   const uint32_t (&r)[16], UpdBlock& x, float4* sF) {
+                                                   const float (&r)[16], UpdBlock& x, float4* sF) {
     const int lane = threadIdx.x & 31, piece = lane & 3, n = n0 + 4 * piece;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        sF[lane * 4 + (k ^ ((lane >> 1) & 3))] = make_float4(__uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]),
-                                                              __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
+        sF[lane * 4 + (k ^ ((lane >> 1) & 3))] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -832,27 +853,30 @@ __device__ __forceinline__ void gemm_body(const Work work) {
             Item w = first;
             for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
                 if (it != (int)blockIdx.x) w = work.item(it);
-                if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
-                uint32_t accumulate = 0;
-                for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    if (!ready && !mbar_wait(&full[stage], phase, abort_flag, g.flags)) { ok = false; break; }
+                for (int c0 = w.kb0; c0 < w.kb1; c0 += w.chain) {
+                    const int c1 = min(w.kb1, c0 + w.chain);
+                    if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.flags)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t al = a0 + stage * (Cfg::kStageBytes >> 4), bl = b0 + stage * (Cfg::kStageBytes >> 4);
-                    umma_bf16<idesc>(tmem_d, al, bl, accumulate);
+                    const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
+                    uint32_t accumulate = 0;
+                    for (int kb = c0; kb < c1; ++kb) {
+                        if (!ready && !mbar_wait(&full[stage], phase, abort_flag, g.flags)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t al = a0 + stage * (Cfg::kStageBytes >> 4), bl = b0 + stage * (Cfg::kStageBytes >> 4);
+                        umma_bf16<idesc>(tmem_d, al, bl, accumulate);
 #pragma unroll
-                    for (int kk = 1; kk < BK / UMMA_K; ++kk)
-                        umma_bf16<idesc>(tmem_d, al + kk * k_step_units<Work::kAMn>(), bl + kk * k_step_units<Work::kBMn>(), 1u);
-                    accumulate = 1u;
-                    issued_any = true;
-                    umma_commit(&empty[stage]);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
-                    ready = mbar_test(&full[stage], phase);
+                        for (int kk = 1; kk < BK / UMMA_K; ++kk)
+                            umma_bf16<idesc>(tmem_d, al + kk * k_step_units<Work::kAMn>(), bl + kk * k_step_units<Work::kBMn>(), 1u);
+                        accumulate = 1u;
+                        issued_any = true;
+                        umma_commit(&empty[stage]);
+                        if (++stage == S) { stage = 0; phase ^= 1u; }
+                        ready = mbar_test(&full[stage], phase);
+                    }
+                    if (!ok) break;
+                    umma_commit(&tfull[acc]);
+                    if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
                 }
-                if (!ok) break;
-                umma_commit(&tfull[acc]);
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
             if (!ok && issued_any) {
                 // let every MMA already issued finish before TMEM is released
@@ -870,6 +894,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
         const int cbeg = (ew >> 2) * (BN / 2);   // this warp's half of the columns
         int acc = 0;
         unsigned acc_phase = 0;
+        constexpr bool kDw = MODE == MODE_DW || MODE == MODE_DWU;
         if constexpr (MODE == MODE_DWU) {
             // this CTA's share of the biases and the error sum, while the first tile accumulates
             const int nb = work.u.bias_blocks + (work.u.sse_out != nullptr ? 1 : 0);
@@ -887,11 +912,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     sbias[c] = n < g.N ? g.bias[n] : 0.f;
                 }
             }
-            UpdBlock cur, nxt;
-            if constexpr (MODE == MODE_DWU) {
-                const DwLayer& y = g.ly[w.l];
-                update_block_load(work.u, work.u.ly[w.l], y.M, y.N, w.mb * BM + q * 32, w.nb * BN + cbeg, cur);
-            }
             const int m0 = w.mb * BM + q * 32, m = m0 + lane;
             Row32 aux[2];   // the targets' or activations' block of this chunk and of the next one
             auto load_aux = [&](int c0, Row32& r) {
@@ -904,40 +924,117 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 }
             };
             load_aux(cbeg, aux[0]);
-            // The epilogue warps leave together: the flag may rise between two warps' reads of it,
-            // and a warp that stayed would wait at the barriers below for those that left.
-            const bool got = mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
-            if (epi_any(!got || *abort_flag != 0)) break;
-            tc_fence_after();
-            const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
-            if constexpr (MODE == MODE_DWU) {
-                const DwLayer& y = g.ly[w.l];
-                const LayerUpd& u = work.u.ly[w.l];
-                float4* sF = reinterpret_cast<float4*>(stage_out + ew * 1024);
-                for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
-                    const int n0 = w.nb * BN + c0;
-                    uint32_t r[16];
-                    update_block_load(work.u, u, y.M, y.N, m0, n0 + 16, nxt);
-                    tmem_ld16(tbase + (uint32_t)c0, r);
-                    update_block_apply(work.u, u, y.M, y.N, m0, n0, r, cur, sF);
-                    if (c0 + 32 < cbeg + BN / 2) update_block_load(work.u, u, y.M, y.N, m0, n0 + 32, cur);
-                    tmem_ld16(tbase + (uint32_t)(c0 + 16), r);
-                    update_block_apply(work.u, u, y.M, y.N, m0, n0 + 16, r, nxt, sF);
-                }
+            // Waits for the accumulator; false if that ran out.  With barriers between the epilogue
+            // warps below, they leave together: the abort flag may rise between two warps' reads
+            // of it, and a warp that stayed would wait for those that left.
+            auto wait_acc = [&] {
+                const bool got = mbar_wait(&tfull[acc], acc_phase, abort_flag, g.flags);
+                const bool leave = kDw ? __any_sync(0xffffffffu, !got) : epi_any(!got || *abort_flag != 0);
+                tc_fence_after();
+                return !leave;
+            };
+            // This warp's lanes of an accumulator; that accumulator is free for the next sum.
+            const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+            auto release = [&](int a) {
                 tc_fence_before();
-                mbar_arrive(&tempty[acc]);
+                mbar_arrive(&tempty[a]);
+            };
+            auto next_acc = [&] {
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-            } else if constexpr (MODE == MODE_DW) {
+            };
+            if constexpr (kDw) {
                 const DwLayer& y = g.ly[w.l];
-                for (int c0 = cbeg; c0 < cbeg + BN / 2 && w.nb * BN + c0 < y.N; c0 += 32) {
-                    float v[32];
-                    tmem_ld32(tbase + (uint32_t)c0, v);
-                    store_partial(y.gpart, y.M, y.N, m, w.nb * BN + c0, w.split, v);
+                const int ncol = y.N - w.nb * BN;   // columns of the layer from this tile on
+                // The sums of the chains before the last one: in registers up to 128 columns, as
+                // many as a thread holds beside the update's loads.  At 256 the two accumulators
+                // take turns: each chain's sum has the one before added in place, which then is
+                // free for the chain after it (its MMAs wait for that, about 1,000 clocks, which
+                // a chain of 128 K blocks, 68,000, does not feel; through global memory, 128 KB
+                // a CTA and tile, 50 steps of 4096^5 took 210.0 ms).
+                constexpr bool kRegs = BN <= 128;
+                float part[kRegs ? BN / 2 : 1];
+                if constexpr (kRegs) {
+#pragma unroll
+                    for (int c = 0; c < BN / 2; ++c) part[c] = 0.f;
                 }
-                tc_fence_before();
-                mbar_arrive(&tempty[acc]);
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                auto add_previous = [&] {   // 256 columns: accumulator 1 - acc into acc
+                    for (int c = cbeg; c < cbeg + BN / 2; c += 16) {
+                        float x[16], v[16];
+                        tmem_ld16(trow + (uint32_t)((1 - acc) * BN + c), x);
+                        tmem_ld16(trow + (uint32_t)(acc * BN + c), v);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) v[k] += x[k];
+                        tmem_st16(trow + (uint32_t)(acc * BN + c), v);
+                    }
+                    tmem_wait_st();
+                    release(1 - acc);
+                };
+                bool stay = true;
+                for (int c0 = w.kb0; c0 + w.chain < w.kb1; c0 += w.chain) {
+                    stay = wait_acc();
+                    if (!stay) break;
+                    if constexpr (kRegs) {
+#pragma unroll
+                        for (int i = 0; i < BN / 64; ++i) {
+                            float v[32];
+                            tmem_ld32(trow + (uint32_t)(acc * BN + cbeg + 32 * i), v);
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) part[32 * i + c] += v[c];
+                        }
+                        release(acc);
+                    } else if (c0 > w.kb0) {
+                        add_previous();
+                    }
+                    next_acc();
+                }
+                if (!stay) break;
+                const bool several = w.kb1 - w.kb0 > w.chain;
+                if constexpr (MODE == MODE_DWU) {
+                    const LayerUpd& u = work.u.ly[w.l];
+                    float4* sF = reinterpret_cast<float4*>(stage_out + ew * 1024);
+                    UpdBlock cur, nxt;
+                    auto load = [&](int c, UpdBlock& b) {
+                        update_block_load(work.u, u, y.M, y.N, m0, w.nb * BN + cbeg + c, b);
+                    };
+                    auto apply = [&](int c, UpdBlock& b) {
+                        float r[16];
+                        tmem_ld16(trow + (uint32_t)(acc * BN + cbeg + c), r);
+                        if constexpr (kRegs) {
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) r[k] += part[c + k];
+                        }
+                        update_block_apply(work.u, u, y.M, y.N, m0, w.nb * BN + cbeg + c, r, b, sF);
+                    };
+                    load(0, cur);
+                    if (!wait_acc()) break;
+                    if (!kRegs && several) add_previous();
+#pragma unroll(kRegs ? BN / 64 : 1)
+                    for (int i = 0; i < BN / 64; ++i) {
+                        if (cbeg + 32 * i >= ncol) break;
+                        load(32 * i + 16, nxt);
+                        apply(32 * i, cur);
+                        if (i + 1 < BN / 64) load(32 * i + 32, cur);
+                        apply(32 * i + 16, nxt);
+                    }
+                } else {
+                    if (!wait_acc()) break;
+                    if (!kRegs && several) add_previous();
+#pragma unroll(kRegs ? BN / 64 : 1)
+                    for (int i = 0; i < BN / 64; ++i) {
+                        if (cbeg + 32 * i >= ncol) break;
+                        float v[32];
+                        tmem_ld32(trow + (uint32_t)(acc * BN + cbeg + 32 * i), v);
+                        if constexpr (kRegs) {
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) v[c] += part[32 * i + c];
+                        }
+                        store_partial(y.gpart, y.M, y.N, m, w.nb * BN + cbeg + 32 * i, w.split, v);
+                    }
+                }
+                release(acc);
+                next_acc();
             } else {
+                if (!wait_acc()) break;
                 const bool row_ok = m < g.M;
                 float sse = 0.f;
                 bf16* sS = stage_out + ew * 1024;
@@ -948,14 +1045,12 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     if (n0 >= g.N) break;   // (column sums past N are not read)
                     if (i + 1 < BN / 64) load_aux(c0 + 32, aux[(i + 1) & 1]);
                     float v[32];
-                    tmem_ld32(tbase + (uint32_t)c0, v);
+                    tmem_ld32(trow + (uint32_t)(acc * BN + c0), v);
                     epilogue_chunk<BN, MODE>(g, m0, n0, v, sse, row_ok, sS, sbias + c0, aux[i & 1],
                                          want_colsum ? colsum + slot * BN + c0 : nullptr);
                 }
-                // TMEM is free for the next accumulation into this buffer
-                tc_fence_before();
-                mbar_arrive(&tempty[acc]);
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                release(acc);   // TMEM is free for the next accumulation into this buffer
+                next_acc();
                 if (want_colsum) {
                     epi_bar();
                     const int t = threadIdx.x - 64;   // 0 .. kEpiThreads - 1
@@ -1346,6 +1441,36 @@ cudaError_t run_forward(Bf16Net* b, const bf16* X, int B, const bf16* T, bf16* Y
     return cudaSuccess;
 }
 
+// K blocks that one sum of a layer's pooled change runs over in TMEM.  The tensor cores
+// truncate as they accumulate, so that a sum's error grows with its chain: 2-norm error
+// against float64 of the change of 4096 x 4096 weights, one chain / this rule, 8,192
+// patterns 8.1e-6 / 3.7e-6, 16,384 1.7e-5 / 8.0e-6; 208 x 1024 by 512 3.4e-7 / 1.2e-7.
+// The epilogue adds the chains' sums, rounding to nearest.  Their number s is the split of K
+// that would be fastest with 128 x 256 tiles and a plane of partial sums each: the least of
+//   ceil(tiles * s / num_sms) / s  (waves of 1/s-K items, in times of a full-K tile)
+//   + s * tiles * plane            (writing and reading a plane; a tile's share of it over
+//                                   its MMAs is 4 / K times the 1.87 bf16 flops an SM does
+//                                   in the time of a byte of DRAM traffic),
+// many for the few tiles of a small layer, one or two for a layer of several waves.  us,
+// one chain / this rule: 25 steps of 8,192 of 1024-2048-2048-512 7,248 / 7,303, 50 steps of
+// 4096^5 201,690 / 201,520, two epochs of 16,200 of 208-1024-32 by 512 1,333 / 1,357.
+constexpr int kMaxChains = 16;
+int sum_chain(int M, int N, int kb_total, int num_sms) {
+    const int tiles = tiles_of(M, N, 256);
+    const double plane = 4.0 * 1.87 / ((double)kb_total * BK);
+    int best = 1;
+    double best_cost = 0.0;
+    for (int s = 1; s <= kMaxChains && s <= kb_total; ++s) {
+        const double waves = (double)(((long long)tiles * s + num_sms - 1) / num_sms) / s;
+        const double cost = waves + s * plane * tiles;
+        if (s == 1 || cost < best_cost * (1.0 - 1e-9)) {
+            best = s;
+            best_cost = cost;
+        }
+    }
+    return ceil_div(kb_total, best);
+}
+
 // How the pooled-change launch of a group of B patterns is cut: the tile width,
 // the number of K splits, and whether the update runs in its epilogue (training, one
 // split).  All layers share the launch, so their tiles fill the last wave together.
@@ -1436,6 +1561,7 @@ cudaError_t run_backward(Bf16Net* b, const bf16* X, int B, const DwPlan& p, cons
         y.num_m = ceil_div(y.M, BM);
         y.num_n = ceil_div(y.N, p.bn);
         y.tile0 = tile;
+        y.chain = sum_chain(y.M, y.N, p.kb_total, b->num_sms);
         tile += y.num_m * y.num_n;
         y.gpart = b->gpart[l];
         if (!make_map(&maps.a[l - 1], b->dlt[l], B, y.M, BK) ||

@@ -2,13 +2,21 @@
 //
 // Every CTA trains its share of the group's patterns (Section 4.1's case
 // parallelism), kP at a time, with all weights in shared memory and the sums of
-// its changes in registers for the whole group: 256 threads, each with a block of
-// TU x 12 changes of [W_1 | b_1] and one of 4 x 4 of [W_2 | b_2].  Inputs,
-// activations and deltas of a pass never leave shared memory (the hidden deltas
-// replace the activations), so a group costs one read of its patterns and, at its
-// end, one parameter vector of sums per CTA: after a grid barrier every CTA adds
-// its share of the words over the CTAs in order, applies the momentum update of
-// Section 6.2.1 and, after a second barrier, copies the new weights in.
+// its changes on chip for the whole group: 256 threads, each with a block of
+// TU x 12 changes of [W_1 | b_1], kept in tensor memory between its uses, and one of
+// 4 x 4 of [W_2 | b_2] in registers.  Inputs, activations and deltas of a pass never
+// leave shared memory (the hidden deltas replace the activations), so a group costs
+// one read of its patterns and, at its end, one parameter vector of sums per CTA:
+// after a grid barrier every CTA adds its share of the words over the CTAs in a fixed
+// order, applies the momentum update of Section 6.2.1 and, after a second barrier,
+// copies the new weights in.
+//
+// No sum runs in one chain: net inputs add up 16 columns at a time, changes 32
+// patterns at a time (kCols, kChain), CTAs in four chains and a tree.  With one chain
+// each, 431 patterns long at groups of 65,536, a change's error against float64 was up to
+// half as large again as that of the tiled weight phase; now it is smaller (2-norm of W_1's
+// change, tiled / one chain / this: 203-60-26 by 16,384 1.65e-7 / 2.4e-7 / 1.6e-7, by 65,536
+// 1.3e-7 / 1.8e-7 / 1.0e-7; 64-50-10 by 65,536 8.6e-8 / 1.2e-7 / 6.5e-8).
 //
 // All five products are register-blocked: 4 patterns x 8 units in layer 1 (12
 // float4 loads for 128 multiply-adds), 4 x 2 in layer 2, 4 x 8 in the hidden
@@ -16,12 +24,12 @@
 // pattern).  What bounds it is shared memory's way into the registers, 128 bytes a
 // clock whatever the lanes share: a pass of 64 patterns of 203-120-26 takes 65,000
 // clocks, 26,000 in layer 1 (20,000 of loads, 13,000 of multiply-adds), 15,000 in
-// the changes of W_1 (12,300 of multiply-adds), 6,000 for the rows.  Blocks of 8 x 8
-// with K split over two halves of the threads, and rows carried through registers,
-// spilled and were slower.
+// the changes of W_1 (12,300 of multiply-adds), 6,000 for the rows.  Tensor memory frees the
+// registers that layer 1's two levels of sums need (kept in registers, W_1's sums made it
+// spill and cost a fifth); adding to them there takes about 700 clocks for TU = 8.
 // us per update, tiled weight phase (k_train) -> this kernel: 203-120-26 at groups of
-// 8,192: 52.8 -> 45.6, 16,384: 103.5 -> 77.8, 65,536: 349 -> 242; 203-60-26 at 65,536:
-// 391 -> 164; 64-50-10: 140 -> 95.
+// 8,192: 52.8 -> 46, 16,384: 103.5 -> 80, 65,536: 349 -> 243; 203-60-26 at 65,536:
+// 391 -> 162; 64-50-10: 140 -> 88.
 #include <cuda_runtime.h>
 
 #include "bp_f32_device.cuh"
@@ -31,6 +39,8 @@ namespace bp {
 namespace {
 
 constexpr int kT = 256;
+constexpr int kChain = 32;   // patterns of one chain of a change's sum
+constexpr int kCols = 16;    // columns of one chain of a net input
 
 struct LargePlan {
     int w1, w2, x, h, d, t, red, total;   // shared-memory offsets (floats)
@@ -42,11 +52,75 @@ template <int TU>
 struct LargeCfg {
     static constexpr int kP = TU == 8 ? 64 : 128;   // patterns of a pass
     static constexpr int kPG = kP / 4;              // pattern groups: patterns pg, pg + kPG, ..
+    // patterns between additions to the sums of W_1 in tensor memory (at TU = 8 the registers
+    // hold one level of sums only)
+    static constexpr int kMerge = TU == 8 ? kChain : kP;
 };
+
+__device__ __forceinline__ float4 add4(float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); }
 
 // A float4 of a row of changes whose bias is component `last` (or lies further on).
 __device__ __forceinline__ float4 pads_cleared(float4 x, int last) {
     return make_float4(x.x, last >= 1 ? x.y : 0.f, last >= 2 ? x.z : 0.f, last >= 3 ? x.w : 0.f);
+}
+
+// A thread's TU x 12 sums of changes of W_1 in its lane of tensor memory, columns from
+// taddr on, 16 at a time.
+__device__ __forceinline__ void sums_st16(uint32_t taddr, const f32x2 (&x)[8]) {
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float2 t = unpack2(x[i]);
+        r[2 * i] = __float_as_uint(t.x);
+        r[2 * i + 1] = __float_as_uint(t.y);
+    }
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]),
+        "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]),
+        "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void sums_ld16(uint32_t taddr, f32x2 (&x)[8]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+}
+__device__ __forceinline__ void sums_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+template <int TU>
+__device__ __forceinline__ void clear_sums(uint32_t taddr) {
+    const f32x2 z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int w = 0; w < TU * 12; w += 16) sums_st16(taddr + w, z);
+    sums_wait_st();
+}
+template <int TU>
+__device__ __forceinline__ void load_sums(uint32_t taddr, f32x2 (&g)[TU][6]) {
+#pragma unroll
+    for (int w = 0; w < TU * 12; w += 16) {
+        f32x2 x[8];
+        sums_ld16(taddr + w, x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g[(w / 2 + i) / 6][(w / 2 + i) % 6] = x[i];
+    }
+}
+template <int TU>
+__device__ __forceinline__ void add_sums(uint32_t taddr, const f32x2 (&g)[TU][6]) {
+#pragma unroll
+    for (int w = 0; w < TU * 12; w += 16) {
+        f32x2 x[8];
+        sums_ld16(taddr + w, x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = add2(x[i], g[(w / 2 + i) / 6][(w / 2 + i) % 6]);
+        sums_st16(taddr + w, x);
+    }
+    sums_wait_st();
 }
 
 template <int TU>
@@ -54,9 +128,12 @@ __global__ void __launch_bounds__(kT, 1)
     k_train_large(const __grid_constant__ F32View v, const __grid_constant__ LargePlan c, const float* X, const float* T,
                   int n_patterns, int minibatch, int n_steps, float* sse_out, int fold_g) {
     constexpr int P = LargeCfg<TU>::kP, PG = LargeCfg<TU>::kPG;
+    constexpr int kMerge = LargeCfg<TU>::kMerge;
+    constexpr int kTmem = 2 * 12 * TU <= 128 ? 128 : 256;   // columns of tensor memory
     extern __shared__ __align__(128) float sm[];
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ float s_sse[kT / 32];
+    __shared__ uint32_t s_tmem;
     if (!bounds_ok((unsigned)c.total <= dyn_smem_floats(), v.flags)) return;   // in every CTA alike
     // a latched timeout means an earlier launch left the barrier half-way
     if (__ldcg(v.flags) & kFlagTimeout) return;
@@ -70,6 +147,10 @@ __global__ void __launch_bounds__(kT, 1)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "n"(kTmem) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
     unsigned target = __ldcg(v.bar);
     // pads: the true unit's 1 after the inputs and the activations, zeros after it
     for (int e = tid; e < P * (kp1 - n0); e += kT) {
@@ -81,7 +162,16 @@ __global__ void __launch_bounds__(kT, 1)
         sm[c.h + r * hp + i] = i == H ? 1.f : 0.f;
     }
     for (int e = tid; e < P * dp; e += kT) sm[c.d + e] = 0.f;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // this thread's sums of W_1 between the passes: two warps a lane quarter
+    const uint32_t tmem = s_tmem, own = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (TU * 12);
+    auto leave = [&] {   // every thread: the CTA's tensor memory is given back
+        __syncthreads();
+        if (warp == 0)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmem) : "memory");
+    };
 
     // this thread's blocks
     const int pg = tid % PG, ug = tid / PG;            // layer 1: patterns pg + PG i, units ug + UG j
@@ -114,12 +204,8 @@ __global__ void __launch_bounds__(kT, 1)
                          "l"(v.theta), "r"((unsigned)v.P * 4u), "r"(smem_u32(&s_bar))
                          : "memory");
         }
-        f32x2 g1[TU][6];   // pairs of columns
         float g2[4][4], sse = 0.f;
-#pragma unroll
-        for (int u = 0; u < TU; ++u)
-#pragma unroll
-            for (int q = 0; q < 6; ++q) g1[u][q] = 0;
+        clear_sums<TU>(own);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -148,7 +234,7 @@ __global__ void __launch_bounds__(kT, 1)
             }
             cp_async_wait<0>();
             ok = __syncthreads_and(ok) != 0;
-            if (!ok) return;   // the copy did not arrive: no update
+            if (!ok) return leave();   // the copy did not arrive: no update
             if (np == 0) break;
             // the next pass's rows on their way to L2
             {
@@ -168,8 +254,7 @@ __global__ void __launch_bounds__(kT, 1)
                 int wo[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) wo[j] = min(ug + UG * j, H - 1) * kp1;
-#pragma unroll 2
-                for (int k = 0; k < kp1; k += 4) {
+                auto columns = [&](int k, float (&sum)[4][8]) {
                     float4 x[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) x[i] = ld4(xr + PG * i * xp + k);
@@ -178,13 +263,28 @@ __global__ void __launch_bounds__(kT, 1)
                         const float4 w = ld4(W1 + wo[j] + k);
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            acc[i][j] = fmaf(w.x, x[i].x, acc[i][j]);
-                            acc[i][j] = fmaf(w.y, x[i].y, acc[i][j]);
-                            acc[i][j] = fmaf(w.z, x[i].z, acc[i][j]);
-                            acc[i][j] = fmaf(w.w, x[i].w, acc[i][j]);
+                            sum[i][j] = fmaf(w.x, x[i].x, sum[i][j]);
+                            sum[i][j] = fmaf(w.y, x[i].y, sum[i][j]);
+                            sum[i][j] = fmaf(w.z, x[i].z, sum[i][j]);
+                            sum[i][j] = fmaf(w.w, x[i].w, sum[i][j]);
                         }
                     }
+                };
+                int k = 0;
+                for (; k + kCols <= kp1; k += kCols) {
+                    float blk[4][8];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) blk[i][j] = 0.f;
+#pragma unroll 2
+                    for (int q = 0; q < kCols; q += 4) columns(k + q, blk);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) acc[i][j] += blk[i][j];
                 }
+                for (; k < kp1; k += 4) columns(k, acc);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int u = ug + UG * j;
@@ -202,22 +302,35 @@ __global__ void __launch_bounds__(kT, 1)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
                 const float* hr = sm + c.h + pp * hp;
-#pragma unroll 2
-                for (int k = 0; k < kp2; k += 4) {
+                auto columns = [&](int k, float (&sum)[4][2]) {
                     const float4 wa = ld4(W2 + k0 * kp2 + k), wb = ld4(W2 + k1 * kp2 + k);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float4 h = ld4(hr + PG * i * hp + k);
-                        acc[i][0] = fmaf(wa.x, h.x, acc[i][0]);
-                        acc[i][1] = fmaf(wb.x, h.x, acc[i][1]);
-                        acc[i][0] = fmaf(wa.y, h.y, acc[i][0]);
-                        acc[i][1] = fmaf(wb.y, h.y, acc[i][1]);
-                        acc[i][0] = fmaf(wa.z, h.z, acc[i][0]);
-                        acc[i][1] = fmaf(wb.z, h.z, acc[i][1]);
-                        acc[i][0] = fmaf(wa.w, h.w, acc[i][0]);
-                        acc[i][1] = fmaf(wb.w, h.w, acc[i][1]);
+                        sum[i][0] = fmaf(wa.x, h.x, sum[i][0]);
+                        sum[i][1] = fmaf(wb.x, h.x, sum[i][1]);
+                        sum[i][0] = fmaf(wa.y, h.y, sum[i][0]);
+                        sum[i][1] = fmaf(wb.y, h.y, sum[i][1]);
+                        sum[i][0] = fmaf(wa.z, h.z, sum[i][0]);
+                        sum[i][1] = fmaf(wb.z, h.z, sum[i][1]);
+                        sum[i][0] = fmaf(wa.w, h.w, sum[i][0]);
+                        sum[i][1] = fmaf(wb.w, h.w, sum[i][1]);
+                    }
+                };
+                int k = 0;
+                for (; k + kCols <= kp2; k += kCols) {
+                    float blk[4][2];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) blk[i][0] = blk[i][1] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < kCols; q += 4) columns(k + q, blk);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        acc[i][0] += blk[i][0];
+                        acc[i][1] += blk[i][1];
                     }
                 }
+                for (; k < kp2; k += 4) columns(k, acc);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int p = pp + PG * i;
@@ -267,14 +380,25 @@ __global__ void __launch_bounds__(kT, 1)
             if (w2c) {
                 const float* dr = sm + c.d + 4 * kr2;
                 const float* hr = sm + c.h + 4 * cg2;
-#pragma unroll 4
-                for (int p = 0; p < P; ++p) {
-                    const float4 d = ld4(dr + p * dp), h = ld4(hr + p * hp);
-                    const float dv[4] = {d.x, d.y, d.z, d.w}, hx[4] = {h.x, h.y, h.z, h.w};
+                for (int pc = 0; pc < P; pc += kChain) {
+                    float l2[4][4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) g2[u][q] = fmaf(dv[u], hx[q], g2[u][q]);
+                        for (int q = 0; q < 4; ++q) l2[u][q] = 0.f;
+#pragma unroll 4
+                    for (int p = pc; p < pc + kChain; ++p) {
+                        const float4 d = ld4(dr + p * dp), h = ld4(hr + p * hp);
+                        const float dv[4] = {d.x, d.y, d.z, d.w}, hx[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) l2[u][q] = fmaf(dv[u], hx[q], l2[u][q]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) g2[u][q] += l2[u][q];
                 }
             }
             __syncthreads();
@@ -293,27 +417,49 @@ __global__ void __launch_bounds__(kT, 1)
             }
             __syncthreads();
             // 4. the changes of W_1
-            if (w1c) {
+            {
                 const float* dr = sm + c.h + TU * ur1;
                 const float* xr = sm + c.x + 12 * cg1;
+                for (int pm = 0; pm < P; pm += kMerge) {
+                    f32x2 g1[TU][6];   // sums of kMerge patterns, pairs of columns
+#pragma unroll
+                    for (int u = 0; u < TU; ++u)
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) g1[u][q] = 0;
+                    if (w1c)
+                        for (int pc = pm; pc < pm + kMerge; pc += kChain) {
+                            f32x2 l1[TU][6];   // of one chain
+#pragma unroll
+                            for (int u = 0; u < TU; ++u)
+#pragma unroll
+                                for (int q = 0; q < 6; ++q) l1[u][q] = 0;
 #pragma unroll 2
-                for (int p = 0; p < P; ++p) {
-                    f32x2 xv[6];
+                            for (int p = pc; p < pc + kChain; ++p) {
+                                f32x2 xv[6];
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        const ulonglong2 x = ld4x2(xr + p * xp + 4 * q);
-                        xv[2 * q] = x.x;
-                        xv[2 * q + 1] = x.y;
-                    }
+                                for (int q = 0; q < 3; ++q) {
+                                    const ulonglong2 x = ld4x2(xr + p * xp + 4 * q);
+                                    xv[2 * q] = x.x;
+                                    xv[2 * q + 1] = x.y;
+                                }
 #pragma unroll
-                    for (int u = 0; u < TU; u += 4) {
-                        const float4 d = ld4(dr + p * hp + u);
-                        const f32x2 dd[4] = {pack2(d.x, d.x), pack2(d.y, d.y), pack2(d.z, d.z), pack2(d.w, d.w)};
+                                for (int u = 0; u < TU; u += 4) {
+                                    const float4 d = ld4(dr + p * hp + u);
+                                    const f32x2 dd[4] = {pack2(d.x, d.x), pack2(d.y, d.y), pack2(d.z, d.z), pack2(d.w, d.w)};
 #pragma unroll
-                        for (int t = 0; t < 4; ++t)
+                                    for (int t = 0; t < 4; ++t)
 #pragma unroll
-                            for (int q = 0; q < 6; ++q) g1[u + t][q] = fma2(dd[t], xv[q], g1[u + t][q]);
-                    }
+                                        for (int q = 0; q < 6; ++q) l1[u + t][q] = fma2(dd[t], xv[q], l1[u + t][q]);
+                                }
+                            }
+#pragma unroll
+                            for (int u = 0; u < TU; ++u)
+#pragma unroll
+                                for (int q = 0; q < 6; ++q)
+                                    g1[u][q] = kMerge > kChain ? add2(g1[u][q], l1[u][q]) : l1[u][q];
+                        }
+                    __syncwarp();
+                    add_sums<TU>(own, g1);
                 }
             }
             __syncthreads();   // the rows may be overwritten
@@ -321,6 +467,8 @@ __global__ void __launch_bounds__(kT, 1)
         // this CTA's sums; those of a row's padding columns are 0 (their inputs are 0, but 0
         // times a NaN or an infinite delta is NaN)
         float* gp = v.gpart + (long long)blockIdx.x * v.P;
+        f32x2 g1[TU][6];
+        load_sums<TU>(own, g1);
         if (w1c) {
 #pragma unroll
             for (int u = 0; u < TU; ++u)
@@ -347,7 +495,7 @@ __global__ void __launch_bounds__(kT, 1)
             for (int k = 0; k < kT / 32; ++k) e += s_sse[k];
             __stcg(v.sse_part + blockIdx.x, e);
         }
-        if (!grid_barrier(v.bar, target += gridDim.x, v.flags, wait_limit_ns(v))) return;
+        if (!grid_barrier(v.bar, target += gridDim.x, v.flags, wait_limit_ns(v))) return leave();
         if (blockIdx.x == gridDim.x - 1 && warp == 0) {
             float e = 0.f;
             for (int k = lane; k < (int)gridDim.x; k += 32) e += __ldcg(v.sse_part + k);
@@ -375,25 +523,31 @@ __global__ void __launch_bounds__(kT, 1)
             }
             if (mine) {
                 const float4* src = reinterpret_cast<const float4*>(v.gpart) + word;
-#pragma unroll 8
-                for (int k = sl; k < (int)gridDim.x; k += SL) {
-                    const float4 t = __ldcg(src + (long long)k * P4);
-                    a.x += t.x;
-                    a.y += t.y;
-                    a.z += t.z;
-                    a.w += t.w;
+                float4 f[4] = {a, a, a, a};   // four chains, then their tree
+                const int n_cta = (int)gridDim.x;
+                int k = sl;
+                for (; k + 7 * SL < n_cta; k += 8 * SL) {
+                    float4 t[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) t[q] = __ldcg(src + (long long)(k + q * SL) * P4);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) f[q & 3] = add4(f[q & 3], t[q]);
                 }
+#pragma unroll
+                for (int q = 0; q < 7; ++q)
+                    if (k + q * SL < n_cta) f[q & 3] = add4(f[q & 3], __ldcg(src + (long long)(k + q * SL) * P4));
+                a = add4(add4(f[0], f[1]), add4(f[2], f[3]));
                 red[sl * njp + (j - jb)] = a;
             }
             __syncthreads();
             if (owner) {
-                for (int k = 1; k < SL; ++k) {
-                    const float4 t = red[k * njp + (j - jb)];
-                    a.x += t.x;
-                    a.y += t.y;
-                    a.z += t.z;
-                    a.w += t.w;
-                }
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 f[4] = {z, z, z, z};
+                for (int k = 0; k < SL; k += 4)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (k + q < SL) f[q] = add4(f[q], red[(k + q) * njp + (j - jb)]);
+                a = add4(add4(f[0], f[1]), add4(f[2], f[3]));
                 float g[4] = {a.x + go.x, a.y + go.y, a.z + go.z, a.w + go.w};
                 float* vv = &vo.x;
                 float* tt = &th.x;
@@ -413,11 +567,12 @@ __global__ void __launch_bounds__(kT, 1)
         }
         // the next group's bulk copy reads theta through the async proxy
         asm volatile("fence.proxy.async.global;" ::: "memory");
-        if (s + 1 < n_steps && !grid_barrier(v.bar, target += gridDim.x, v.flags, wait_limit_ns(v))) return;
+        if (s + 1 < n_steps && !grid_barrier(v.bar, target += gridDim.x, v.flags, wait_limit_ns(v))) return leave();
     }
     // every CTA has passed a barrier, so every CTA has read bar[0]: publish the
     // count for the next launch
     if (blockIdx.x == 0 && tid == 0) v.bar[0] = target;
+    leave();
 }
 
 template <int TU>

@@ -459,25 +459,35 @@ bp_status bp_update(bp_net* net, void* stream) {
 static bp_status run_epoch(bp_net* net, const void* d_X, const void* d_T, int n_patterns,
                            int minibatch, float* d_sse, cudaStream_t s) {
     const int n_steps = (int)(((long long)n_patterns + minibatch - 1) / minibatch);
-    if (net->dtype == BP_F32 && !net->g_dirty && f32_cluster_ok(net->view, minibatch)) {
-        // groups of a few patterns of a one-hidden-layer net: one cluster keeps the net on chip
-        BP_CUDA(f32_train_cluster(net->view, (const float*)d_X, (const float*)d_T, n_patterns,
-                                  minibatch, n_steps, d_sse, s),
-                "training launch");
-    } else if (net->dtype == BP_F32 && !net->g_dirty && f32_small_ok(net->view, minibatch)) {
-        // groups of a few patterns: one CTA keeps the weights resident
-        BP_CUDA(f32_train_small(net->view, (const float*)d_X, (const float*)d_T, n_patterns,
-                                minibatch, n_steps, d_sse, s),
-                "training launch");
-    } else if (net->dtype == BP_F32 && f32_large_ok(net->view, minibatch, net->num_sms)) {
-        BP_CUDA(f32_train_large(net->view, (const float*)d_X, (const float*)d_T, n_patterns, minibatch,
-                                n_steps, d_sse, net->g_dirty, net->num_sms, s),
-                "training launch");
-    } else if (net->dtype == BP_F32) {
-        const F32Plan plan = f32_plan(net->view, minibatch, net->num_sms);
-        BP_CUDA(f32_train(net->view, (const float*)d_X, (const float*)d_T, n_patterns, minibatch,
-                          n_steps, d_sse, net->g_dirty, plan, s),
-                "training launch");
+    if (net->dtype == BP_F32) {
+        const F32View& v = net->view;
+        const float *X = (const float*)d_X, *T = (const float*)d_T;
+        auto grid = [&](const float* x, const float* t, int n, int steps, float* sse, bool fold) {
+            return f32_train(v, x, t, n, minibatch, steps, sse, fold, f32_plan(v, minibatch, net->num_sms), s);
+        };
+        switch (f32_route(v, minibatch, n_patterns, net->num_sms, net->g_dirty, v.gpart != nullptr)) {
+            case kRouteCluster:   // one cluster keeps the net on chip
+                BP_CUDA(f32_train_cluster(v, X, T, n_patterns, minibatch, n_steps, d_sse, s), "training launch");
+                break;
+            case kRouteSmall:   // one CTA keeps the weights resident
+                BP_CUDA(f32_train_small(v, X, T, n_patterns, minibatch, n_steps, d_sse, s), "training launch");
+                break;
+            case kRouteLarge: {
+                // a last group too short for this kernel takes the grid-wide one (f32_route)
+                const int last = n_patterns % minibatch, rest = last < kLargeMinPerCta * net->num_sms ? last : 0;
+                const int n = n_patterns - rest, steps = n_steps - (rest > 0 ? 1 : 0);
+                BP_CUDA(f32_train_large(v, X, T, n, minibatch, steps, d_sse, net->g_dirty, net->num_sms, s),
+                        "training launch");
+                if (rest > 0)
+                    BP_CUDA(grid(X + (size_t)n * v.n[0], T + (size_t)n * v.n[v.L], rest, 1,
+                                 d_sse != nullptr ? d_sse + steps : nullptr, false),
+                            "training launch");
+                break;
+            }
+            case kRouteGrid:
+                BP_CUDA(grid(X, T, n_patterns, n_steps, d_sse, net->g_dirty), "training launch");
+                break;
+        }
     } else {
         BP_CUDA(bf16_train(net->bf, d_X, d_T, n_patterns, minibatch, d_sse, net->lr, net->momentum,
                            net->grad_scale, net->g_dirty, s),
@@ -625,6 +635,16 @@ bp_status bp_train_epoch_host(bp_net* net, const void* h_X, const void* h_T, int
 }
 
 }  // extern "C"
+
+// For the tests (not part of the ABI): the kernel that a training call of a float32 net takes
+// (F32Route), from its sizes alone; calls nothing of CUDA.  -1: a size that bp_create refuses.
+extern "C" int bp_internal_f32_route(const int* sizes, int n_layers, int minibatch, int n_patterns, int num_sms,
+                                     int pending) {
+    if (n_layers < 2 || n_layers > BP_MAX_SIZES || f32_max_pg(sizes, n_layers - 1) < 1) return -1;
+    F32View v{};
+    f32_layout(v, sizes, n_layers - 1, minibatch);
+    return (int)f32_route(v, minibatch, n_patterns, num_sms, pending != 0, true);
+}
 
 namespace bp {
 // Lets other translation units report a message through bp_last_error().

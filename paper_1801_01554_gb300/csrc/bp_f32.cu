@@ -1782,6 +1782,17 @@ cudaError_t f32_train_small(const F32View& v, const float* X, const float* T, in
     return cudaGetLastError();
 }
 
+// Small groups by `minibatch` (their kernels hold that many patterns); large ones by the
+// patterns there are: a pass of the large-group kernel costs the same however few rows it has
+// (100 patterns of 203-60-26 with a minibatch of 8,192: 56 us there, 20 on the grid-wide kernel).
+F32Route f32_route(const F32View& v, int minibatch, int n_patterns, int num_sms, bool pending, bool large_sums) {
+    if (!pending && f32_cluster_ok(v, minibatch)) return kRouteCluster;
+    if (!pending && f32_small_ok(v, minibatch)) return kRouteSmall;
+    if (large_sums && std::min(minibatch, n_patterns) >= kLargeMinPerCta * num_sms && f32_large_shape_ok(v))
+        return kRouteLarge;
+    return kRouteGrid;
+}
+
 // ------------------------------------------------------------ diagnostic mode
 cudaError_t f32_diagnose(const F32View& v, const float* X, const float* T, int batch, float* d_sse,
                          int* d_sm, int num_sms, cudaStream_t s) {

@@ -617,12 +617,6 @@ bool f32_large_shape_ok(const F32View& v) {
     return large_tu(v, c) != 0;
 }
 
-bool f32_large_ok(const F32View& v, int minibatch, int num_sms) {
-    LargePlan c;
-    if (v.gpart == nullptr || minibatch < kLargeMinPerCta * num_sms) return false;
-    return large_tu(v, c) != 0;
-}
-
 cudaError_t f32_train_large(const F32View& v, const float* X, const float* T, int n_patterns, int minibatch,
                             int n_steps, float* sse_out, bool fold_g, int num_sms, cudaStream_t s) {
     LargePlan c;

@@ -154,8 +154,7 @@ cudaError_t f32_train_cluster(const F32View& v, const float* X, const float* T, 
                               int minibatch, int n_steps, float* sse_out, cudaStream_t s);
 
 // Large groups of a one-hidden-layer net (bp_f32_large.cu): each CTA keeps its sums
-// in registers; needs v.gpart of num_sms * P floats.  f32_large_shape_ok: the net
-// fits; f32_large_ok: and the group is worth it.
+// on chip; needs v.gpart of num_sms * P floats.  f32_large_shape_ok: the net fits.
 // Patterns per CTA from which one pass (64 or 128 patterns, mostly fixed time: 45 us
 // at 203-120-26, 46 at 203-60-26) beats the tiled weight phase: 6,100 patterns take
 // 45.2 against 46.1 us at 203-120-26, 46.4 against 51.2 at 203-60-26; 4,096 take 29.1
@@ -163,9 +162,14 @@ cudaError_t f32_train_cluster(const F32View& v, const float* X, const float* T, 
 constexpr int kLargeMinPerCta = 40;
 cudaError_t f32_large_setup();
 bool f32_large_shape_ok(const F32View& v);
-bool f32_large_ok(const F32View& v, int minibatch, int num_sms);
 cudaError_t f32_train_large(const F32View& v, const float* X, const float* T, int n_patterns, int minibatch,
                             int n_steps, float* sse_out, bool fold_g, int num_sms, cudaStream_t s);
+
+// The kernel that trains groups of `minibatch` patterns of a set of n_patterns.
+enum F32Route { kRouteCluster, kRouteSmall, kRouteLarge, kRouteGrid };
+// pending: a pooled change of bp_backward waits to be added; large_sums: the per-CTA sums
+// of the large-group kernel are there.
+F32Route f32_route(const F32View& v, int minibatch, int n_patterns, int num_sms, bool pending, bool large_sums);
 
 // Diagnostic mode (Section 8): num_sms CTAs each run the forward pass and error
 // of all `batch` patterns; per-CTA error sums to d_sse, SM ids to d_sm.

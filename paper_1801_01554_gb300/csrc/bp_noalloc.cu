@@ -151,9 +151,10 @@ extern "C" bp_status bp_train_epoch_noalloc(const int* layer_sizes, int n_layers
     // must start at zero
     cudaError_t e = f32_pad_device(v, d_theta, d_V, reinterpret_cast<unsigned*>(base), 4 + (int)bar_words, s);
     const int n_steps = (int)(((long long)n_patterns + minibatch - 1) / minibatch);
-    if (e == cudaSuccess && f32_cluster_ok(v, minibatch)) {
+    const F32Route route = f32_route(v, minibatch, n_patterns, sms, false, false);
+    if (e == cudaSuccess && route == kRouteCluster) {
         e = f32_train_cluster(v, d_X, d_T, n_patterns, minibatch, n_steps, d_sse, s);
-    } else if (e == cudaSuccess && f32_small_ok(v, minibatch)) {
+    } else if (e == cudaSuccess && route == kRouteSmall) {
         e = f32_train_small(v, d_X, d_T, n_patterns, minibatch, n_steps, d_sse, s);
     } else if (e == cudaSuccess) {
         const F32Plan plan = f32_plan(v, minibatch, sms);

@@ -72,3 +72,24 @@ def test_error_of_the_changes_of_large_groups(sizes, B, bar):
     d2 = (T.double() - o) * o * (1 - o)
     ref = (((d2 @ W2) * h * (1 - h)).T @ X.double()).flatten()
     assert float((V[:n0 * H] - ref).norm() / ref.norm()) <= bar
+
+
+@pytest.mark.parametrize("sizes,n,mb", [((203, 60, 26), 100, 8192), ((203, 60, 26), 2 * 6080 + 1, 6080),
+                                        ((64, 50, 10), 6079, 16384), ((203, 120, 26), 6080 + 6079, 6080)])
+def test_short_groups_take_the_grid_wide_kernel_step_by_step(sizes, n, mb):
+    """Fewer patterns than a pass is worth, in all or in the last group; the first of them
+    with a pending change."""
+    X, T, theta = problem(sizes, n, seed=44)
+    stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.002, 0.9)
+    st = O.State(sizes, theta, lr=0.002, momentum=0.9)
+    with bp.Net(sizes, 0.002, 0.9, bp.BP_F32, max_batch=mb) as net:
+        net.set_weights(theta)
+        Xd, Td = dev(X), dev(T)
+        net.forward(Xd, 64)
+        net.backward(Td, 64)
+        net.train_epoch(Xd, Td, n, mb)
+        net.check()
+        O.backward_accumulate(st, X[:64], T[:64])
+        O.train_epoch(st, X, T, mb)
+        np.testing.assert_allclose(net.get_weights(), st.theta, rtol=0, atol=1e-5 * np.max(np.abs(st.theta)))
+        np.testing.assert_array_equal(net.get_grads(), 0.0)

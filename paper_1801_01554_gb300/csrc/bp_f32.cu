@@ -429,13 +429,31 @@ __device__ __forceinline__ void forward_any(const float* W, int kp, int n_out, c
 // Hidden deltas of layer l for PG patterns: d_l[p][i] = (sum_j W_{l+1}[j][i]
 // d_{l+1}[p][j]) a_l[p][i] (1 - a_l[p][i]), summed over the next layer's units in
 // order.  One thread per unit sums all PG patterns, so that a weight and one read of
-// the PG deltas feed PG multiply-adds (a thread per pattern and unit read both for
+// the PG deltas feed PG multiply-adds (a thread per pattern and unit reads both for
 // each one: 11.7 us per update at groups of 512 of 203-120-26 and 25.1 at 2,000,
-// against 11.6 and 24.0).  dnt holds d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl,
-// pitch dpl) and, if dlt is not null, pattern-minor (dlt).
+// against 11.6 and 24.0); where that leaves most threads without work, up to kPairs
+// patterns times units, one thread each (the same sums).  us per update, one per unit / one
+// each: 8-4-900 by 5,000 181 / 158, 100-10-500 by 2,000 51.1 / 45.9, 500-30-30-500 by 1,000
+// (240) 33.6 / 32.0; past the line 100-62-100 by 2,000 (496) 26.3 / 27.5.  dnt holds
+// d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl, pitch dpl) and, if dlt is not
+// null, pattern-minor (dlt).
+constexpr int kPairs = 256;   // half of the threads
 template <int PG>
 __device__ void hidden_delta(const float* Wn, int kpn, int n, int nn, const float* dnt,
                              const float* al, int apl, float* dl, int dpl, float* dlt) {
+    if (PG > 1 && n * PG <= kPairs) {
+        for (int e = threadIdx.x; e < PG * n; e += kThreads) {
+            const int p = e / n, i = e - p * n;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int j = 0; j < nn; ++j) acc = fmaf(dnt[j * PG + p], Wn[(size_t)j * kpn + i], acc);
+            const float a = al[p * apl + i];
+            const float d = acc * a * (1.f - a);
+            dl[p * dpl + i] = d;
+            if (dlt != nullptr) dlt[i * PG + p] = d;
+        }
+        return;
+    }
     for (int i = threadIdx.x; i < n; i += kThreads) {
         float acc[PG];
 #pragma unroll

@@ -636,3 +636,12 @@ def test_nettalk120_workload_full():
         O.train_epoch(st, X, T, mb)
     print("640-update trajectory, W-W0 per part:", layer_errors(sizes, W - theta, st.theta - theta),
           "V per part:", layer_errors(sizes, V, st.V))
+
+
+@pytest.mark.parametrize("sizes,n,mb", [((20, 8, 60), 1216, 1216), ((100, 32, 40), 1100, 1100),
+                                        ((100, 33, 40), 1100, 1100), ((9, 1, 70), 700, 304), ((16, 64, 20), 600, 304)])
+def test_hidden_deltas_of_few_and_many_units_step_by_step(sizes, n, mb):
+    """Both sides of the line between a thread per pattern and unit and a thread per unit (256
+    pairs: 32 units at 8 patterns a pass, 64 at 4), and a single hidden unit."""
+    X, T, theta = problem(sizes, n, seed=92)
+    stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.002, 0.9)

@@ -272,9 +272,11 @@ bp_status bp_train_epoch_noalloc(const int* layer_sizes, int n_layers, float lr,
  * time; unreachable == 2 makes the first chunk copy of each CTA's weight phase
  * a copy that never comes (its barrier is armed for the bytes, no copy is
  * issued), so that the chunk waits run out; large groups, which run without
- * chunks, wait for weights of which some bytes never come.  Either way the launch latches the timeout,
- * every CTA returns with every copy it issued landed and no update applied,
- * and bp_check reports BP_ETIMEOUT and resets the barrier; 0 turns both off.
+ * chunks, wait for weights of which some bytes never come, and groups of 1-4
+ * on a cluster for sums of its CTAs (they have no grid barrier to stall).
+ * Either way the launch latches the timeout, every CTA returns with every copy
+ * it issued landed and no update applied, and bp_check reports BP_ETIMEOUT and
+ * resets the barrier; 0 turns both off.
  * Synchronises the device.  Errors: BP_EINVAL (NULL, a BP_BF16 net),
  * BP_ESTATE (a library built without BP_CHECK: the hook does nothing there),
  * BP_ECUDA. */

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
     const float lr = v.lr * v.grad_scale, mom = v.momentum, guard = v.guard;
     const bool table = v.sig_table != 0;
     unsigned n_bad = 0;
+    const int latched = __ldcg(v.flags);   // nothing in this launch latches a timeout before the cluster's barrier
     sigmoid_table_init(v);
 
     // weights: W_1 rows to registers, W_2 columns and b_2 to shared memory
@@ -165,10 +166,19 @@ __global__ void __launch_bounds__(kCThreads, 1)
         for (int k = 0; k < kStagesX - 1; ++k) load_next();
         cp_async_wait<kStagesX - 2>();
     }
+    // a latched timeout: nothing is trained until bp_check has cleared it (every CTA returns)
+    if (latched & kFlagTimeout) {
+        cp_async_wait<0>();
+        return;
+    }
     cluster_barrier();   // every CTA of the cluster has started; its shared memory is set up
 
     if (tid == 0) {
-        arm(s_bar, C * n2 * PG * 4);
+        unsigned lost = 0;
+#ifdef BP_CHECK
+        lost = v.debug_stall != 0 ? 16u : 0u;   // test hook: the first exchange waits for bytes that never come
+#endif
+        arm(s_bar, C * n2 * PG * 4 + lost);
         arm(s_bar + 1, C * n2 * PG * 4);
     }
     int stage = 0, buf = 0;
@@ -249,7 +259,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
         }
         if (loader) cp_async_wait<kStagesX - 3>();   // the next pass's rows
         ok = __syncthreads_and(ok) != 0;
-        if (!ok) break;   // a peer's sums did not arrive: no update, wait for the peers below
+        if (!ok) break;   // a peer's sums did not arrive
         // 4. hidden deltas and the changes of this lane's weights
         if (tid < c.uthr) {
             float hv[PG], a[PG];
@@ -353,9 +363,15 @@ __global__ void __launch_bounds__(kCThreads, 1)
         parity ^= buf == 0 ? 1u : 0u;
     }
     cp_async_wait<0>();
+    // No CTA sends anything after this barrier, so that a CTA whose sums all came may leave; one
+    // whose wait ran out gives the missing ones as long again to land in its shared memory.
+    cluster_barrier();
+    if (!ok) wait_bytes(s_bar + buf, parity, v.flags, wait_limit_ns(v));
+    // A wait that ran out in one CTA leaves the others an update ahead: then none writes
+    // back, and the weights are those before the launch.
+    if (__ldcg(v.flags) & kFlagTimeout) return;
     if (n_bad != 0) atomicAdd(v.faults, n_bad);
-    // weights and weight changes back to global memory (after a wait that ran out:
-    // those of the updates so far)
+    // weights and weight changes back to global memory
 #pragma unroll
     for (int j = 0; j < 2 * KC4; ++j) {
         const int col = 4 * (s + S * (j >> 1)) + 2 * (j & 1);
@@ -369,7 +385,6 @@ __global__ void __launch_bounds__(kCThreads, 1)
             v.V[row1 + col + 1] = vj.y;
         }
     }
-    __syncthreads();   // the last pass's shared-memory updates
     for (int e = tid; e < n2 * nu; e += nthr) {
         const int k = e / nu, u = e - k * nu;
         const long long g = v.woff[2] + (long long)k * v.kp[2] + u0 + u;
@@ -382,7 +397,6 @@ __global__ void __launch_bounds__(kCThreads, 1)
             v.theta[g] = sm[c.b2 + k];
             v.V[g] = sm[c.vb2 + k];
         }
-    cluster_barrier();   // no CTA leaves while a peer may still address its shared memory
 }
 
 // Largest group.  us per update of 203-120-26, one-CTA kernel -> this one: 6.76 -> 2.2

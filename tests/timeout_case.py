@@ -3,8 +3,9 @@ build named on the command line (argv: library, "barrier" or "chunk", case
 name): makes a wait of a training launch run out of time with a 1 ms limit,
 either its first grid barrier (a count that no CTA will reach) or the first
 chunk of each CTA's weight phase (a copy that never comes: the barrier is armed,
-no copy is issued), then trains the same epoch normally, and prints what
-happened as JSON.
+no copy is issued; in kernels without chunks, bytes that never come of the first weight
+copy or exchange), then trains the same epoch normally, and prints what happened as
+JSON.
 
 No GPU fault is involved: every wait is bounded, the kernel latches the
 timeout and every CTA returns with every copy it issued landed."""
@@ -24,7 +25,8 @@ from paper_1801_01554_gb300 import bp, synth  # noqa: E402
 bp.load(sys.argv[1])
 MODE = sys.argv[2] if len(sys.argv) > 2 else "barrier"
 CASES = {"nettalk120_512": ((203, 120, 26), 2048, 512),      # whole-tile weight phase
-         "nettalk60_12288": ((203, 60, 26), 24576, 12288)}   # balanced weight phase
+         "nettalk60_12288": ((203, 60, 26), 24576, 12288),   # large groups: the copy of the weights
+         "nettalk120_4": ((203, 120, 26), 24, 4)}            # one cluster: the exchange of the CTAs' sums
 sizes, n, mb = CASES[sys.argv[3] if len(sys.argv) > 3 else "nettalk120_512"]
 X, T = synth.nettalk_patterns(n, seed=71)
 theta = synth.round_to(synth.init_uniform(sizes, -0.3, 0.3, 71), "f32")

@@ -1710,7 +1710,14 @@ cudaError_t bf16_refresh_weights(Bf16Net* b, cudaStream_t s) {
 }
 
 cudaError_t bf16_forward(Bf16Net* b, const void* X, int batch, void* Y, cudaStream_t s) {
-    return run_forward(b, (const bf16*)X, batch, nullptr, (bf16*)Y, s);
+    // One layer: tiles still read rows of X that others have written to Y, so a Y that overlaps
+    // X is copied to at the end.  (With more layers X is read before the last one writes.)
+    const size_t nx = (size_t)batch * b->n[0] * sizeof(bf16), ny = (size_t)batch * b->n[b->L] * sizeof(bf16);
+    const uintptr_t x = (uintptr_t)X, y = (uintptr_t)Y;
+    if (b->L > 1 || Y == nullptr || y + ny <= x || x + nx <= y)
+        return run_forward(b, (const bf16*)X, batch, nullptr, (bf16*)Y, s);
+    const cudaError_t e = run_forward(b, (const bf16*)X, batch, nullptr, nullptr, s);
+    return e != cudaSuccess ? e : cudaMemcpyAsync(Y, b->act[b->L], ny, cudaMemcpyDeviceToDevice, s);
 }
 
 cudaError_t bf16_backward(Bf16Net* b, const void* X, const void* T, int batch, float* sse,

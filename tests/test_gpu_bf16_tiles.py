@@ -129,3 +129,19 @@ def test_chains_of_two_layers_in_one_launch():
     d1 = (d2 @ W2) * h * (1 - h)
     for got, ref in ((V[:nw], d1.T @ X.double()), (V[nw + sizes[1]:-sizes[2]], d2.T @ h)):
         assert normwise(got.double().cpu().numpy(), ref.flatten().cpu().numpy()) <= TOL
+
+
+@pytest.mark.parametrize("n,B,shift", [(2048, 8192, 0), (768, 20000, 0), (512, 20000, 640)])
+def test_forward_of_one_layer_may_write_over_its_input(n, B, shift):
+    """Y may be X itself, or overlap it by rows (a square one-layer net), also where the tiles
+    of a row block run in different waves: the outputs of a call with a buffer of its own."""
+    X, _, theta = problem((n, n), B, seed=53)
+    buf = torch.zeros((B + shift, n), dtype=torch.bfloat16, device="cuda")
+    buf[:B] = dev_bf16(X)
+    Y = torch.empty((B, n), dtype=torch.bfloat16, device="cuda")
+    with bp.Net((n, n), 0.01, 0.9, bp.BP_BF16, max_batch=B) as net:
+        net.set_weights(theta)
+        net.forward(buf[:B], B, Y)
+        net.forward(buf[:B], B, buf[shift:])
+        net.check()
+    assert torch.equal(buf[shift:], Y)

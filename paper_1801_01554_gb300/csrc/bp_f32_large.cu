@@ -28,8 +28,12 @@
 // registers that layer 1's two levels of sums need (kept in registers, W_1's sums made it
 // spill and cost a fifth); adding to them there takes about 700 clocks for TU = 8.
 // us per update, tiled weight phase (k_train) -> this kernel: 203-120-26 at groups of
-// 8,192: 52.8 -> 46, 16,384: 103.5 -> 80, 65,536: 349 -> 243; 203-60-26 at 65,536:
-// 391 -> 162; 64-50-10: 140 -> 88.
+// 8,192: 52.8 -> 45.1, 16,384: 103.5 -> 76.7, 65,536: 349 -> 242; 203-60-26 at 65,536:
+// 391 -> 157; 64-50-10: 140 -> 88.  The changes run over the rows a pass has: 9,729 patterns, a
+// second pass of one row, take 67 us (79 when it summed 64), 11,777 of 203-90-26 68 (75; tiled 71).
+//
+// Which nets: one block of each product per thread (plan_tu), for 203 inputs up to 120 hidden
+// units, for 255 up to 88; wider ones keep the tiled weight phase.
 #include <cuda_runtime.h>
 
 #include "bp_f32_device.cuh"
@@ -213,6 +217,7 @@ __global__ void __launch_bounds__(kT, 1)
         bool have_w = false, ok = true;
         for (long long p0 = lo; p0 < hi || !have_w; p0 += P) {
             const int np = (int)max(0LL, min((long long)P, hi - p0));
+            const int np4 = (np + 3) & ~3;   // rows that the sums of changes run over
             // rows of this pass; those past the share are zero
             for (int r = warp; r < P; r += kT / 32) {
                 float* dst = sm + c.x + r * xp;
@@ -380,14 +385,14 @@ __global__ void __launch_bounds__(kT, 1)
             if (w2c) {
                 const float* dr = sm + c.d + 4 * kr2;
                 const float* hr = sm + c.h + 4 * cg2;
-                for (int pc = 0; pc < P; pc += kChain) {
+                for (int pc = 0; pc < np4; pc += kChain) {
                     float l2[4][4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
 #pragma unroll
                         for (int q = 0; q < 4; ++q) l2[u][q] = 0.f;
 #pragma unroll 4
-                    for (int p = pc; p < pc + kChain; ++p) {
+                    for (int p = pc; p < min(pc + kChain, np4); ++p) {
                         const float4 d = ld4(dr + p * dp), h = ld4(hr + p * hp);
                         const float dv[4] = {d.x, d.y, d.z, d.w}, hx[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
@@ -420,21 +425,21 @@ __global__ void __launch_bounds__(kT, 1)
             {
                 const float* dr = sm + c.h + TU * ur1;
                 const float* xr = sm + c.x + 12 * cg1;
-                for (int pm = 0; pm < P; pm += kMerge) {
+                for (int pm = 0; pm < np4; pm += kMerge) {
                     f32x2 g1[TU][6];   // sums of kMerge patterns, pairs of columns
 #pragma unroll
                     for (int u = 0; u < TU; ++u)
 #pragma unroll
                         for (int q = 0; q < 6; ++q) g1[u][q] = 0;
                     if (w1c)
-                        for (int pc = pm; pc < pm + kMerge; pc += kChain) {
+                        for (int pc = pm; pc < min(pm + kMerge, np4); pc += kChain) {
                             f32x2 l1[TU][6];   // of one chain
 #pragma unroll
                             for (int u = 0; u < TU; ++u)
 #pragma unroll
                                 for (int q = 0; q < 6; ++q) l1[u][q] = 0;
 #pragma unroll 2
-                            for (int p = pc; p < pc + kChain; ++p) {
+                            for (int p = pc; p < min(pc + kChain, np4); ++p) {
                                 f32x2 xv[6];
 #pragma unroll
                                 for (int q = 0; q < 3; ++q) {

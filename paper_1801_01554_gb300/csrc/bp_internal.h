@@ -155,10 +155,10 @@ cudaError_t f32_train_cluster(const F32View& v, const float* X, const float* T, 
 
 // Large groups of a one-hidden-layer net (bp_f32_large.cu): each CTA keeps its sums
 // on chip; needs v.gpart of num_sms * P floats.  f32_large_shape_ok: the net fits.
-// Patterns per CTA from which one pass (64 or 128 patterns, mostly fixed time: 45 us
-// at 203-120-26, 46 at 203-60-26) beats the tiled weight phase: 6,100 patterns take
-// 45.2 against 46.1 us at 203-120-26, 46.4 against 51.2 at 203-60-26; 4,096 take 29.1
-// and 36.7 in the tiled form.
+// Patterns per CTA from which one pass (64 or 128 patterns, whatever its rows: they
+// shorten the sums of changes only) beats the tiled weight phase.  us per update, 6,079
+// patterns (tiled) / 6,080: 203-120-26 48.2 / 42.1, 203-60-26 47.5 / 37.9, 64-50-10
+// 31.3 / 21.6; a pass of 203-120-26 takes 36 at the least, 4,096 patterns 29.7 tiled.
 constexpr int kLargeMinPerCta = 40;
 cudaError_t f32_large_setup();
 bool f32_large_shape_ok(const F32View& v);

@@ -1,8 +1,8 @@
 """Run by tests/test_gpu_checked.py in a fresh process: loads the library named
 on the command line and prints, as JSON, the results of a few training runs
-that go through every float32 kernel (persistent training with whole-tile and
-balanced weight phases, one-CTA groups, forward/backward/update, the
-allocation-free entry point, diagnostic mode)."""
+that go through every float32 kernel (grid-wide training with whole-tile and
+balanced weight phases, cluster, one-CTA and large groups, forward/backward/update,
+the allocation-free entry point, diagnostic mode)."""
 import json
 import os
 import sys
@@ -23,9 +23,11 @@ def dev(a):
 
 
 out = {}
-# the last case runs two groups of 24 chunks (the balanced weight phase) and a ragged third
+# the last two cases run two groups of 24 chunks and a ragged third: the large-group kernel,
+# whose short last group takes the grid-wide one, and the balanced weight phase
 for sizes, n, mb in (((203, 120, 26), 1100, 512), ((203, 60, 26), 40, 2), ((64, 33, 17, 9), 300, 300),
-                     ((7, 9, 5, 11, 6, 8, 4, 10, 3), 66, 33), ((203, 60, 26), 26000, 12288)):
+                     ((64, 33, 17, 9), 41, 2), ((7, 9, 5, 11, 6, 8, 4, 10, 3), 66, 33),
+                     ((203, 60, 26), 26000, 12288), ((203, 60, 30, 26), 26000, 12288)):
     X, T = synth.gaussian_patterns(n, sizes[0], sizes[-1], 0.3, seed=3)
     theta = synth.round_to(synth.init_uniform(sizes, -0.5, 0.5, 3), "f32")
     key = "-".join(map(str, sizes)) + f"/{mb}"

@@ -49,12 +49,13 @@ def test_checked_build_passes_its_checks_and_matches(checked_lib):
 
 
 @pytest.mark.parametrize("mode,case", [("barrier", "nettalk120_512"), ("chunk", "nettalk120_512"),
-                                       ("chunk", "nettalk60_12288"), ("chunk", "nettalk120_4")])
+                                       ("chunk", "nettalk60_12288"), ("chunk", "deeper_12288"),
+                                       ("chunk", "nettalk120_4")])
 def test_wait_that_runs_out_is_reported_and_recovered(checked_lib, mode, case):
     """Section 8's failure detection without a fault, with a 1 ms limit: either
     the first grid barrier of a training launch waits for a count no CTA
     reaches, or the first chunk copy of every CTA's weight phase never comes
-    (whole-tile weight phase), or bytes of the first weight copy (large groups) or of the
+    (whole-tile and balanced weight phases), or bytes of the first weight copy (large groups) or of the
     first exchange (groups on a cluster).  The launch latches the timeout
     and no update is applied; bp_check reports BP_ETIMEOUT, clears the latch
     and resets the barrier; the next epoch on the same net matches the oracle
@@ -68,6 +69,7 @@ def test_wait_that_runs_out_is_reported_and_recovered(checked_lib, mode, case):
     assert r["seconds"] < 1.0          # the 1 ms limit, not the default 2 s
     sizes, n, mb = {"nettalk120_512": ((203, 120, 26), 2048, 512),
                     "nettalk60_12288": ((203, 60, 26), 24576, 12288),
+                    "deeper_12288": ((203, 60, 30, 26), 24576, 12288),
                     "nettalk120_4": ((203, 120, 26), 24, 4)}[case]
     X, T = synth.nettalk_patterns(n, seed=71)
     theta = synth.round_to(synth.init_uniform(sizes, -0.3, 0.3, 71), "f32")

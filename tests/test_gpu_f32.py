@@ -185,8 +185,8 @@ def test_train_batch_matches_oracle(sizes, B):
 
 @pytest.mark.parametrize("B,lr", [(200, 0.1), (12288, 0.01)])
 def test_pending_change_is_folded_into_train_batch(B, lr):
-    """bp_backward's pending G is added into the next training update; at
-    B = 12,288 (24 chunks) the update runs in the balanced weight phase."""
+    """bp_backward's pending G is added into the next training update, by the grid-wide
+    kernel (B = 200) and by the large-group kernel (B = 12,288)."""
     sizes = (203, 60, 26)
     X, T, theta = problem(sizes, B, seed=4)
     X2, T2, _ = problem(sizes, B, seed=5)
@@ -247,17 +247,60 @@ def test_weights_beyond_shared_memory_at_large_groups_step_by_step():
     stepwise(sizes, X, T, theta, np.zeros_like(theta), 4096, 0.01, 0.9)
 
 
-# Groups of at least 24 chunks of 512 patterns, on nets with fewer weight tiles
-# than SMs, run the balanced weight phase: each CTA takes an equal run of the
-# tiles' chunk sequence and the pieces are added in CTA order after a grid
-# barrier.  Cases: two balanced groups then a ragged one of 12 chunks in the
-# same launch; a 2-tile net (fewer chunks than CTAs, so some runs are empty);
-# exactly 24 chunks.
+# Groups of 24 chunks of 512 patterns and more.  One-hidden-layer nets of these sizes
+# run on the large-group kernel; the first and second case end in a short group, which
+# the grid-wide kernel trains (12 whole-tile chunks, one chunk).
 @pytest.mark.parametrize("sizes,n,mb", [((203, 120, 26), 30000, 12288), ((20, 8, 3), 25500, 12500),
                                         ((203, 60, 26), 24576, 12288)])
 def test_balanced_weight_phase_matches_oracle_step_by_step(sizes, n, mb):
     X, T, theta = problem(sizes, n, seed=71)
     stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.02, 0.9)
+
+
+# The balanced weight phase: groups of at least 24 chunks on nets with fewer weight tiles than
+# SMs and more than one hidden layer, or too many units for the large-group kernel.  Each
+# CTA takes an equal run of the tiles' chunk sequence and the pieces are added in CTA order
+# after a grid barrier.  Cases: two balanced groups then a ragged one of 12 chunks in the same
+# launch; a 3-tile net (fewer chunks than CTAs, so some runs are empty); exactly 24 chunks.
+BALANCED = [((203, 60, 30, 26), 30000, 12288), ((20, 8, 6, 3), 25500, 12500), ((203, 128, 26), 24576, 12288)]
+
+
+@pytest.mark.parametrize("sizes,n,mb", BALANCED)
+def test_balanced_weight_phase_of_other_nets_step_by_step(sizes, n, mb):
+    X, T, theta = problem(sizes, n, seed=71)
+    stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.005, 0.9)
+
+
+def test_pending_change_and_guard_in_the_balanced_weight_phase():
+    """On a two-hidden-layer net: bp_backward's G folded into the update, then an update whose
+    guard zeroes and counts the oracle's changes."""
+    sizes, B = (203, 60, 30, 26), 12288
+    X, T, theta = problem(sizes, B, seed=72)
+    kap = kappa(sizes, theta, X, T)
+    st = O.State(sizes, theta, lr=0.002, momentum=0.5)
+    with bp.Net(sizes, 0.002, 0.5, bp.BP_F32, max_batch=B) as net:
+        net.set_weights(theta)
+        Xd, Td = dev(X), dev(T)
+        net.forward(Xd, B)
+        net.backward(Td, B)
+        net.train_batch(Xd, Td, B)
+        net.check()
+        O.backward_accumulate(st, X, T)
+        O.train_batch(st, X, T)
+        check_state(sizes, theta, net.get_weights(), net.get_velocity(), st, kap, "folded")
+        assert not net.get_grads().any()
+    probe = O.State(sizes, theta, lr=0.002, momentum=0.9)
+    O.backward_accumulate(probe, X, T)
+    guard = _gap_threshold(probe.G)
+    st = O.State(sizes, theta, lr=0.002, momentum=0.9, guard=guard)
+    O.train_batch(st, X, T)
+    with bp.Net(sizes, 0.002, 0.9, bp.BP_F32, max_batch=B) as net:
+        net.set_weights(theta)
+        net.set_guard(guard)
+        net.train_batch(Xd, Td, B)
+        net.check()
+        assert net.get_faults() == st.faults > 0
+        check_state(sizes, theta, net.get_weights(), net.get_velocity(), st, kap, "guarded")
 
 
 @pytest.mark.parametrize("sizes,n,mb,lr", [((203, 120, 26), 777, 1, 0.05), ((203, 120, 26), 300, 1, 0.05),
@@ -327,9 +370,18 @@ def test_table_sigmoid_matches_oracle(sizes, n, mb):
 
 @pytest.mark.parametrize("sizes,n,mb", [((203, 60, 26), 300, 1), ((203, 60, 26), 301, 4)])
 def test_table_sigmoid_on_small_groups_step_by_step(sizes, n, mb):
-    """The table-lookup logistic on the one-CTA kernel, update by update."""
+    """The table-lookup logistic on the cluster kernel, update by update."""
     X, T, theta = problem(sizes, n, seed=31, lo=-1.0, hi=1.0)
     stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.05, 0.9, squash="table")
+
+
+@pytest.mark.parametrize("mb", [1, 2, 4])
+def test_table_sigmoid_on_one_cta_step_by_step(mb):
+    """The table-lookup logistic on the one-CTA kernel (a deeper net)."""
+    sizes, n = (64, 33, 17, 9), 61
+    X, T, theta = problem(sizes, n, seed=31, lo=-1.0, hi=1.0)
+    stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.05, 0.9, squash="table")
+
 
 def test_table_sigmoid_mode_errors():
     with bp.Net((4, 3, 2), 0.1, 0.9, bp.BP_F32, max_batch=8) as net:
@@ -356,9 +408,9 @@ def _gap_threshold(G):
 
 @pytest.mark.parametrize("B", [512, 2, 16384])
 def test_fault_guard_matches_oracle(B):
-    """Section 8's guard on the persistent (B = 512), one-CTA (B = 2) and
-    balanced (B = 16,384) weight phases: the same changes are zeroed and
-    counted, the other weights update as usual."""
+    """Section 8's guard on the grid-wide (B = 512), cluster (B = 2) and large-group
+    (B = 16,384) kernels: the same changes are zeroed and counted, the other
+    weights update as usual."""
     sizes = (203, 120, 26)
     X, T, theta = problem(sizes, B, seed=41)
     probe = O.State(sizes, theta, lr=0.05, momentum=0.9)
@@ -374,6 +426,25 @@ def test_fault_guard_matches_oracle(B):
         assert net.get_faults(reset=True) == st.faults > 0
         assert net.get_faults() == 0
         check_state(sizes, theta, net.get_weights(), net.get_velocity(), st, None, "guarded")
+
+
+@pytest.mark.parametrize("B", [1, 2, 4])
+def test_fault_guard_on_one_cta_matches_oracle(B):
+    """The guarded instantiation of the one-CTA kernel (a deeper net)."""
+    sizes = (64, 33, 17, 9)
+    X, T, theta = problem(sizes, B, seed=41)
+    probe = O.State(sizes, theta, lr=0.05, momentum=0.9)
+    O.backward_accumulate(probe, X, T)
+    guard = _gap_threshold(probe.G)
+    st = O.State(sizes, theta, lr=0.05, momentum=0.9, guard=guard)
+    O.train_batch(st, X, T)
+    with bp.Net(sizes, 0.05, 0.9, bp.BP_F32, max_batch=B) as net:
+        net.set_weights(theta)
+        net.set_guard(guard)
+        net.train_batch(dev(X), dev(T), B)
+        net.check()
+        assert net.get_faults() == st.faults > 0
+        check_state(sizes, theta, net.get_weights(), net.get_velocity(), st, kappa(sizes, theta, X, T), "guarded")
 
 
 def test_fault_guard_on_backward_then_update_and_off_by_default():

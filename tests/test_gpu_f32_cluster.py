@@ -1,7 +1,8 @@
 """Groups of up to 4 patterns of one-hidden-layer nets on one cluster, against the
 float64 oracle update by update: every group size, ragged groups, 1 to 8 CTAs, CTAs without
 units, both row splits (4 and 7 float4 columns a lane) and the widest output
-layer; and the nets just past the limits, which other kernels take.  The bars
+layer (128 outputs, groups of 1); and the nets and groups just past the limits, which other
+kernels take (test_routes.py says which case runs where).  The bars
 are test_gpu_f32.py's (1e-5 of each sum's magnitude, plus the roundings of the
 stored weight changes)."""
 import numpy as np
@@ -14,12 +15,16 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("sizes,n,mb,lr", [
+CASES = [
     ((203, 120, 26), 23, 4, 0.05), ((203, 120, 26), 65, 3, 0.05), ((203, 120, 26), 70, 5, 0.05),
     ((203, 300, 26), 30, 1, 0.05), ((203, 300, 26), 45, 4, 0.05), ((203, 250, 26), 21, 2, 0.05),
     ((3, 1, 1), 9, 2, 0.05), ((17, 9, 3), 41, 4, 0.05), ((15, 33, 5), 33, 3, 0.05), ((16, 57, 7), 40, 4, 0.05),
     ((895, 90, 3), 12, 2, 0.02), ((511, 40, 100), 9, 1, 0.02), ((40, 20, 128), 10, 2, 0.02),
-    ((896, 20, 4), 6, 2, 0.02), ((40, 20, 129), 6, 1, 0.02), ((203, 120, 26), 40, 17, 0.05)])
+    ((896, 20, 4), 6, 2, 0.02), ((40, 20, 129), 6, 1, 0.02), ((203, 120, 26), 40, 17, 0.05),
+    ((40, 20, 128), 7, 1, 0.02)]
+
+
+@pytest.mark.parametrize("sizes,n,mb,lr", CASES)
 def test_cluster_groups_match_oracle_step_by_step(sizes, n, mb, lr):
     X, T, theta = problem(sizes, n, seed=31)
     V0 = synth.round_to(np.random.default_rng(4).uniform(-1e-3, 1e-3, theta.size), "f32")

@@ -1,9 +1,10 @@
-"""Large groups of one-hidden-layer nets, whose sums of changes stay in
-registers, against the float64 oracle update by update: both pass widths (64 and
-128 patterns), shares that end inside a pass, a ragged last group that leaves
-CTAs without patterns, layers that end inside a register block, even and odd row
-pitches; a pending change and the fault guard on this path; and a deeper net,
-which keeps the tiled (balanced) weight phase.  The bars are test_gpu_f32.py's."""
+"""Large groups of one-hidden-layer nets, whose sums of changes stay
+on chip, against the float64 oracle update by update: both pass widths (64 and
+128 patterns), shares that end inside a pass, groups that leave CTAs with fewer rows,
+layers that end inside a register block and at the largest numbers of hidden units
+that fit, even and odd row pitches; a pending change and the fault guard on this
+path; and nets past its limits and a deeper one, which keep the tiled (balanced) weight
+phase (test_routes.py says which case runs where).  The bars are test_gpu_f32.py's."""
 import numpy as np
 import pytest
 
@@ -15,10 +16,14 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("sizes,n,mb", [
+CASES = [
     ((203, 120, 26), 6100 + 37, 6100), ((203, 120, 26), 20000, 20000), ((203, 60, 26), 20500, 20000),
     ((203, 128, 26), 6500, 6500), ((203, 121, 3), 6200, 6200), ((17, 9, 3), 6300 + 1, 6300), ((40, 33, 40), 6400, 6400),
-    ((100, 1, 1), 6080, 6080), ((255, 57, 7), 6100, 6100), ((203, 60, 30, 26), 12500, 12300)])
+    ((100, 1, 1), 6080, 6080), ((255, 57, 7), 6100, 6100), ((203, 60, 30, 26), 12500, 12300),
+    ((203, 117, 26), 6200, 6200), ((203, 59, 26), 2 * 6200, 6200), ((255, 88, 7), 6100, 6100)]
+
+
+@pytest.mark.parametrize("sizes,n,mb", CASES)
 def test_large_groups_match_oracle_step_by_step(sizes, n, mb):
     X, T, theta = problem(sizes, n, seed=41)
     stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.002, 0.9)

@@ -26,6 +26,7 @@ bp.load(sys.argv[1])
 MODE = sys.argv[2] if len(sys.argv) > 2 else "barrier"
 CASES = {"nettalk120_512": ((203, 120, 26), 2048, 512),      # whole-tile weight phase
          "nettalk60_12288": ((203, 60, 26), 24576, 12288),   # large groups: the copy of the weights
+         "deeper_12288": ((203, 60, 30, 26), 24576, 12288),  # balanced weight phase
          "nettalk120_4": ((203, 120, 26), 24, 4)}            # one cluster: the exchange of the CTAs' sums
 sizes, n, mb = CASES[sys.argv[3] if len(sys.argv) > 3 else "nettalk120_512"]
 X, T = synth.nettalk_patterns(n, seed=71)

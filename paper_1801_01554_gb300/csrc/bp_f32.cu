@@ -1325,7 +1325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                           (int)min((long long)minibatch, (long long)n_patterns - pn), pat[(s + 1) & 1]);
         }
         // momentum update of every weight from this group's deltas and inputs
-        int l = 0, K4 = 1, c = 0, j0 = 0, R = 1;
+        int l = 0, K4 = 1, c = 0, j0 = 0, R = 1, last = 0;
         unsigned n_bad = 0;
         float4 a[PG];
 #pragma unroll
@@ -1337,6 +1337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 R = kThreads / K4;
                 c = tid % K4;
                 j0 = tid / K4;
+                last = v.n[l - 1] - 4 * c;   // the bias is component `last` of this column, or lies further on
 #pragma unroll
                 for (int p = 0; p < PG; ++p) a[p] = ld4(ps + q.sa[l - 1] + p * v.apitch[l - 1] + 4 * c);
             }
@@ -1356,7 +1357,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (GUARD) {
                     // columns past the bias are no weights: their inputs are 0, but 0 times a NaN
                     // or an infinite delta is NaN, which is nothing for the guard to count
-                    const int last = v.n[l - 1] - 4 * c;
                     g.x = guard_count(guard, g.x, n_bad);
                     g.y = last >= 1 ? guard_count(guard, g.y, n_bad) : 0.f;
                     g.z = last >= 2 ? guard_count(guard, g.z, n_bad) : 0.f;

@@ -107,6 +107,10 @@ __global__ void __launch_bounds__(kCThreads, 1)
     const int latched = __ldcg(v.flags);   // nothing in this launch latches a timeout before the cluster's barrier
     sigmoid_table_init(v);
 
+    unsigned pads = 0;   // this lane's columns past the bias
+    if (GUARD)
+        for (int i = 0; i < KC4; ++i) pads += (unsigned)min(max(4 * (s + S * i) + 3 - n0, 0), 4);
+
     // weights: W_1 rows to registers, W_2 columns and b_2 to shared memory
     const long long row1 = v.woff[1] + (long long)(u0 + ul) * v.kp[1];
     f32x2 w[2 * KC4], vel[2 * KC4];   // pairs of columns
@@ -315,15 +319,18 @@ __global__ void __launch_bounds__(kCThreads, 1)
                     }
                 }
                 if (GUARD) {
-                    // Columns past the bias are no weights: their inputs are 0, but 0 times a NaN
-                    // or an infinite delta is NaN, which is nothing for the guard to count.
 #pragma unroll
                     for (int j = 0; j < 2 * KC4; ++j) {
-                        const int col = 4 * (s + S * (j >> 1)) + 2 * (j & 1);
                         const float2 t = unpack2(g[j]);
-                        g[j] = pack2(col <= n0 ? guard_count(guard, t.x, n_bad) : 0.f,
-                                     col + 1 <= n0 ? guard_count(guard, t.y, n_bad) : 0.f);
+                        g[j] = pack2(guard_count(guard, t.x, n_bad), guard_count(guard, t.y, n_bad));
                     }
+                    // Columns past the bias are no weights: their inputs are 0, but 0 times a NaN
+                    // or an infinite delta is NaN, zeroed and counted above; not to be counted.
+                    // (masking each column instead cost 10-20%)
+                    float z = 0.f;
+#pragma unroll
+                    for (int p = 0; p < PG; ++p) z = fmaf(0.f, d1[p], z);
+                    if (z != 0.f) n_bad -= pads;
                 }
                 const f32x2 lr2 = pack2(lr, lr), mom2 = pack2(mom, mom);
 #pragma unroll

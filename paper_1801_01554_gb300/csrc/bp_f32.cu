@@ -428,32 +428,34 @@ __device__ __forceinline__ void forward_any(const float* W, int kp, int n_out, c
 
 // Hidden deltas of layer l for PG patterns: d_l[p][i] = (sum_j W_{l+1}[j][i]
 // d_{l+1}[p][j]) a_l[p][i] (1 - a_l[p][i]), summed over the next layer's units in
-// order.  One thread per unit sums all PG patterns, so that a weight and one read of
-// the PG deltas feed PG multiply-adds (a thread per pattern and unit reads both for
-// each one: 11.7 us per update at groups of 512 of 203-120-26 and 25.1 at 2,000,
-// against 11.6 and 24.0); where that leaves most threads without work, up to kPairs
-// patterns times units, one thread each (the same sums).  us per update, one per unit / one
-// each: 8-4-900 by 5,000 181 / 158, 100-10-500 by 2,000 51.1 / 45.9, 500-30-30-500 by 1,000
-// (240) 33.6 / 32.0; past the line 100-62-100 by 2,000 (496) 26.3 / 27.5.  dnt holds
-// d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl, pitch dpl) and, if dlt is not
-// null, pattern-minor (dlt).
-constexpr int kPairs = 256;   // half of the threads
+// order.  dnt holds d_{l+1} pattern-minor ([nn][PG]).  Writes d_l as rows (dl, pitch
+// dpl) and, if dlt is not null, pattern-minor (dlt).  Two forms with the same sums: a
+// thread per pattern and unit, or a thread per unit for all PG patterns, for which a
+// weight and one read of the PG deltas feed PG multiply-adds but which leaves most
+// threads without work where units are few.  us per update, per pair / per unit:
+//   203-120-26 by 512 (PG 4) 11.7 / 11.6, by 2,000 (8) 25.1 / 24.0; 203-300-26 by 304 (2)
+//   23.4 / 22.6; 8-4-900 by 5,000 (8) 158 / 181, by 300 (2) 22.1 / 24.7; 100-10-500 by
+//   2,000 (8) 45.9 / 51.1; 500-30-30-500 by 1,000 (8: 240 pairs) 32.0 / 33.6; 100-62-100 by
+//   2,000 (8: 496 pairs) 27.5 / 26.3; 17-9-12-5-2 by 2 (one-CTA kernel) 6.6 / 6.2.
+// So pairs up to kPairs at 8 patterns.  Both forms in one kernel cost 1-4% at 2 and 4
+// patterns, which keep one: pairs at 2, units at 4 and in the one-CTA kernel (PAIRS false).
 template <int PG>
-__device__ void hidden_delta(const float* Wn, int kpn, int n, int nn, const float* dnt,
-                             const float* al, int apl, float* dl, int dpl, float* dlt) {
-    if (PG > 1 && n * PG <= kPairs) {
-        for (int e = threadIdx.x; e < PG * n; e += kThreads) {
-            const int p = e / n, i = e - p * n;
-            float acc = 0.f;
+__device__ __forceinline__ void hidden_delta_pairs(const float* Wn, int kpn, int n, int nn, const float* dnt,
+                                                   const float* al, int apl, float* dl, int dpl, float* dlt) {
+    for (int e = threadIdx.x; e < PG * n; e += kThreads) {
+        const int p = e / n, i = e - p * n;
+        float acc = 0.f;
 #pragma unroll 4
-            for (int j = 0; j < nn; ++j) acc = fmaf(dnt[j * PG + p], Wn[(size_t)j * kpn + i], acc);
-            const float a = al[p * apl + i];
-            const float d = acc * a * (1.f - a);
-            dl[p * dpl + i] = d;
-            if (dlt != nullptr) dlt[i * PG + p] = d;
-        }
-        return;
+        for (int j = 0; j < nn; ++j) acc = fmaf(dnt[j * PG + p], Wn[(size_t)j * kpn + i], acc);
+        const float a = al[p * apl + i];
+        const float d = acc * a * (1.f - a);
+        dl[p * dpl + i] = d;
+        if (dlt != nullptr) dlt[i * PG + p] = d;
     }
+}
+template <int PG>
+__device__ __forceinline__ void hidden_delta_units(const float* Wn, int kpn, int n, int nn, const float* dnt,
+                                                   const float* al, int apl, float* dl, int dpl, float* dlt) {
     for (int i = threadIdx.x; i < n; i += kThreads) {
         float acc[PG];
 #pragma unroll
@@ -482,6 +484,20 @@ __device__ void hidden_delta(const float* Wn, int kpn, int n, int nn, const floa
             dl[p * dpl + i] = d;
             if (dlt != nullptr) dlt[i * PG + p] = d;
         }
+    }
+}
+
+constexpr int kPairs = 256;   // half of the threads
+template <int PG, bool PAIRS>
+__device__ void hidden_delta(const float* Wn, int kpn, int n, int nn, const float* dnt,
+                             const float* al, int apl, float* dl, int dpl, float* dlt) {
+    if constexpr (PAIRS && PG == 2) {
+        hidden_delta_pairs<PG>(Wn, kpn, n, nn, dnt, al, apl, dl, dpl, dlt);
+    } else if constexpr (PAIRS && PG == 8) {
+        if (n * PG <= kPairs) hidden_delta_pairs<PG>(Wn, kpn, n, nn, dnt, al, apl, dl, dpl, dlt);
+        else hidden_delta_units<PG>(Wn, kpn, n, nn, dnt, al, apl, dl, dpl, dlt);
+    } else {
+        hidden_delta_units<PG>(Wn, kpn, n, nn, dnt, al, apl, dl, dpl, dlt);
     }
 }
 
@@ -595,7 +611,7 @@ struct PhaseResult {
     float sse;
     bool ok;
 };
-template <int PG>
+template <int PG, bool PAIRS = true>
 __device__ PhaseResult pattern_phase(const F32View& v, const PatLayout& q, const float* Wb,
                                      const float* __restrict__ X, const float* __restrict__ T, int B,
                                      bool do_fwd, bool do_bwd, float* __restrict__ Y, float* smem,
@@ -682,7 +698,7 @@ __device__ PhaseResult pattern_phase(const F32View& v, const PatLayout& q, const
                                               smem + q.sdt[l + 1], smem + q.sa[l], v.apitch[l], smem + q.sd[l],
                                               v.dpitch[l], l >= 2 ? smem + q.sdt[l] : nullptr);
                 else
-                    hidden_delta<PG>(Wb + v.woff[l + 1], v.kp[l + 1], v.n[l], v.n[l + 1], smem + q.sdt[l + 1],
+                    hidden_delta<PG, PAIRS>(Wb + v.woff[l + 1], v.kp[l + 1], v.n[l], v.n[l + 1], smem + q.sdt[l + 1],
                                      smem + q.sa[l], v.apitch[l], smem + q.sd[l], v.dpitch[l],
                                      l >= 2 ? smem + q.sdt[l] : nullptr);
                 __syncthreads();
@@ -1313,7 +1329,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const long long p0 = (long long)s * minibatch;
         const int B = (int)min((long long)minibatch, (long long)n_patterns - p0);
         float* ps = pat[s & 1];
-        const float e = pattern_phase<PG>(v, q, smem, X + p0 * n0, T + p0 * nL, B, true, true, nullptr,
+        const float e = pattern_phase<PG, false>(v, q, smem, X + p0 * n0, T + p0 * nL, B, true, true, nullptr,
                                           ps, WeightCopy{nullptr, 0u, 0}, false, true).sse;
         if (tid == 0) {
             if (sse_out != nullptr) sse_out[s] = e;
@@ -1325,8 +1341,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                           (int)min((long long)minibatch, (long long)n_patterns - pn), pat[(s + 1) & 1]);
         }
         // momentum update of every weight from this group's deltas and inputs
-        int l = 0, K4 = 1, c = 0, j0 = 0, R = 1, last = 0;
-        unsigned n_bad = 0;
+        int l = 0, K4 = 1, c = 0, j0 = 0, R = 1;
+        unsigned n_bad = 0, pads = 0;
         float4 a[PG];
 #pragma unroll
         for (int m = 0; m < NV4; ++m) {
@@ -1337,7 +1353,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 R = kThreads / K4;
                 c = tid % K4;
                 j0 = tid / K4;
-                last = v.n[l - 1] - 4 * c;   // the bias is component `last` of this column, or lies further on
+                pads = (unsigned)max(4 * c + 3 - v.n[l - 1], 0);   // of this float4: the bias is column n
 #pragma unroll
                 for (int p = 0; p < PG; ++p) a[p] = ld4(ps + q.sa[l - 1] + p * v.apitch[l - 1] + 4 * c);
             }
@@ -1356,11 +1372,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float4 w = *wp;
                 if (GUARD) {
                     // columns past the bias are no weights: their inputs are 0, but 0 times a NaN
-                    // or an infinite delta is NaN, which is nothing for the guard to count
+                    // or an infinite delta is NaN, zeroed and counted below; not to be counted
+                    if (g.w != g.w) n_bad -= pads;
                     g.x = guard_count(guard, g.x, n_bad);
-                    g.y = last >= 1 ? guard_count(guard, g.y, n_bad) : 0.f;
-                    g.z = last >= 2 ? guard_count(guard, g.z, n_bad) : 0.f;
-                    g.w = last >= 3 ? guard_count(guard, g.w, n_bad) : 0.f;
+                    g.y = guard_count(guard, g.y, n_bad);
+                    g.z = guard_count(guard, g.z, n_bad);
+                    g.w = guard_count(guard, g.w, n_bad);
                 }
                 float4& u = vel[m];
                 u.x = a_lr * g.x + mom * u.x;

@@ -710,9 +710,9 @@ def test_nettalk120_workload_full():
 
 
 @pytest.mark.parametrize("sizes,n,mb", [((20, 8, 60), 1216, 1216), ((100, 32, 40), 1100, 1100),
-                                        ((100, 33, 40), 1100, 1100), ((9, 1, 70), 700, 304), ((16, 64, 20), 600, 304)])
+                                        ((100, 33, 40), 1100, 1100), ((9, 1, 70), 700, 304), ((16, 64, 20), 600, 600)])
 def test_hidden_deltas_of_few_and_many_units_step_by_step(sizes, n, mb):
-    """Both sides of the line between a thread per pattern and unit and a thread per unit (256
-    pairs: 32 units at 8 patterns a pass, 64 at 4), and a single hidden unit."""
+    """Both forms of the hidden deltas: at 8 patterns a pass (1,216, 1,100) both sides of the
+    line of 256 pairs of pattern and unit, at 2 and 4 (304, 600), and a single hidden unit."""
     X, T, theta = problem(sizes, n, seed=92)
     stepwise(sizes, X, T, theta, np.zeros_like(theta), mb, 0.002, 0.9)

@@ -260,12 +260,12 @@ def synth_sizes(name):
 
 
 # DRAM bytes (read + write) per pattern of each workload's roofline unit, from
-# single-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum; the
-# commands are in profiles/dram_traffic_all_workloads.md): one training launch
-# for the float32 nets (one epoch; 203-120-26 captured on a 16,384-pattern epoch
-# and scaled by patterns, as its traffic is the inputs read once), the whole
-# training step (all launches) for the bf16 nets.  Re-measure after any change
-# to these kernels.
+# single-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum; see
+# profiles/dram_traffic_all_workloads.md): one training launch for the float32
+# nets (one epoch; 203-120-26 captured on a 16,384-pattern epoch and scaled by
+# patterns, as its traffic is the inputs read once), the sum over a training
+# step's launches for the bf16 nets.  After a change to a kernel capture that
+# kernel again, one or two launches of it, and replace its share.
 TRAFFIC_PER_PATTERN = {
     "nettalk60": 1_116_928 / 1024,          # 1.12 MB per launch (one update of 1,024)
     "nettalk120": 15_412_224 / 16384,       # 61.6 MB per 65,536-pattern launch

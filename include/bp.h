@@ -254,7 +254,9 @@ bp_status bp_check(bp_net* net, void* stream);
  *   calls on a device share the array and find the previous call's contents:
  *   the call clears what must start at zero, and calls that overlap on the GPU
  *   (different streams, or several host threads) race on it.
- *   Groups run on the kernels that bp_train_epoch picks for their size.
+ *   Groups run on the kernels that bp_train_epoch picks for their size, but for
+ *   large groups of one-hidden-layer nets, which take the grid-wide kernel here
+ *   (the call keeps no per-CTA sums): the same updates, added up in another order.
  *   Asynchronous with respect to the host like bp_train_epoch.  Pointers are
  *   checked before any CUDA call: d_theta, d_V, d_X, d_T, d_sse and d_status
  *   must be 4-byte aligned.  Errors: BP_EINVAL, BP_ESHAPE, BP_ECUDA. */

@@ -1486,7 +1486,8 @@ int sum_chain(int M, int N, int kb_total, int num_sms) {
 // patterns 21.9 / 20.6 / 24.4 / 29.7; 1024-2048-2048-512 at 1,001 90.6 / 82.2 / 84.5 /
 // 93.5, at 8,192 294.0 / 313.4 / 281.4 / 296.4; 2048-2048-2048 at 2,048 117.7 / 109.9 /
 // 114.3 / 116.4; 128-256-256-64 at 8,192, whose 16 tiles leave the chip idle unsplit,
-// 39.9 / 48.5 / 57.1 / 75.2.
+// 39.9 / 48.5 / 57.1 / 75.2.  (All with one chain per run of K blocks; in chains, see
+// sum_chain, the 20.6 of 208-1024-32 are 21.0, the others change by less than 1%.)
 constexpr int kMaxSplits = 16;
 struct DwPlan {
     int bn, tiles, splits, kb_total, kb_per_split;

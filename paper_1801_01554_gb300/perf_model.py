@@ -11,8 +11,8 @@ Two models live here:
   GB300: microseconds per update from the phases of the persistent kernel
   (two grid barriers, the weight copy into shared memory, pattern passes of PG
   patterns per CTA, 512-pattern chunks of the weight phase), of the kernel for
-  large groups of one-hidden-layer nets (a fixed cost, then one cost per pass of
-  64 patterns a CTA), and of the kernels for groups of 1-4 patterns.  Its
+  large groups of one-hidden-layer nets (a fixed cost, one per pass of 64 patterns
+  a CTA and one per pattern), and of the kernels for groups of 1-4 patterns.  Its
   constants are fitted to per-update times measured on GB300.
 
 Readings of the printed model (Section 6.1):
@@ -98,16 +98,18 @@ class GB300Phases:
     balanced_chunk_us: float = 2.12
     balanced_min_chunks: int = 24
     chunk_rows: int = 512
-    # large groups of one-hidden-layer nets (changes summed in registers), from
-    # this many patterns per CTA on: barriers, the reduction over the CTAs and the
-    # weight copy, then one cost per pass of 64 patterns
+    # large groups of one-hidden-layer nets (changes summed on chip), from this many
+    # patterns per CTA on: barriers, the reduction over the CTAs and the weight copy,
+    # then one cost per pass of 64 rows (layers and deltas run over all of them) and
+    # one per pattern (the changes)
     large_min_per_cta: int = 40
-    large_fixed_us: float = 12.0
+    large_fixed_us: float = 13.4
     large_pass: int = 64
-    large_pass_us: float = 32.9
+    large_pass_us: float = 20.7
+    large_pattern_us: float = 0.201
     # groups of up to 4 patterns: one CTA (any depth), one cluster (one hidden layer)
     small_us: tuple = ((1, 6.68), (2, 7.37), (4, 9.17))
-    cluster_us: tuple = ((1, 2.0), (2, 2.2), (4, 2.7))
+    cluster_us: tuple = ((1, 1.8), (2, 2.0), (4, 2.4))
 
 
 def gb300_group_size(B, n_sm=152, max_pg=8, wide=True):
@@ -132,7 +134,8 @@ def gb300_update_us(B, tiles=121, tiles16=64, ph: GB300Phases = GB300Phases(), s
             if B <= b:
                 return us
     if B >= ph.large_min_per_cta * ph.n_sm:
-        return ph.large_fixed_us + -(-(-(-B // ph.n_sm)) // ph.large_pass) * ph.large_pass_us
+        share = -(-B // ph.n_sm)
+        return ph.large_fixed_us + -(-share // ph.large_pass) * ph.large_pass_us + share * ph.large_pattern_us
     pg = gb300_group_size(B, ph.n_sm)
     passes = -(-(-(-B // ph.n_sm)) // pg)
     t = ph.pattern_fixed_us + passes * dict(ph.pass_us)[pg]

@@ -592,14 +592,13 @@ struct GemmCfg {
     static constexpr int kABytes = BM * BK * 2;
     static constexpr int kBBytes = BN * BK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kTmemCols = 2 * BN;   // two accumulators
     // tile ring, then barriers and scratch
     static constexpr int kRingBytes = kStages * kStageBytes;
     static constexpr int kColsumBytes = 4 * BN * 4;
     static constexpr int kStageOutBytes = kEpiWarps * 32 * 32 * 2;   // one 32 x 32 bf16 block per epilogue warp
     static constexpr int kBiasBytes = 2 * BN * 4;   // the tile's biases, one block per accumulator
     static constexpr int kSmemBytes =
-        1024 + kRingBytes + kColsumBytes + kStageOutBytes + kBiasBytes + 256;
+        1024 + kRingBytes + kColsumBytes + kStageOutBytes + kBiasBytes + 512;
 };
 
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
@@ -770,10 +769,17 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                                                  Cfg::kStageOutBytes + Cfg::kBiasBytes);
     uint64_t* full = bars;              // [S]
     uint64_t* empty = bars + S;         // [S]
-    uint64_t* tfull = bars + 2 * S;     // [2]
-    uint64_t* tempty = bars + 2 * S + 2;   // [2]
-    uint64_t* drain = bars + 2 * S + 4;    // [1] used only when a wait ran out
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
+    // Accumulators: two, so that the epilogue of a tile overlaps the next one's MMAs; as many as
+    // fit in the pooled changes, whose chains are short where tiles are narrow (208-128-32 by
+    // 512, eight chains of one K block: 19.2 us per update with two, 17.7 with eight).
+    constexpr bool kDw = MODE == MODE_DW || MODE == MODE_DWU;
+    constexpr int kAcc = kDw ? 512 / BN : 2;
+    constexpr int kTmemCols = kAcc * BN;
+    static_assert((2 * S + 2 * kAcc + 2) * sizeof(uint64_t) <= 512, "room for the barriers");
+    uint64_t* tfull = bars + 2 * S;            // [kAcc]
+    uint64_t* tempty = tfull + kAcc;           // [kAcc]
+    uint64_t* drain = tempty + kAcc;           // [1] used only when a wait ran out
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -788,7 +794,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < kAcc; ++a) {
             mbar_init(&tfull[a], 1);
             mbar_init(&tempty[a], kEpiThreads);
         }
@@ -799,7 +805,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tmem_slot)),
-                     "r"(Cfg::kTmemCols)
+                     "r"(kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -875,7 +881,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     }
                     if (!ok) break;
                     umma_commit(&tfull[acc]);
-                    if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                    if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
                 }
             }
             if (!ok && issued_any) {
@@ -894,7 +900,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
         const int cbeg = (ew >> 2) * (BN / 2);   // this warp's half of the columns
         int acc = 0;
         unsigned acc_phase = 0;
-        constexpr bool kDw = MODE == MODE_DW || MODE == MODE_DWU;
         if constexpr (MODE == MODE_DWU) {
             // this CTA's share of the biases and the error sum, while the first tile accumulates
             const int nb = work.u.bias_blocks + (work.u.sse_out != nullptr ? 1 : 0);
@@ -940,7 +945,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 mbar_arrive(&tempty[a]);
             };
             auto next_acc = [&] {
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
             };
             if constexpr (kDw) {
                 const DwLayer& y = g.ly[w.l];
@@ -969,6 +974,12 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                     tmem_wait_st();
                     release(1 - acc);
                 };
+                UpdBlock cur, nxt;
+                auto load = [&](int c, UpdBlock& b) {
+                    if constexpr (MODE == MODE_DWU)
+                        update_block_load(work.u, work.u.ly[w.l], y.M, y.N, m0, w.nb * BN + cbeg + c, b);
+                };
+                load(0, cur);   // arrives while the chains accumulate (after them: 17.7 us, not 17.2)
                 bool stay = true;
                 for (int c0 = w.kb0; c0 + w.chain < w.kb1; c0 += w.chain) {
                     stay = wait_acc();
@@ -992,10 +1003,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                 if constexpr (MODE == MODE_DWU) {
                     const LayerUpd& u = work.u.ly[w.l];
                     float4* sF = reinterpret_cast<float4*>(stage_out + ew * 1024);
-                    UpdBlock cur, nxt;
-                    auto load = [&](int c, UpdBlock& b) {
-                        update_block_load(work.u, u, y.M, y.N, m0, w.nb * BN + cbeg + c, b);
-                    };
                     auto apply = [&](int c, UpdBlock& b) {
                         float r[16];
                         tmem_ld16(trow + (uint32_t)(acc * BN + cbeg + c), r);
@@ -1005,7 +1012,6 @@ __device__ __forceinline__ void gemm_body(const Work work) {
                         }
                         update_block_apply(work.u, u, y.M, y.N, m0, w.nb * BN + cbeg + c, r, b, sF);
                     };
-                    load(0, cur);
                     if (!wait_acc()) break;
                     if (!kRegs && several) add_previous();
 #pragma unroll(kRegs ? BN / 64 : 1)
@@ -1082,7 +1088,7 @@ __device__ __forceinline__ void gemm_body(const Work work) {
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
-                     "r"(Cfg::kTmemCols)
+                     "r"(kTmemCols)
                      : "memory");
     }
 }
@@ -1453,7 +1459,8 @@ cudaError_t run_forward(Bf16Net* b, const bf16* X, int B, const bf16* T, bf16* Y
 //                                   in the time of a byte of DRAM traffic),
 // many for the few tiles of a small layer, one or two for a layer of several waves.  us,
 // one chain / this rule: 25 steps of 8,192 of 1024-2048-2048-512 7,248 / 7,303, 50 steps of
-// 4096^5 201,690 / 201,520, two epochs of 16,200 of 208-1024-32 by 512 1,333 / 1,357.
+// 4096^5 201,690 / 201,520, two epochs of 16,200 of 208-1024-32 by 512 1,332 / 1,333, an
+// update of 208-128-32 by 512 16.7 / 17.2.
 constexpr int kMaxChains = 16;
 int sum_chain(int M, int N, int kb_total, int num_sms) {
     const int tiles = tiles_of(M, N, 256);
@@ -1487,7 +1494,7 @@ int sum_chain(int M, int N, int kb_total, int num_sms) {
 // 93.5, at 8,192 294.0 / 313.4 / 281.4 / 296.4; 2048-2048-2048 at 2,048 117.7 / 109.9 /
 // 114.3 / 116.4; 128-256-256-64 at 8,192, whose 16 tiles leave the chip idle unsplit,
 // 39.9 / 48.5 / 57.1 / 75.2.  (All with one chain per run of K blocks; in chains, see
-// sum_chain, the 20.6 of 208-1024-32 are 21.0, the others change by less than 1%.)
+// sum_chain, they change by less than 1%.)
 constexpr int kMaxSplits = 16;
 struct DwPlan {
     int bn, tiles, splits, kb_total, kb_per_split;

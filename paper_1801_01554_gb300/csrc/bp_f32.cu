@@ -29,7 +29,7 @@
 // barrier is bounded and latches kFlagTimeout instead of hanging.  Groups of at
 // most 4 patterns of a one-hidden-layer net run on one cluster instead
 // (bp_f32_cluster.cu), its groups of 40 or more patterns per CTA with the sums of
-// changes in registers (bp_f32_large.cu), and other nets' groups of at most 4 on
+// changes on chip (bp_f32_large.cu), and other nets' groups of at most 4 on
 // one CTA (k_train_small), with the weights resident on chip for the whole launch.
 #include <cuda_runtime.h>
 
